@@ -70,14 +70,13 @@ __device__ __forceinline__ void load_d(const R *__restrict__ f, long long s, lon
     for (int a = 0; a < NC; ++a) v[a] = widen(ld_field<COHERENT>(f + i + a));
 }
 
-// Adds one site's raw sums to acc.  c: phi_n at the site, xm..zp: its neighbours in the order
-// -x, +x, -y, +y, -z, +z; p: pi_{n-1/2}.  Explicit round-to-nearest operations keep the
+// Adds one site's raw sums to acc.  c: phi_n at the site, xp, yp, zp: its neighbours +x, +y, +z;
+// nb: its neighbour sums (sum6); p: pi_{n-1/2}.  Explicit round-to-nearest operations keep the
 // stand-alone and fused kernels bitwise equal; the half kick is the FP64 kick's arithmetic.
 template <int NC>
-__device__ __forceinline__ void energy_site(const double (&c)[NC], const double (&xm)[NC], const double (&xp)[NC],
-                                            const double (&ym)[NC], const double (&yp)[NC], const double (&zm)[NC],
-                                            const double (&zp)[NC], const double (&p)[NC], double (&acc)[kNs<NC>],
-                                            const CoefE &k) {
+__device__ __forceinline__ void energy_site(const double (&c)[NC], const double (&xp)[NC], const double (&yp)[NC],
+                                            const double (&zp)[NC], const double (&nb)[NC], const double (&p)[NC],
+                                            double (&acc)[kNs<NC>], const CoefE &k) {
     double s2 = __dmul_rn(c[0], c[0]);
 #pragma unroll
     for (int b = 1; b < NC; ++b) s2 = __fma_rn(c[b], c[b], s2);
@@ -85,8 +84,7 @@ __device__ __forceinline__ void energy_site(const double (&c)[NC], const double 
     const double w = __dsub_rn(s2, k.eta2);
 #pragma unroll
     for (int a = 0; a < NC; ++a) {
-        const double nb = __dadd_rn(__dadd_rn(xm[a], xp[a]), __dadd_rn(__dadd_rn(ym[a], yp[a]), __dadd_rn(zm[a], zp[a])));
-        const double pin = __fma_rn(k.ah, nb, __fma_rn(-gh, c[a], p[a]));
+        const double pin = __fma_rn(k.ah, nb[a], __fma_rn(-gh, c[a], p[a]));
         acc[kKin] = __fma_rn(pin, pin, acc[kKin]);
         const double ex = __dsub_rn(xp[a], c[a]), ey = __dsub_rn(yp[a], c[a]), ez = __dsub_rn(zp[a], c[a]);
         acc[kGrad] = __fma_rn(ez, ez, __fma_rn(ey, ey, __fma_rn(ex, ex, acc[kGrad])));
@@ -202,7 +200,9 @@ __global__ void __launch_bounds__(kEnergyThreads) k_energy(const R *__restrict__
         load_d<R, NC>(phi, n.zm, g.sites, zm);
         load_d<R, NC>(phi, n.zp, g.sites, zp);
         load_d<R, NC>(pi, s, g.sites, p);
-        energy_site<NC>(c, xm, xp, ym, yp, zm, zp, p, acc, k);
+        double nb[NC];
+        neighbour_sums<NC>(xm, xp, ym, yp, zm, zp, nb);
+        energy_site<NC>(c, xp, yp, zp, nb, p, acc, k);
     }
     finish_energy<NC>(acc, sh, scratch, k, record);
 }
@@ -225,8 +225,10 @@ __device__ __forceinline__ void site_step_energy_f64(const double *__restrict__ 
     const long long o = checked(s * NC, NC, g.sites * NC);
 #pragma unroll
     for (int a = 0; a < NC; ++a) p[a] = pi[o + a];
-    energy_site<NC>(c, xm, xp, ym, yp, zm, zp, p, acc, ke);
-    update_f64<NC>(c, xm, xp, ym, yp, zm, zp, p, out, k);
+    double nb[NC];
+    neighbour_sums<NC>(xm, xp, ym, yp, zm, zp, nb);
+    energy_site<NC>(c, xp, yp, zp, nb, p, acc, ke);
+    update_f64_nb<NC>(c, nb, p, out, k);
 #pragma unroll
     for (int a = 0; a < NC; ++a) {
         pi[o + a] = p[a];
@@ -271,7 +273,9 @@ __device__ __forceinline__ void site_step_energy_f32(const float *__restrict__ p
         dzp[a] = widen(zp[a]);
         dp[a] = widen(p[a]);
     }
-    energy_site<NC>(dc, dxm, dxp, dym, dyp, dzm, dzp, dp, acc, ke);
+    double nb[NC];
+    neighbour_sums<NC>(dxm, dxp, dym, dyp, dzm, dzp, nb);
+    energy_site<NC>(dc, dxp, dyp, dzp, nb, dp, acc, ke);
     update_f32<NC, KAHAN>(c, xm, xp, ym, yp, zm, zp, p, cm, out, k);
 #pragma unroll
     for (int a = 0; a < NC; ++a) {

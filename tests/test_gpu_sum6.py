@@ -1,0 +1,91 @@
+"""GPU: the FP64 neighbour sum, done on the integer pipes, at the edges of its range.
+
+With lambda = m2 = 0, dt = dx = 1 and pi = 0 one FP64 step gives pi' = nb - 6 phi and
+phi' = phi + pi', so the neighbour sum nb shows in the result.  The reference is the exact
+rational sum.  Derivation of the tolerance, with u = 2^-53 and M the largest neighbour: the sum is
+off by at most u |nb| + 6 units of 2^-59 M (bits below its fixed-point grid) or, outside the grid's
+exponent range, by the five FP64 additions' 3 u sum|phi_i|; -6 phi is rounded once and its fma with
+nb once, each at most u (6 |phi| + |nb|): in all below 6 u (sum|phi_i| + 6 |phi|) + 2^-56 M, plus
+the smallest subnormal for each rounding.  (The range's high end, 2^1017, cannot be seen in a step:
+phi^2 overflows above 2^512 and the step gives NaN whatever the sum.)"""
+from fractions import Fraction
+
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+SHAPE = (6, 4, 5)  # nx, ny, nz
+
+
+@pytest.fixture(scope="module")
+def lf2():
+    import torch
+    if not torch.cuda.is_available():
+        pytest.skip("needs a GPU")
+    from paper_1508_05610_gb300 import build, lf2 as binding
+    build.build()
+    binding.load()
+    return binding
+
+
+def values(kind, rng):
+    n = SHAPE[::-1] + (1,)
+    v = rng.standard_normal(n)
+    if kind == "spread":  # exponents up to 140 apart: small operands drop below the grid
+        return np.ldexp(v, rng.integers(-70, 70, n))
+    if kind == "equal":  # all significands full, sums of up to six equal values
+        return np.where(rng.random(n) < 0.5, 1.0, -1.0) * (2.0 - 2.0 ** -52)
+    if kind == "cancel":  # sums that vanish or keep only the last bits
+        return np.where(np.indices(n).sum(0) % 2 == 0, 1.0, -1.0) * (1.0 + 2.0 ** -52 * rng.integers(0, 3, n))
+    if kind == "zeros":
+        return np.where(rng.random(n) < 0.6, 0.0, v) * np.where(rng.random(n) < 0.5, 1.0, -1.0)
+    assert kind == "low"  # around the low end of the grid's range (2^-959), and subnormal
+    return np.ldexp(v, rng.integers(-1073, -950, n))
+
+
+@pytest.mark.parametrize("kernel", ["site", "stream", "tblock"])
+@pytest.mark.parametrize("kind", ["spread", "equal", "cancel", "zeros", "low"])
+def test_neighbour_sum_against_exact_rationals(lf2, kind, kernel):
+    phi = values(kind, np.random.default_rng(5))
+    p = lf2.params(dx=1.0, dt=1.0, lam=0.0, eta=0.0, m2=0.0)
+    steps = 2 if kernel == "tblock" else 1
+    with lf2.System(SHAPE, 1, "f64") as s, lf2.System(SHAPE, 1, "f64") as t:
+        for q in (s, t):
+            q.upload(phi, np.zeros_like(phi))
+        if kernel == "tblock":
+            lf2.lf2_leapfrog_ex(s.phi, s.pi, p, steps, kernel=lf2.LF2_KERNEL_TBLOCK, depth=2, cx=1, tile_x=4, tile_y=4)
+        else:
+            lf2.lf2_leapfrog_ex(s.phi, s.pi, p, steps, kernel={"site": 1, "stream": 2}[kernel])
+        lf2.lf2_leapfrog_ex(t.phi, t.pi, p, steps, kernel=lf2.LF2_KERNEL_SITE)
+        got, ref = s.download(), t.download()
+    assert np.array_equal(got[0], ref[0], equal_nan=True) and np.array_equal(got[1], ref[1], equal_nan=True)
+    if steps > 1:
+        return
+    f = phi[..., 0]
+    nbrs = [np.roll(f, sh, ax) for ax in range(3) for sh in (1, -1)]
+    u, sub = Fraction(1, 2 ** 53), Fraction(1, 2 ** 1074)
+    for at in np.ndindex(f.shape):
+        c, nb = Fraction(f[at]), [Fraction(n[at]) for n in nbrs]
+        scale, top = sum(map(abs, nb)) + 6 * abs(c), max(map(abs, nb))
+        err = abs(Fraction(got[1][at][0]) - (sum(nb) - 6 * c))
+        assert err <= 6 * u * scale + top / 2 ** 56 + 8 * sub, (at, float(err), float(scale))
+
+
+def test_infinities_and_nan_reach_the_result(lf2):
+    """As IEEE additions give them: an infinite neighbour makes pi' infinite, opposite infinities
+    and NaN make it NaN (as does an infinite site itself: lambda phi^2 is 0 times infinity), the
+    other sites stay finite."""
+    phi = np.random.default_rng(6).standard_normal(SHAPE[::-1] + (1,))
+    phi[0, 0, 0], phi[0, 0, 2], phi[3, 2, 4] = np.inf, -np.inf, np.nan
+    f = phi[..., 0]
+    with np.errstate(invalid="ignore"):
+        want = sum(np.roll(f, sh, ax) for ax in range(3) for sh in (1, -1)) - (0.0 * f * f + 6) * f
+    p = lf2.params(dx=1.0, dt=1.0, lam=0.0, eta=0.0, m2=0.0)
+    with lf2.System(SHAPE, 1, "f64") as s:
+        s.upload(phi, np.zeros_like(phi))
+        lf2.lf2_leapfrog(s.phi, s.pi, p, 1)
+        got = s.download()[1][..., 0]
+    assert np.array_equal(np.isnan(got), np.isnan(want)) and np.array_equal(np.isinf(got), np.isinf(want))
+    assert np.array_equal(got[np.isinf(got)], want[np.isinf(want)])
+    fine = np.isfinite(want)
+    assert np.allclose(got[fine], want[fine], rtol=1e-14, atol=1e-13)
