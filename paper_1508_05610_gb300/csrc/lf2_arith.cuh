@@ -382,6 +382,53 @@ struct Geom {
     long long sites;
 };
 
+// The coordinates of the sites s, s + stride, s + 2 stride, ... that a thread of a grid-stride loop
+// visits.  The stride is split into (x, y, z) once on the host, so a step is three additions with
+// carries; two 64-bit divisions per site (about 150 instructions) took most of the issue slots of
+// the per-site kernels (a step of k_site on 257 x 193 x 161 real FP32+Kahan: 53.3 -> 45.5 us; of the
+// multi-step step + energy on 32^3 real FP64: 5.59 -> 5.36 us).
+struct Stride3 {
+    int x, y, z;
+    long long sites;
+};
+
+inline Stride3 make_stride3(long long stride, const Geom &g) {
+    const long long r = stride / g.nx;
+    return Stride3{(int)(stride % g.nx), (int)(r % g.ny), (int)(r / g.ny), stride};
+}
+
+struct SiteWalk {
+    int x, y, z;
+    long long s;
+    __device__ __forceinline__ SiteWalk(long long first, const Geom &g) : s(first) {
+        if (first < (1LL << 31)) {
+            const unsigned f = (unsigned)first, r = f / (unsigned)g.nx;
+            x = (int)(f - r * (unsigned)g.nx);
+            z = (int)(r / (unsigned)g.ny);
+            y = (int)(r - (unsigned)z * (unsigned)g.ny);
+        } else {
+            const long long r = first / g.nx;
+            x = (int)(first - r * g.nx);
+            z = (int)(r / g.ny);
+            y = (int)(r - (long long)z * g.ny);
+        }
+    }
+    __device__ __forceinline__ void advance(const Stride3 &d, const Geom &g) {
+        s += d.sites;
+        x += d.x;
+        y += d.y;
+        z += d.z;
+        if (x >= g.nx) {
+            x -= g.nx;
+            ++y;
+        }
+        if (y >= g.ny) {
+            y -= g.ny;
+            ++z;
+        }
+    }
+};
+
 __device__ __forceinline__ int wrap_dn(int i, int n) { return i == 0 ? n - 1 : i - 1; }
 __device__ __forceinline__ int wrap_up(int i, int n) { return i == n - 1 ? 0 : i + 1; }
 

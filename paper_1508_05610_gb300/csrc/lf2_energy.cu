@@ -171,26 +171,24 @@ struct Nbr {
     long long xm, xp, ym, yp, zm, zp;
 };
 
-__device__ __forceinline__ Nbr neighbours(long long s, const Geom &g) {
-    const int x = (int)(s % g.nx);
-    const long long r = s / g.nx;
-    const int y = (int)(r % g.ny);
-    const int z = (int)(r / g.ny);
+__device__ __forceinline__ Nbr neighbours(const SiteWalk &w, const Geom &g) {
     const long long row = g.nx, plane = (long long)g.nx * g.ny;
-    return Nbr{s - x + wrap_dn(x, g.nx),       s - x + wrap_up(x, g.nx),       s + (wrap_dn(y, g.ny) - y) * row,
-               s + (wrap_up(y, g.ny) - y) * row, s + (wrap_dn(z, g.nz) - z) * plane, s + (wrap_up(z, g.nz) - z) * plane};
+    return Nbr{w.s + (w.x == 0 ? g.nx - 1 : -1),          w.s + (w.x == g.nx - 1 ? 1 - g.nx : 1),
+               w.s + (wrap_dn(w.y, g.ny) - w.y) * row,    w.s + (wrap_up(w.y, g.ny) - w.y) * row,
+               w.s + (wrap_dn(w.z, g.nz) - w.z) * plane,  w.s + (wrap_up(w.z, g.nz) - w.z) * plane};
 }
 
 template <typename R, int NC>
 __global__ void __launch_bounds__(kEnergyThreads) k_energy(const R *__restrict__ phi, const R *__restrict__ pi, Geom g,
-                                                           CoefE k, double *__restrict__ scratch, double *__restrict__ record) {
+                                                           Stride3 d, CoefE k, double *__restrict__ scratch,
+                                                           double *__restrict__ record) {
     __shared__ double sh[kNs<NC>][kEnergyThreads];
     double acc[kNs<NC>];
 #pragma unroll
     for (int j = 0; j < kNs<NC>; ++j) acc[j] = 0.0;
-    const long long stride = (long long)gridDim.x * blockDim.x;
-    for (long long s = (long long)blockIdx.x * blockDim.x + threadIdx.x; s < g.sites; s += stride) {
-        const Nbr n = neighbours(s, g);
+    for (SiteWalk w((long long)blockIdx.x * blockDim.x + threadIdx.x, g); w.s < g.sites; w.advance(d, g)) {
+        const Nbr n = neighbours(w, g);
+        const long long s = w.s;
         double c[NC], xm[NC], xp[NC], ym[NC], yp[NC], zm[NC], zp[NC], p[NC];
         load_d<R, NC>(phi, s, g.sites, c);
         load_d<R, NC>(phi, n.xm, g.sites, xm);
@@ -211,9 +209,10 @@ __global__ void __launch_bounds__(kEnergyThreads) k_energy(const R *__restrict__
 // to acc and writes the step to (phi_{n+1}, pi_{n+1/2}), from one read of the site's stencil.
 template <int NC, bool COHERENT>
 __device__ __forceinline__ void site_step_energy_f64(const double *__restrict__ phi, double *__restrict__ phi_out,
-                                                     double *__restrict__ pi, long long s, const Geom &g,
+                                                     double *__restrict__ pi, const SiteWalk &w, const Geom &g,
                                                      const Coef64 &k, const CoefE &ke, double (&acc)[kNs<NC>]) {
-    const Nbr n = neighbours(s, g);
+    const Nbr n = neighbours(w, g);
+    const long long s = w.s;
     double c[NC], xm[NC], xp[NC], ym[NC], yp[NC], zm[NC], zp[NC], p[NC], out[NC];
     load_d<double, NC, COHERENT>(phi, s, g.sites, c);
     load_d<double, NC, COHERENT>(phi, n.xm, g.sites, xm);
@@ -240,10 +239,11 @@ __device__ __forceinline__ void site_step_energy_f64(const double *__restrict__ 
 // the exact conversions of the stored values.
 template <int NC, bool KAHAN, bool COHERENT>
 __device__ __forceinline__ void site_step_energy_f32(const float *__restrict__ phi, float *__restrict__ phi_out,
-                                                     float *__restrict__ pi, float *__restrict__ comp, long long s,
+                                                     float *__restrict__ pi, float *__restrict__ comp, const SiteWalk &w,
                                                      const Geom &g, const Coef32 &k, const CoefE &ke,
                                                      double (&acc)[kNs<NC>]) {
-    const Nbr n = neighbours(s, g);
+    const Nbr n = neighbours(w, g);
+    const long long s = w.s;
     const long long cnt = g.sites * NC;
     const long long o = checked(s * NC, NC, cnt), ixm = checked(n.xm * NC, NC, cnt), ixp = checked(n.xp * NC, NC, cnt),
                     iym = checked(n.ym * NC, NC, cnt), iyp = checked(n.yp * NC, NC, cnt),
@@ -289,29 +289,27 @@ __device__ __forceinline__ void site_step_energy_f32(const float *__restrict__ p
 template <int NC>
 __global__ void __launch_bounds__(kEnergyThreads)
     k_step_energy_f64(const double *__restrict__ phi, double *__restrict__ phi_out, double *__restrict__ pi, Geom g,
-                      Coef64 k, CoefE ke, double *__restrict__ scratch, double *__restrict__ record) {
+                      Stride3 d, Coef64 k, CoefE ke, double *__restrict__ scratch, double *__restrict__ record) {
     __shared__ double sh[kNs<NC>][kEnergyThreads];
     double acc[kNs<NC>];
 #pragma unroll
     for (int j = 0; j < kNs<NC>; ++j) acc[j] = 0.0;
-    const long long stride = (long long)gridDim.x * blockDim.x;
-    for (long long s = (long long)blockIdx.x * blockDim.x + threadIdx.x; s < g.sites; s += stride)
-        site_step_energy_f64<NC, false>(phi, phi_out, pi, s, g, k, ke, acc);
+    for (SiteWalk w((long long)blockIdx.x * blockDim.x + threadIdx.x, g); w.s < g.sites; w.advance(d, g))
+        site_step_energy_f64<NC, false>(phi, phi_out, pi, w, g, k, ke, acc);
     finish_energy<NC>(acc, sh, scratch, ke, record);
 }
 
 template <int NC, bool KAHAN>
 __global__ void __launch_bounds__(kEnergyThreads)
     k_step_energy_f32(const float *__restrict__ phi, float *__restrict__ phi_out, float *__restrict__ pi,
-                      float *__restrict__ comp, Geom g, Coef32 k, CoefE ke, double *__restrict__ scratch,
-                      double *__restrict__ record) {
+                      float *__restrict__ comp, Geom g, Stride3 d, Coef32 k, CoefE ke,
+                      double *__restrict__ scratch, double *__restrict__ record) {
     __shared__ double sh[kNs<NC>][kEnergyThreads];
     double acc[kNs<NC>];
 #pragma unroll
     for (int j = 0; j < kNs<NC>; ++j) acc[j] = 0.0;
-    const long long stride = (long long)gridDim.x * blockDim.x;
-    for (long long s = (long long)blockIdx.x * blockDim.x + threadIdx.x; s < g.sites; s += stride)
-        site_step_energy_f32<NC, KAHAN, false>(phi, phi_out, pi, comp, s, g, k, ke, acc);
+    for (SiteWalk w((long long)blockIdx.x * blockDim.x + threadIdx.x, g); w.s < g.sites; w.advance(d, g))
+        site_step_energy_f32<NC, KAHAN, false>(phi, phi_out, pi, comp, w, g, k, ke, acc);
     finish_energy<NC>(acc, sh, scratch, ke, record);
 }
 
@@ -395,17 +393,17 @@ __device__ __forceinline__ void poison_records(double *records, int from, int ns
         for (int i = 0; i < kEnergySlots; ++i) records[(size_t)j * kEnergySlots + i] = __longlong_as_double(0x7ff8000000000000LL);
 }
 
-// The step loop shared by the FP64 and FP32 kernels.  site(src, dst, s, acc) performs the
-// fused step + energy of site s.
+// The step loop shared by the FP64 and FP32 kernels.  site(src, dst, w, acc) performs the
+// fused step + energy of the site that w stands on; d is the site blocks' grid stride.
 template <int NC, typename R, typename Site>
-__device__ __forceinline__ void steps_energy_loop(R *phi_a, R *phi_b, Geom g, const CoefE &ke, int nsteps,
+__device__ __forceinline__ void steps_energy_loop(R *phi_a, R *phi_b, Geom g, const Stride3 &d, const CoefE &ke, int nsteps,
                                                   double *__restrict__ scratch, double *__restrict__ records,
                                                   unsigned polls, double (&sh)[kNs<NC>][kEnergyThreads], Site site) {
     constexpr int NS = kNs<NC>;
     unsigned *bar = reinterpret_cast<unsigned *>(scratch + kBarrierOffset);
     const int nsb = (int)gridDim.x - 1;  // site blocks; the last block reduces
     const bool reducer = (int)blockIdx.x == nsb;
-    const long long stride = (long long)nsb * blockDim.x;
+    const SiteWalk first((long long)blockIdx.x * blockDim.x + threadIdx.x, g);
     // rows [first, first + count) of the set of `step`, inside the row-set region (checked in
     // the debug build against that region, so neither the reduction layout before it nor the
     // barrier row after it can be hit)
@@ -421,8 +419,7 @@ __device__ __forceinline__ void steps_energy_loop(R *phi_a, R *phi_b, Geom g, co
         if (!reducer && step < nsteps) {
             const R *src = (step & 1) ? phi_b : phi_a;
             R *dst = (step & 1) ? phi_a : phi_b;
-            for (long long s = (long long)blockIdx.x * blockDim.x + threadIdx.x; s < g.sites; s += stride)
-                site(src, dst, s, acc);
+            for (SiteWalk w = first; w.s < g.sites; w.advance(d, g)) site(src, dst, w, acc);
         }
         const unsigned gen = grid_arrive(bar);  // step's fields published (the final pass: rows only)
         if (!reducer && step < nsteps) {
@@ -440,24 +437,24 @@ __device__ __forceinline__ void steps_energy_loop(R *phi_a, R *phi_b, Geom g, co
 
 template <int NC>
 __global__ void __launch_bounds__(kEnergyThreads)
-    k_steps_energy_f64(double *phi_a, double *phi_b, double *__restrict__ pi, Geom g, Coef64 k, CoefE ke, int nsteps,
+    k_steps_energy_f64(double *phi_a, double *phi_b, double *__restrict__ pi, Geom g, Stride3 d, Coef64 k, CoefE ke, int nsteps,
                        double *__restrict__ scratch, double *__restrict__ records, unsigned polls) {
     __shared__ double sh[kNs<NC>][kEnergyThreads];
-    steps_energy_loop<NC>(phi_a, phi_b, g, ke, nsteps, scratch, records, polls, sh,
-                          [&](const double *src, double *dst, long long s, double (&acc)[kNs<NC>]) {
-                              site_step_energy_f64<NC, true>(src, dst, pi, s, g, k, ke, acc);
+    steps_energy_loop<NC>(phi_a, phi_b, g, d, ke, nsteps, scratch, records, polls, sh,
+                          [&](const double *src, double *dst, const SiteWalk &w, double (&acc)[kNs<NC>]) {
+                              site_step_energy_f64<NC, true>(src, dst, pi, w, g, k, ke, acc);
                           });
 }
 
 template <int NC, bool KAHAN>
 __global__ void __launch_bounds__(kEnergyThreads)
-    k_steps_energy_f32(float *phi_a, float *phi_b, float *__restrict__ pi, float *__restrict__ comp, Geom g, Coef32 k,
-                       CoefE ke, int nsteps, double *__restrict__ scratch, double *__restrict__ records,
+    k_steps_energy_f32(float *phi_a, float *phi_b, float *__restrict__ pi, float *__restrict__ comp, Geom g, Stride3 d,
+                       Coef32 k, CoefE ke, int nsteps, double *__restrict__ scratch, double *__restrict__ records,
                        unsigned polls) {
     __shared__ double sh[kNs<NC>][kEnergyThreads];
-    steps_energy_loop<NC>(phi_a, phi_b, g, ke, nsteps, scratch, records, polls, sh,
-                          [&](const float *src, float *dst, long long s, double (&acc)[kNs<NC>]) {
-                              site_step_energy_f32<NC, KAHAN, true>(src, dst, pi, comp, s, g, k, ke, acc);
+    steps_energy_loop<NC>(phi_a, phi_b, g, d, ke, nsteps, scratch, records, polls, sh,
+                          [&](const float *src, float *dst, const SiteWalk &w, double (&acc)[kNs<NC>]) {
+                              site_step_energy_f32<NC, KAHAN, true>(src, dst, pi, comp, w, g, k, ke, acc);
                           });
 }
 
@@ -472,10 +469,11 @@ template <typename R>
 cudaError_t launch_typed(const void *phi, const void *pi, const Geom &g, int ncomp, const CoefE &k, double *scratch,
                          double *record, cudaStream_t s) {
     const int nb = energy_grid(g.sites);
+    const Stride3 d = make_stride3((long long)nb * kEnergyThreads, g);
     switch (ncomp) {
 #define LF2_E(NC)                                                                                               \
     case NC:                                                                                                    \
-        k_energy<R, NC><<<nb, kEnergyThreads, 0, s>>>((const R *)phi, (const R *)pi, g, k, scratch, record); \
+        k_energy<R, NC><<<nb, kEnergyThreads, 0, s>>>((const R *)phi, (const R *)pi, g, d, k, scratch, record); \
         break;
         LF2_E(1) LF2_E(2) LF2_E(3) LF2_E(4) LF2_E(5) LF2_E(6)
 #undef LF2_E
@@ -486,18 +484,19 @@ cudaError_t launch_typed(const void *phi, const void *pi, const Geom &g, int nco
 
 template <int NC>
 void step_energy_nc(const StepArgs &a, const CoefE &ke, int nb, double *scratch, double *record, cudaStream_t s) {
+    const Stride3 d = make_stride3((long long)nb * kEnergyThreads, a.g);
     if (a.prec == LF2_F64) {
         k_step_energy_f64<NC><<<nb, kEnergyThreads, 0, s>>>((const double *)a.phi, (double *)a.phi_out, (double *)a.pi,
-                                                            a.g, make_coef64(a.p, a.dt), ke, scratch, record);
+                                                            a.g, d, make_coef64(a.p, a.dt), ke, scratch, record);
         return;
     }
     const Coef32 k = make_coef32(a.p, a.dt);
     if (a.prec == LF2_F32_KAHAN)
         k_step_energy_f32<NC, true><<<nb, kEnergyThreads, 0, s>>>((const float *)a.phi, (float *)a.phi_out,
-                                                                  (float *)a.pi, a.comp, a.g, k, ke, scratch, record);
+                                                                  (float *)a.pi, a.comp, a.g, d, k, ke, scratch, record);
     else
         k_step_energy_f32<NC, false><<<nb, kEnergyThreads, 0, s>>>((const float *)a.phi, (float *)a.phi_out,
-                                                                   (float *)a.pi, a.comp, a.g, k, ke, scratch, record);
+                                                                   (float *)a.pi, a.comp, a.g, d, k, ke, scratch, record);
 }
 
 // ------------------------------------------------------------ error norms (a12)
@@ -640,16 +639,17 @@ cudaError_t launch_cooperative(K kern, int nb, cudaStream_t s, Args... args) {
 template <int NC>
 cudaError_t steps_energy_nc(const StepArgs &a, int nsteps, int nb, const CoefE &ke, double *scratch, double *records,
                             unsigned polls, cudaStream_t s) {
+    const Stride3 d = make_stride3((long long)nb * kEnergyThreads, a.g);
     nb += 1;
     if (a.prec == LF2_F64)
         return launch_cooperative(k_steps_energy_f64<NC>, nb, s, (double *)a.phi, (double *)a.phi_out, (double *)a.pi,
-                                  a.g, make_coef64(a.p, a.dt), ke, nsteps, scratch, records, polls);
+                                  a.g, d, make_coef64(a.p, a.dt), ke, nsteps, scratch, records, polls);
     const Coef32 k = make_coef32(a.p, a.dt);
     if (a.prec == LF2_F32_KAHAN)
         return launch_cooperative(k_steps_energy_f32<NC, true>, nb, s, (float *)a.phi, (float *)a.phi_out,
-                                  (float *)a.pi, a.comp, a.g, k, ke, nsteps, scratch, records, polls);
+                                  (float *)a.pi, a.comp, a.g, d, k, ke, nsteps, scratch, records, polls);
     return launch_cooperative(k_steps_energy_f32<NC, false>, nb, s, (float *)a.phi, (float *)a.phi_out, (float *)a.pi,
-                              a.comp, a.g, k, ke, nsteps, scratch, records, polls);
+                              a.comp, a.g, d, k, ke, nsteps, scratch, records, polls);
 }
 
 }  // namespace

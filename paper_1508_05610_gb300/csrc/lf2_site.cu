@@ -24,13 +24,11 @@ __device__ __forceinline__ void load_site(const R *__restrict__ f, long long s, 
 
 template <int NC>
 __global__ void __launch_bounds__(kThreads) k_site_f64(const double *__restrict__ phi, double *__restrict__ phi_out,
-                                                       double *__restrict__ pi, Geom g, Coef64 k, int drift) {
-    const long long stride = (long long)gridDim.x * blockDim.x;
-    for (long long s = (long long)blockIdx.x * blockDim.x + threadIdx.x; s < g.sites; s += stride) {
-        const int x = (int)(s % g.nx);
-        const long long r = s / g.nx;
-        const int y = (int)(r % g.ny);
-        const int z = (int)(r / g.ny);
+                                                       double *__restrict__ pi, Geom g, Stride3 d, Coef64 k,
+                                                       int drift) {
+    for (SiteWalk w((long long)blockIdx.x * blockDim.x + threadIdx.x, g); w.s < g.sites; w.advance(d, g)) {
+        const long long s = w.s;
+        const int x = w.x, y = w.y, z = w.z;
         const long long row = (long long)g.nx;
         const long long plane = row * g.ny;
         double c[NC], xm[NC], xp[NC], ym[NC], yp[NC], zm[NC], zp[NC], p[NC], out[NC];
@@ -57,13 +55,10 @@ __global__ void __launch_bounds__(kThreads) k_site_f64(const double *__restrict_
 template <int NC, int MODE>
 __global__ void __launch_bounds__(kThreads) k_site_f32(const float *__restrict__ phi, float *__restrict__ phi_out,
                                                        float *__restrict__ pi, float *__restrict__ comp, Geom g,
-                                                       Coef32 k) {
-    const long long stride = (long long)gridDim.x * blockDim.x;
-    for (long long s = (long long)blockIdx.x * blockDim.x + threadIdx.x; s < g.sites; s += stride) {
-        const int x = (int)(s % g.nx);
-        const long long r = s / g.nx;
-        const int y = (int)(r % g.ny);
-        const int z = (int)(r / g.ny);
+                                                       Stride3 d, Coef32 k) {
+    for (SiteWalk w((long long)blockIdx.x * blockDim.x + threadIdx.x, g); w.s < g.sites; w.advance(d, g)) {
+        const long long s = w.s;
+        const int x = w.x, y = w.y, z = w.z;
         const long long row = (long long)g.nx;
         const long long plane = row * g.ny;
         float c[NC], xm[NC], xp[NC], ym[NC], yp[NC], zm[NC], zp[NC], p[NC], cm[NC], out[NC];
@@ -119,8 +114,9 @@ cudaError_t bounds_violations_site(unsigned long long *n, bool reset) { return b
 
 template <int NC>
 void site_launch(const StepArgs &a, int grid, cudaStream_t s) {
+    const Stride3 d = make_stride3((long long)grid * kThreads, a.g);
     if (a.prec == LF2_F64) {
-        k_site_f64<NC><<<grid, kThreads, 0, s>>>((const double *)a.phi, (double *)a.phi_out, (double *)a.pi, a.g,
+        k_site_f64<NC><<<grid, kThreads, 0, s>>>((const double *)a.phi, (double *)a.phi_out, (double *)a.pi, a.g, d,
                                                  make_coef64(a.p, a.dt), a.drift ? 1 : 0);
         return;
     }
@@ -128,11 +124,11 @@ void site_launch(const StepArgs &a, int grid, cudaStream_t s) {
     const float *phi = (const float *)a.phi;
     float *out = (float *)a.phi_out, *pi = (float *)a.pi;
     if (!a.drift)
-        k_site_f32<NC, 2><<<grid, kThreads, 0, s>>>(phi, out, pi, a.comp, a.g, k);
+        k_site_f32<NC, 2><<<grid, kThreads, 0, s>>>(phi, out, pi, a.comp, a.g, d, k);
     else if (a.prec == LF2_F32_KAHAN)
-        k_site_f32<NC, 1><<<grid, kThreads, 0, s>>>(phi, out, pi, a.comp, a.g, k);
+        k_site_f32<NC, 1><<<grid, kThreads, 0, s>>>(phi, out, pi, a.comp, a.g, d, k);
     else
-        k_site_f32<NC, 0><<<grid, kThreads, 0, s>>>(phi, out, pi, a.comp, a.g, k);
+        k_site_f32<NC, 0><<<grid, kThreads, 0, s>>>(phi, out, pi, a.comp, a.g, d, k);
 }
 
 cudaError_t launch_site_step(const StepArgs &a, cudaStream_t s) {
