@@ -365,6 +365,222 @@ __device__ __forceinline__ void tb_iteration(TbState<R, T, CX * NC> &st, R *__re
         __syncthreads();
 }
 
+// ------------------------------------------------ FP32, packed pairs (f32x2) throughout
+// The wavefront of FP32 threads with 4 or 6 values per plane, on pairs: two adjacent columns of a
+// real field, two components of a site otherwise.  Bound: the FMA pipe (a packed instruction holds
+// it for two cycles, as two scalar ones do) with the warps in step at the barrier of every plane.
+// Against tb_iteration, which updates each site from its six neighbours:
+//   - differences are shared: phi(z+1) - phi(z) of one plane is, negated, the phi(z-1) - phi(z) of
+//     the next, so each level keeps its centre plane and that difference in registers instead of
+//     three planes; and in x, phi(x+1) - phi(x) serves both its columns.  Rounding is symmetric,
+//     RN(a - b) = -RN(b - a), so every sum keeps its bits (a zero may keep another sign).  77 instead of 84 FMA cycles and 43
+//     instead of 54 instructions for the arithmetic of a stage of 4 real sites;
+//   - with the region's size fixed at compile time (16 threads x 32 rows, the best of the tuner's
+//     regions for one and two components) the shared addresses are immediates, which leaves
+//     registers to issue ahead;
+//   - the next plane's loads stand first in the iteration and stay there.
+// 512^3 real, depth 4, 56x24 tiles, FP32+Kahan: 576 -> 673 GSU/s (warp instructions 398 -> 299 M a
+// pass of 512x512x256, FMA pipe 66 -> 61 % busy in 486 -> 406 us); 256^3 complex, 24x24: 249 -> 275.
+// Tried and slower: momentum and compensation in fixed register slots with the loop unrolled over
+// them (fewer copies, but spills: 601), unrolled by two (637), coefficients in scalar instructions
+// from the constant bank (597), loads through cp.async (556), L2 prefetches (620), 8 values per
+// thread in 256 threads (235 complex), a split mbarrier in place of __syncthreads (668).
+// Loads issued where they stand: the compiler sank plain ones towards their use, an iteration later.
+template <int N>
+__device__ __forceinline__ void vload_early(const float *__restrict__ p, float (&v)[N]) {
+    using C = VecChunk<float, N>;
+#pragma unroll
+    for (int q = 0; q < C::COUNT; ++q) {
+        const float *a = p + q * C::E;
+        float *d = v + q * C::E;
+        if constexpr (C::CH == 16)
+            asm volatile("ld.global.nc.v4.f32 {%0, %1, %2, %3}, [%4];\n" : "=f"(d[0]), "=f"(d[1]), "=f"(d[2]), "=f"(d[3]) : "l"(a));
+        else if constexpr (C::CH == 8)
+            asm volatile("ld.global.nc.v2.f32 {%0, %1}, [%2];\n" : "=f"(d[0]), "=f"(d[1]) : "l"(a));
+        else
+            asm volatile("ld.global.nc.f32 %0, [%1];\n" : "=f"(d[0]) : "l"(a));
+    }
+}
+
+template <int T, int P>
+struct PairState {
+    f32x2 c[T][P];             // level l (0..T-1): the plane stage l+1 centres on next
+    f32x2 d[T][P];             // its difference to the plane below, phi(q) - phi(q-1)
+    f32x2 pi[T][P], cm[T][P];  // momentum and compensation of planes i-1, ..., i-T
+    float in_phi[2 * P], in_pi[2 * P], in_cm[2 * P];  // loaded ahead: phi of plane i+1, the others of plane i
+};
+
+template <int N>
+__device__ __forceinline__ void pack(const float (&v)[N], f32x2 (&p)[N / 2]) {
+#pragma unroll
+    for (int q = 0; q < N / 2; ++q) p[q] = pk2(v[2 * q], v[2 * q + 1]);
+}
+template <int N>
+__device__ __forceinline__ void unpack(const f32x2 (&p)[N / 2], float (&v)[N]) {
+#pragma unroll
+    for (int q = 0; q < N / 2; ++q) up2(p[q], v[2 * q], v[2 * q + 1]);
+}
+
+// Iteration i of the wavefront.  cur, prev, ps2, row_e, push, rank, band as in tb_iteration;
+// phi_next: plane i+1, pi_now / cm_now: plane i (loads of own columns).
+template <int NC, int MODE, int T, int CX, int CL>
+__device__ __forceinline__ void pair_iteration(PairState<T, CX * NC / 2> &st, float *__restrict__ cur,
+                                               const float *__restrict__ prev, int ps2, int row_e, const Coef32 &k,
+                                               const float *__restrict__ phi_next, const float *__restrict__ pi_now,
+                                               const float *__restrict__ cm_now, bool store, float *__restrict__ ophi, float *__restrict__ opi,
+                                               float *__restrict__ ocomp, bool shfl_x, unsigned push, unsigned rank,
+                                               int band) {
+    constexpr int W = CX * NC, P = W / 2;
+    const Coef32x2 k2 = make_coef32x2(k, k.zero);
+    f32x2 up_level[P];  // the plane above each stage's centre: level s-1 as it was just made
+    pack<W>(st.in_phi, up_level);
+    vstore_s<float, W>(cur, st.in_phi);
+    push_edges<float, W, CL>(cur, push, rank, band, st.in_phi);
+    vload_early<W>(phi_next, st.in_phi);
+#pragma unroll
+    for (int l = T - 1; l > 0; --l)
+#pragma unroll
+        for (int q = 0; q < P; ++q) {
+            st.pi[l][q] = st.pi[l - 1][q];
+            if (MODE == 1) st.cm[l][q] = st.cm[l - 1][q];
+        }
+    pack<W>(st.in_pi, st.pi[0]);
+    vload_early<W>(pi_now, st.in_pi);
+    if (MODE == 1) {
+        pack<W>(st.in_cm, st.cm[0]);
+        vload_early<W>(cm_now, st.in_cm);
+    }
+#pragma unroll
+    for (int s = 1; s <= T; ++s) {
+        f32x2(&C)[P] = st.c[s - 1];
+        f32x2(&D)[P] = st.d[s - 1];
+        const float *src = prev + (s - 1) * ps2;
+        f32x2 dsum[P], dy[P];
+        {
+            float v[W];
+            f32x2 w[P];
+            vload_s<float, W>(src + row_e, v);
+            pack<W>(v, w);
+#pragma unroll
+            for (int q = 0; q < P; ++q) dy[q] = sub2(w[q], C[q]);
+            vload_s<float, W>(src - row_e, v);
+            pack<W>(v, w);
+#pragma unroll
+            for (int q = 0; q < P; ++q) dy[q] = add2(sub2(w[q], C[q]), dy[q]);
+        }
+        // x: differences between neighbouring columns, then of neighbouring differences
+        float cv[W], left[NC], right[NC];
+        unpack<W>(C, cv);
+        if (shfl_x) {
+#pragma unroll
+            for (int a = 0; a < NC; ++a) {
+                left[a] = __shfl_up_sync(0xffffffffu, cv[(CX - 1) * NC + a], 1);
+                right[a] = __shfl_down_sync(0xffffffffu, cv[a], 1);
+            }
+        } else {
+#pragma unroll
+            for (int a = 0; a < NC; ++a) {
+                left[a] = src[a - NC];
+                right[a] = src[W + a];
+            }
+        }
+        if constexpr (NC == 1) {
+            float e[CX + 1];
+            e[0] = __fsub_rn(cv[0], left[0]);
+#pragma unroll
+            for (int j = 1; j < CX; ++j) e[j] = __fsub_rn(cv[j], cv[j - 1]);
+            e[CX] = __fsub_rn(right[0], cv[CX - 1]);
+#pragma unroll
+            for (int q = 0; q < P; ++q)
+                dsum[q] = pk2(__fsub_rn(e[2 * q + 1], e[2 * q]), __fsub_rn(e[2 * q + 2], e[2 * q + 1]));
+        } else {
+            constexpr int H = NC / 2;  // pairs per site
+#pragma unroll
+            for (int h = 0; h < H; ++h) {
+                f32x2 e = sub2(C[h], pk2(left[2 * h], left[2 * h + 1]));
+#pragma unroll
+                for (int j = 0; j < CX; ++j) {
+                    const f32x2 nx = j == CX - 1 ? pk2(right[2 * h], right[2 * h + 1]) : C[(j + 1) * H + h];
+                    const f32x2 f = sub2(nx, C[j * H + h]);
+                    dsum[j * H + h] = sub2(f, e);
+                    e = f;
+                }
+            }
+        }
+#pragma unroll
+        for (int q = 0; q < P; ++q) {
+            const f32x2 dn = sub2(up_level[q], C[q]);
+            const f32x2 dz = sub2(dn, D[q]);
+            D[q] = dn;
+            dsum[q] = add2(add2(dsum[q], dy[q]), dz);
+        }
+        // minus the potential's coefficient, per pair
+        f32x2 ng[P];
+        if constexpr (NC == 1) {
+#pragma unroll
+            for (int q = 0; q < P; ++q) {
+                const f32x2 s2 = fma2(C[q], C[q], k2.zero);
+                ng[q] = fma2(k2.nlam, sub2(s2, k2.eta2), k2.nm2);
+            }
+        } else {
+#pragma unroll
+            for (int j = 0; j < CX; ++j) {
+                float s2 = __fmul_rn(cv[j * NC], cv[j * NC]);
+#pragma unroll
+                for (int a = 1; a < NC; ++a) s2 = __fmaf_rn(cv[j * NC + a], cv[j * NC + a], s2);
+                const float g = __fmaf_rn(-k.lam, __fsub_rn(s2, k.eta2), -k.m2);
+#pragma unroll
+                for (int h = 0; h < NC / 2; ++h) ng[j * (NC / 2) + h] = pk2(g, g);
+            }
+        }
+        f32x2 out[P];
+        f32x2(&pn)[P] = st.pi[s - 1];
+        f32x2(&cn)[P] = st.cm[s - 1];
+#pragma unroll
+        for (int q = 0; q < P; ++q) {
+            const f32x2 F = fma2(dsum[q], k2.inv_dx2, mul2(ng[q], C[q]));
+            pn[q] = fma2(k2.dt, F, pn[q]);
+            if (MODE == 1) {
+                const f32x2 ny = fma2(k2.ndt, pn[q], cn[q]);
+                const f32x2 t = sub2(C[q], ny);
+                cn[q] = add2(sub2(t, C[q]), ny);
+                out[q] = t;
+            } else {
+                out[q] = fma2(k2.dt, pn[q], C[q]);
+            }
+            C[q] = up_level[q];
+        }
+        float v[W];
+        unpack<W>(out, v);
+        if (s < T) {
+#pragma unroll
+            for (int q = 0; q < P; ++q) up_level[q] = out[q];
+            vstore_s<float, W>(cur + s * ps2, v);
+            push_edges<float, W, CL>(cur + s * ps2, push, rank, band, v);
+        } else if (store) {
+            vstore_g<float, W>(ophi, v);
+            unpack<W>(pn, v);
+            vstore_g<float, W>(opi, v);
+            if (MODE == 1) {
+                unpack<W>(cn, v);
+                vstore_g<float, W>(ocomp, v);
+            }
+        }
+    }
+    if constexpr (CL > 1)
+        cluster_sync();
+    else
+        __syncthreads();
+}
+
+// Whether a configuration runs on pairs: 16 or 24 bytes per thread and plane (8-byte threads share
+// an SM between two blocks of 64 registers a thread, which pairs exceed; 6 components with the plain
+// drift are 2 % slower on pairs, with the compensated one 5 to 8 % faster).
+template <int NC, int MODE, int CX>
+constexpr bool tb_pairs() {
+    return MODE != 3 && CX * NC >= 4 && (NC == 1 ? CX % 2 == 0 : NC % 2 == 0) && !(NC == 6 && MODE == 0);
+}
+
 // MODE: 0 = FP32 plain drift, 1 = FP32 Kahan drift, 3 = FP64.
 // Light configurations (shallow, narrow) are held to 64 registers so two blocks fit per SM.
 template <typename R, int NC, int T, int CX>
@@ -372,10 +588,17 @@ constexpr int tb_min_blocks() {
     return (T <= 4 && CX * NC * sizeof(R) <= 8) ? 2 : 1;
 }
 
+// The region that passes on pairs have as compile-time constants (FIXED): 16 threads x 32 rows.
+constexpr int kFixedThreadsX = 16, kFixedRows = 32;
+template <int NC, int MODE, int T, int CX>
+constexpr bool tb_fixed_built() {
+    return tb_pairs<NC, MODE, CX>() && NC <= 2 && T <= 4;
+}
+
 // One tile x z-chunk of a temporal-blocking pass: (bx, by) is the tile, bz the chunk.  With
 // CL > 1 the tile's region rows (TY + 2T) are split into CL bands of equal height, one per CTA
 // of a cluster, and `rank` is this CTA's band; CL = 1 is one CTA per tile.
-template <typename R, int NC, int MODE, int T, int CX, typename CoefT, int CL = 1>
+template <typename R, int NC, int MODE, int T, int CX, typename CoefT, int CL = 1, bool FIXED = false>
 __device__ __forceinline__ void tb_block(const R *__restrict__ phi, R *__restrict__ phi_out, const R *__restrict__ pi,
                                          R *__restrict__ pi_out, const float *__restrict__ comp,
                                          float *__restrict__ comp_out, const Geom &g, const CoefT &k, int TX, int TY,
@@ -385,7 +608,7 @@ __device__ __forceinline__ void tb_block(const R *__restrict__ phi, R *__restric
     extern __shared__ __align__(16) unsigned char smem_raw[];
     R *sm = reinterpret_cast<R *>(smem_raw);
 
-    const int RX = TX + 2 * TP, RY = (TY + 2 * T) / CL;  // RY: this CTA's rows
+    const int RX = FIXED ? kFixedThreadsX * CX : TX + 2 * TP, RY = FIXED ? kFixedRows : (TY + 2 * T) / CL;  // RY: this CTA's rows
     const int RXT = RX / CX;
     const int ps = (RY + 2) * RX * NC;  // elements per shared plane (one halo row above and below)
     const int t = threadIdx.x;
@@ -410,32 +633,8 @@ __device__ __forceinline__ void tb_block(const R *__restrict__ phi, R *__restric
     // edge rows of a band with a neighbouring band in the cluster
     const unsigned push = CL > 1 ? ((ry == 0 && rank > 0) ? 1u : 0u) | ((ry == RY - 1 && rank + 1 < CL) ? 2u : 0u) : 0u;
 
-    TbState<R, T, W> st;
-#pragma unroll
-    for (int l = 0; l < T; ++l)
-#pragma unroll
-        for (int m = 0; m < 3; ++m)
-#pragma unroll
-            for (int e = 0; e < W; ++e) st.lv[l][m][e] = R(0);
-#pragma unroll
-    for (int l = 0; l <= T; ++l)
-#pragma unroll
-        for (int e = 0; e < W; ++e) st.pq[l][e] = st.cq[l][e] = R(0);
-#pragma unroll
-    for (int e = 0; e < W; ++e) st.pf_c[e] = R(0);
-
     // plane index of the next load, advanced with a compare instead of a modulo
     int pl = wrap_any(z0 - T, g.nz);
-    {
-#ifdef LF2_DEBUG_BOUNDS
-        const long long off = checked((long long)pl * planeE + colE, W, total);
-#else
-        const long long off = (long long)pl * planeE + colE;
-#endif
-        vload_g<R, W>(phi + off, st.pf_phi);
-        vload_cg<R, W>(pi + off, st.pf_pi);
-        if (MODE == 1) vload_cg<R, W>(reinterpret_cast<const R *>(comp) + off, st.pf_c);
-    }
     const int ibeg = z0 - T, iend = z1 + T;
     // output plane of stage T in iteration i is i - T; stores start at i = z0 + T
     long long out_off = (long long)(z0 - 2 * T - 1) * planeE + colE;  // advanced before each use
@@ -450,38 +649,96 @@ __device__ __forceinline__ void tb_block(const R *__restrict__ phi, R *__restric
 #endif
     // x-neighbours by warp shuffle when every region row is a whole group of lanes within one
     // warp and the block is whole warps
-    const bool shfl_x = (32 % RXT == 0) && ((RXT * RY) % 32 == 0);
-    for (int i = ibeg; i < iend; ++i) {
-        pl = (pl + 1 == g.nz) ? 0 : pl + 1;
+    const bool shfl_x = FIXED || ((32 % RXT == 0) && ((RXT * RY) % 32 == 0));
+    if constexpr (tb_pairs<NC, MODE, CX>()) {
+        PairState<T, W / 2> st;
+#pragma unroll
+        for (int e = 0; e < W; ++e) st.in_pi[e] = st.in_cm[e] = 0.0f;
+#pragma unroll
+        for (int q = 0; q < W / 2; ++q) {
+#pragma unroll
+            for (int l = 0; l < T; ++l) st.c[l][q] = st.d[l][q] = st.pi[l][q] = st.cm[l][q] = 0ull;
+        }
 #ifdef LF2_DEBUG_BOUNDS
-        const long long noff = checked((long long)pl * planeE + colE, W, total);
+        long long off = checked((long long)pl * planeE + colE, W, total);
 #else
-        const long long noff = (long long)pl * planeE + colE;
+        long long off = (long long)pl * planeE + colE;  // plane i
 #endif
-        out_off += planeE;
-        const int par = i & 1;
+        vload_g<float, W>(phi + off, st.in_phi);
+        for (int i = ibeg; i < iend; ++i) {
+            pl = (pl + 1 == g.nz) ? 0 : pl + 1;  // also after the last plane: a load inside the lattice, unused
+            out_off += planeE;
+            const int par = i & 1;
+            const bool store = out_col && i - T >= z0;
 #ifdef LF2_DEBUG_BOUNDS
-        const bool store = out_col && i - T >= z0;
-        const long long oo = store ? checked(out_off, W, total) : out_off;
-        tb_iteration<R, NC, MODE, T, CX, CoefT, CL>(st, base + par * ps, base + (par ^ 1) * ps, 2 * ps, row_e, k,
-                                                    i + 1 < iend, phi + noff, pi + noff, comp + noff, store,
-                                                    phi_out + oo, pi_out + oo, comp_out + oo, shfl_x, push, rank,
-                                                    RY * row_e);
+            const long long noff = checked((long long)pl * planeE + colE, W, total);
+            const long long oo = store ? checked(out_off, W, total) : out_off;
 #else
-        tb_iteration<R, NC, MODE, T, CX, CoefT, CL>(st, base + par * ps, base + (par ^ 1) * ps, 2 * ps, row_e, k,
-                                                    i + 1 < iend, phi + noff, pi + noff, comp + noff,
-                                                    out_col && i - T >= z0, phi_out + out_off, pi_out + out_off,
-                                                    comp_out + out_off, shfl_x, push, rank, RY * row_e);
+            const long long noff = (long long)pl * planeE + colE;
+            const long long oo = out_off;
 #endif
+            pair_iteration<NC, MODE, T, CX, CL>(st, base + par * ps, base + (par ^ 1) * ps, 2 * ps, row_e, k, phi + noff,
+                                                pi + off, comp + off, store, phi_out + oo, pi_out + oo, comp_out + oo,
+                                                shfl_x, push, rank, RY * row_e);
+            off = noff;
+        }
+    } else {
+        TbState<R, T, W> st;
+#pragma unroll
+        for (int l = 0; l < T; ++l)
+#pragma unroll
+            for (int m = 0; m < 3; ++m)
+#pragma unroll
+                for (int e = 0; e < W; ++e) st.lv[l][m][e] = R(0);
+#pragma unroll
+        for (int l = 0; l <= T; ++l)
+#pragma unroll
+            for (int e = 0; e < W; ++e) st.pq[l][e] = st.cq[l][e] = R(0);
+#pragma unroll
+        for (int e = 0; e < W; ++e) st.pf_c[e] = R(0);
+
+        {
+#ifdef LF2_DEBUG_BOUNDS
+            const long long off = checked((long long)pl * planeE + colE, W, total);
+#else
+            const long long off = (long long)pl * planeE + colE;
+#endif
+            vload_g<R, W>(phi + off, st.pf_phi);
+            vload_cg<R, W>(pi + off, st.pf_pi);
+            if (MODE == 1) vload_cg<R, W>(reinterpret_cast<const R *>(comp) + off, st.pf_c);
+        }
+        for (int i = ibeg; i < iend; ++i) {
+            pl = (pl + 1 == g.nz) ? 0 : pl + 1;
+#ifdef LF2_DEBUG_BOUNDS
+            const long long noff = checked((long long)pl * planeE + colE, W, total);
+#else
+            const long long noff = (long long)pl * planeE + colE;
+#endif
+            out_off += planeE;
+            const int par = i & 1;
+#ifdef LF2_DEBUG_BOUNDS
+            const bool store = out_col && i - T >= z0;
+            const long long oo = store ? checked(out_off, W, total) : out_off;
+            tb_iteration<R, NC, MODE, T, CX, CoefT, CL>(st, base + par * ps, base + (par ^ 1) * ps, 2 * ps, row_e, k,
+                                                        i + 1 < iend, phi + noff, pi + noff, comp + noff, store,
+                                                        phi_out + oo, pi_out + oo, comp_out + oo, shfl_x, push, rank,
+                                                        RY * row_e);
+#else
+            tb_iteration<R, NC, MODE, T, CX, CoefT, CL>(st, base + par * ps, base + (par ^ 1) * ps, 2 * ps, row_e, k,
+                                                        i + 1 < iend, phi + noff, pi + noff, comp + noff,
+                                                        out_col && i - T >= z0, phi_out + out_off, pi_out + out_off,
+                                                        comp_out + out_off, shfl_x, push, rank, RY * row_e);
+#endif
+        }
     }
 }
 
-template <typename R, int NC, int MODE, int T, int CX, typename CoefT>
+template <typename R, int NC, int MODE, int T, int CX, typename CoefT, bool FIXED>
 __global__ void __launch_bounds__(kTbMaxThreads, (tb_min_blocks<R, NC, T, CX>()))
     k_tblock(const R *__restrict__ phi, R *__restrict__ phi_out, const R *__restrict__ pi, R *__restrict__ pi_out,
              const float *__restrict__ comp, float *__restrict__ comp_out, Geom g, CoefT k, int TX, int TY,
              int zchunk) {
-    tb_block<R, NC, MODE, T, CX, CoefT>(phi, phi_out, pi, pi_out, comp, comp_out, g, k, TX, TY, zchunk, blockIdx.x,
+    tb_block<R, NC, MODE, T, CX, CoefT, 1, FIXED>(phi, phi_out, pi, pi_out, comp, comp_out, g, k, TX, TY, zchunk, blockIdx.x,
                                         blockIdx.y, blockIdx.z);
 }
 
@@ -499,7 +756,7 @@ __global__ void __launch_bounds__(kTbMaxThreads, 1)
 // Ensemble pass: one launch covers the tiles of every member lattice, items ordered longest
 // chunk first.  Which block computes an item does not change its result, so the dynamic
 // assignment keeps the output bitwise deterministic.
-template <typename R, int NC, int MODE, int T, int CX, typename CoefT>
+template <typename R, int NC, int MODE, int T, int CX, typename CoefT, bool FIXED>
 __global__ void __launch_bounds__(kTbMaxThreads, (tb_min_blocks<R, NC, T, CX>()))
     k_tblock_ensemble(const TbMember *__restrict__ members, const int4 *__restrict__ items, int nitems, int flip,
                       int TX, int TY, int *__restrict__ counter) {
@@ -521,9 +778,9 @@ __global__ void __launch_bounds__(kTbMaxThreads, (tb_min_blocks<R, NC, T, CX>())
             k = m.k64;
         else
             k = m.k32;
-        tb_block<R, NC, MODE, T, CX, CoefT>((const R *)m.phi[f], (R *)m.phi[f ^ 1], (const R *)m.pi[f],
-                                            (R *)m.pi[f ^ 1], m.comp[f], const_cast<float *>(m.comp[f ^ 1]), m.g, k, TX, TY, m.zchunk,
-                                            w.y, w.z, w.w);
+        tb_block<R, NC, MODE, T, CX, CoefT, 1, FIXED>((const R *)m.phi[f], (R *)m.phi[f ^ 1], (const R *)m.pi[f],
+                                                      (R *)m.pi[f ^ 1], m.comp[f], const_cast<float *>(m.comp[f ^ 1]),
+                                                      m.g, k, TX, TY, m.zchunk, w.y, w.z, w.w);
         __syncthreads();
     }
 }
@@ -534,7 +791,9 @@ cudaError_t launch_t(const TbArgs &a, const TbConfig &c, const CoefT &k, cudaStr
     const int RX = c.tile_x + 2 * TP, RY = c.tile_y + 2 * T;
     const int threads = (RX / CX) * RY;
     const size_t smem = (size_t)2 * T * (RY + 2) * RX * NC * sizeof(R);
-    auto kern = k_tblock<R, NC, MODE, T, CX, CoefT>;
+    auto kern = k_tblock<R, NC, MODE, T, CX, CoefT, false>;
+    if constexpr (tb_fixed_built<NC, MODE, T, CX>())
+        if (RX == kFixedThreadsX * CX && RY == kFixedRows) kern = k_tblock<R, NC, MODE, T, CX, CoefT, true>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     dim3 grid((a.g.nx + c.tile_x - 1) / c.tile_x, (a.g.ny + c.tile_y - 1) / c.tile_y,
@@ -606,7 +865,9 @@ cudaError_t launch_ens_t(const TbEnsembleLaunch &e, cudaStream_t s) {
     const int RX = e.c.tile_x + 2 * TP, RY = e.c.tile_y + 2 * T;
     const int threads = (RX / CX) * RY;
     const size_t smem = (size_t)2 * T * (RY + 2) * RX * NC * sizeof(R);
-    auto kern = k_tblock_ensemble<R, NC, MODE, T, CX, CoefT>;
+    auto kern = k_tblock_ensemble<R, NC, MODE, T, CX, CoefT, false>;
+    if constexpr (tb_fixed_built<NC, MODE, T, CX>())
+        if (RX == kFixedThreadsX * CX && RY == kFixedRows) kern = k_tblock_ensemble<R, NC, MODE, T, CX, CoefT, true>;
     cudaError_t err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (err != cudaSuccess) return err;
     int per_sm = 0;
