@@ -77,11 +77,22 @@ inline CoefE make_coefE(const lf2_params &p) {
 // with them.  Operands outside the grid's range (E < 64: all zero or below 2^-959; E >= 2040: huge,
 // infinite or NaN) are added in FP64.
 //
-// hi/lo: the operands' high and low words.
 __device__ __forceinline__ unsigned long long shr_clamped(unsigned long long v, unsigned n) {
     unsigned long long r;
     asm("shr.u64 %0, %1, %2;" : "=l"(r) : "l"(v), "r"(n));  // shifts of 64 and more give 0
     return r;
+}
+
+// acc (|acc| < 2^63) times 2^(x0 - 1086), rounded once to nearest even; +0 for 0.  The exponent field
+// of the result, x0 - (leading zeros of |acc|), must lie in the normal range.
+__device__ __forceinline__ double round_fixed(unsigned long long acc, int x0) {
+    const int sign = (int)(acc >> 32) >> 31;
+    const unsigned long long n0 = (acc ^ (unsigned long long)(long long)sign) - (unsigned long long)(long long)sign;
+    const int lz = __clzll((long long)n0);  // 1 to 63, or 64 for 0
+    const unsigned long long n = n0 << (lz - 1);  // leading bit at 62: 10 bits below the 53
+    const unsigned long long r = (n + 0x1ffu + ((n >> 10) & 1u)) >> 10;
+    const unsigned hi = (unsigned)(r >> 32) + ((unsigned)(x0 - 1 - lz) << 20);  // the hidden bit adds 1
+    return n0 ? __hiloint2double((int)(hi | ((unsigned)sign & 0x80000000u)), (int)(unsigned)r) : 0.0;
 }
 
 // The sum in FP64.  A function of its own: inlined, its five additions were issued under a false
@@ -108,13 +119,7 @@ __device__ __forceinline__ double sum6(double a, double b, double c, double d, d
         const long long s = (long long)(hi >> 31);
         acc += (m ^ (unsigned long long)s) - (unsigned long long)s;  // +-m
     }
-    const int sign = (int)(acc >> 32) >> 31;
-    const unsigned long long n0 = (acc ^ (unsigned long long)(long long)sign) - (unsigned long long)(long long)sign;
-    const int lz = __clzll((long long)n0);  // 1 to 63, or 64 for a zero sum
-    const unsigned long long n = n0 << (lz - 1);  // leading bit at 62: 10 bits below the 53
-    const unsigned long long r = (n + 0x1ffu + ((n >> 10) & 1u)) >> 10;
-    const unsigned hi = (unsigned)(r >> 32) + ((unsigned)(E + 3 - lz) << 20);  // the hidden bit adds 1
-    return n0 ? __hiloint2double((int)(hi | ((unsigned)sign & 0x80000000u)), (int)(unsigned)r) : 0.0;
+    return round_fixed(acc, (int)E + 4);
 }
 
 // FP64 kick (+ drift).  pi <- pi + dt F(phi);  phi_out <- phi + dt pi.

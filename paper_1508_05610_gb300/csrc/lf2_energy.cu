@@ -31,6 +31,14 @@ namespace {
 // doubles of which the first kNs<NC> are used.
 template <int NC>
 constexpr int kNs = 3 + 2 * NC;
+// Resident blocks per SM that the kernels' registers allow: four for one component (64 registers),
+// two for more (128).  The full grid is four blocks per SM, so four or two resident blocks run it in
+// whole waves, where three leave the fourth block alone on its SM (256^3 real FP32 energy with 72
+// registers: 470 us, with 64: 387 us).  5 and 6 components would take up to 185 registers by
+// themselves, one block per SM (96x80x112 6-component FP32 step with energy 1818 us, now 980 us
+// for 8 steps).  The multi-step launch counts on two.
+template <int NC>
+constexpr int kEnergyResident = NC == 1 ? 4 : 2;
 constexpr int kKin = 0, kGrad = 1, kPot = 2, kSum = 3;
 
 // L2 loads (COHERENT) where other blocks of the same launch wrote the data; the read-only
@@ -64,34 +72,127 @@ __device__ __forceinline__ double widen(float v) {
 }
 
 template <typename R, int NC, bool COHERENT = false>
-__device__ __forceinline__ void load_d(const R *__restrict__ f, long long s, long long sites, double (&v)[NC]) {
+__device__ __forceinline__ void load_site(const R *__restrict__ f, long long s, long long sites, R (&v)[NC]) {
     const long long i = checked(s * NC, NC, sites * NC);
 #pragma unroll
-    for (int a = 0; a < NC; ++a) v[a] = widen(ld_field<COHERENT>(f + i + a));
+    for (int a = 0; a < NC; ++a) v[a] = ld_field<COHERENT>(f + i + a);
 }
 
-// Adds one site's raw sums to acc.  c: phi_n at the site, xp, yp, zp: its neighbours +x, +y, +z;
-// nb: its neighbour sums (sum6); p: pi_{n-1/2}.  Explicit round-to-nearest operations keep the
-// stand-alone and fused kernels bitwise equal; the half kick is the FP64 kick's arithmetic.
-template <int NC>
-__device__ __forceinline__ void energy_site(const double (&c)[NC], const double (&xp)[NC], const double (&yp)[NC],
-                                            const double (&zp)[NC], const double (&nb)[NC], const double (&p)[NC],
-                                            double (&acc)[kNs<NC>], const CoefE &k) {
-    double s2 = __dmul_rn(c[0], c[0]);
+// --------------------------------------- sums and differences of the energy, in integers
+// The FP64 pipe bounds the energy kernels while the integer pipes have time left (see sum6), so the
+// forward differences are subtracted as integers too: both significands on one grid, an exact
+// difference, rounded once.  FP32 values are widened for the FP64 energy, and their neighbour sums
+// and differences are taken directly from the FP32 words: each operand is its signed 24-bit
+// significand times a power of two, one wide multiply-add.  All bit for bit the FP64 operations on
+// the (widened) values; operands outside a fast range (orders of magnitude apart, tiny, huge,
+// infinite, NaN) take those, in functions of their own so that their instructions are not issued
+// under a false predicate.
+// 256^3, one energy: 1 component FP64 476 -> 390 us, 2 components 811 -> 718 (differences);
+// FP32 storage 485 -> 387 and 854 -> 657 us (sums and differences).
+__device__ __noinline__ double sum6_widened(float a, float b, float c, float d, float e, float f) {
+    return sum6(widen(a), widen(b), widen(c), widen(d), widen(e), widen(f));
+}
+__device__ __noinline__ double sub_widened(float a, float b) { return __dsub_rn(widen(a), widen(b)); }
+
+// The signed 24-bit significand of a normal number.
+__device__ __forceinline__ int significand(float v) {
+    const int u = __float_as_int(v), s = u >> 31;
+    return (((u & 0x007fffff) | 0x00800000) ^ s) - s;
+}
+__device__ __forceinline__ unsigned magnitude(float v) { return __float_as_uint(v) & 0x7fffffffu; }
+// 2^n for n in 0..31, 0 for any other n (as unsigned)
+__device__ __forceinline__ int pow2_clamped(unsigned n) {
+    int r;
+    asm("shl.b32 %0, 1, %1;" : "=r"(r) : "r"(n));
+    return r;
+}
+
+__device__ __forceinline__ double neighbour_sum(double a, double b, double c, double d, double e, double f) {
+    return sum6(a, b, c, d, e, f);
+}
+__device__ __forceinline__ double neighbour_sum(float a, float b, float c, float d, float e, float f) {
+    const float v[6] = {a, b, c, d, e, f};
+    unsigned m[6];
 #pragma unroll
-    for (int b = 1; b < NC; ++b) s2 = __fma_rn(c[b], c[b], s2);
+    for (int i = 0; i < 6; ++i) m[i] = magnitude(v[i]);
+    const unsigned hi = __vimax3_u32(__vimax3_u32(m[0], m[1], m[2]), __vimax3_u32(m[3], m[4], m[5]), 0u);
+    // the smallest but for zeros, which wrap to the largest and contribute nothing below
+    const unsigned lo = __vimin3_u32(__vimin3_u32(m[0] - 1u, m[1] - 1u, m[2] - 1u),
+                                     __vimin3_u32(m[3] - 1u, m[4] - 1u, m[5] - 1u), 0xffffffffu);
+    const unsigned E = hi >> 23;
+    // m - 1 may have an exponent one lower: 29 binary orders keep every operand within 30
+    if (E - 32u >= 255u - 32u || (lo >> 23) + 29u < E) return sum6_widened(a, b, c, d, e, f);
+    long long acc = 0;
+#pragma unroll
+    for (int i = 0; i < 6; ++i) acc += (long long)significand(v[i]) * pow2_clamped(30u - E + (m[i] >> 23));
+    return round_fixed((unsigned long long)acc, (int)E + 906);
+}
+
+// a - b, exact in FP64 when the exponents are at most 28 apart.
+__device__ __forceinline__ double sub_exact(float a, float b) {
+    const unsigned ma = magnitude(a), mb = magnitude(b);
+    const unsigned E = max(ma, mb) >> 23, F = min(ma, mb) >> 23;
+    if (F - 1u >= 254u || E == 255u || F + 28u < E) return sub_widened(a, b);  // F = 0: zero or subnormal
+    const unsigned long long d = (unsigned long long)((long long)significand(a) * pow2_clamped(28u - E + (ma >> 23)) -
+                                                      (long long)significand(b) * pow2_clamped(28u - E + (mb >> 23)));
+    const int sign = (int)(d >> 32) >> 31;
+    const unsigned long long n0 = (d ^ (unsigned long long)(long long)sign) - (unsigned long long)(long long)sign;
+    const int lz = __clzll((long long)n0);        // 11 to 63, or 64 for 0
+    const unsigned long long n = n0 << (lz - 11);  // leading bit at 52, nothing to round
+    const unsigned hi = (unsigned)(n >> 32) + ((E + 907u - (unsigned)lz) << 20);
+    return n0 ? __hiloint2double((int)(hi | ((unsigned)sign & 0x80000000u)), (int)(unsigned)n) : 0.0;
+}
+// FP64: with exponents at most 9 apart no bit is lost and the difference stays below 2^63.
+__device__ __noinline__ double sub_fp64(double a, double b) { return __dsub_rn(a, b); }
+__device__ __forceinline__ double sub_exact(double a, double b) {
+    const int ha = __double2hiint(a), hb = __double2hiint(b);
+    const unsigned ma = (unsigned)ha & 0x7fffffffu, mb = (unsigned)hb & 0x7fffffffu;
+    const unsigned E = max(ma, mb) >> 20, F = min(ma, mb) >> 20;
+    if (E - 64u >= 2040u - 64u || F + 9u < E) return sub_fp64(a, b);
+    const unsigned long long A = (((unsigned long long)((ma & 0x000fffffu) | 0x00100000u) << 32) |
+                                  (unsigned)__double2loint(a)) << (9u - E + (ma >> 20));
+    const unsigned long long B = (((unsigned long long)((mb & 0x000fffffu) | 0x00100000u) << 32) |
+                                  (unsigned)__double2loint(b)) << (9u - E + (mb >> 20));
+    const unsigned long long sa = (unsigned long long)(long long)(ha >> 31), sb = (unsigned long long)(long long)(~hb >> 31);
+    return round_fixed((A ^ sa) + (B ^ sb) - sa - sb, (int)E + 2);
+}
+
+// Adds one site's raw sums to acc.  c: phi_n at the site, xm..zp: its neighbours in the order
+// -x, +x, -y, +y, -z, +z; p: pi_{n-1/2}, in the storage type.  Explicit round-to-nearest
+// operations keep the stand-alone and fused kernels bitwise equal; the half kick is the FP64 kick's
+// arithmetic.  Component by component, so that few widened values are live at once.  nb: the
+// neighbour sums, for the FP64 update that follows.  INTSUB: the differences in integers (the
+// multi-step kernel's FP64 instance, bound by latency, is 3 % faster with FP64 subtractions).
+template <typename R, int NC, bool INTSUB>
+__device__ __forceinline__ void energy_site(const R (&c)[NC], const R (&xm)[NC], const R (&xp)[NC], const R (&ym)[NC],
+                                            const R (&yp)[NC], const R (&zm)[NC], const R (&zp)[NC], const R (&p)[NC],
+                                            double (&nb)[NC], double (&acc)[kNs<NC>], const CoefE &k) {
+    double s2;
+    {
+        const double d = widen(c[0]);
+        s2 = __dmul_rn(d, d);
+    }
+#pragma unroll
+    for (int b = 1; b < NC; ++b) {
+        const double d = widen(c[b]);
+        s2 = __fma_rn(d, d, s2);
+    }
     const double gh = __fma_rn(k.hl, s2, k.hb0);
     const double w = __dsub_rn(s2, k.eta2);
+    acc[kPot] = __fma_rn(w, w, acc[kPot]);
 #pragma unroll
     for (int a = 0; a < NC; ++a) {
-        const double pin = __fma_rn(k.ah, nb[a], __fma_rn(-gh, c[a], p[a]));
+        nb[a] = neighbour_sum(xm[a], xp[a], ym[a], yp[a], zm[a], zp[a]);
+        const double d = widen(c[a]);
+        const double pin = __fma_rn(k.ah, nb[a], __fma_rn(-gh, d, widen(p[a])));
         acc[kKin] = __fma_rn(pin, pin, acc[kKin]);
-        const double ex = __dsub_rn(xp[a], c[a]), ey = __dsub_rn(yp[a], c[a]), ez = __dsub_rn(zp[a], c[a]);
+        const double ex = INTSUB ? sub_exact(xp[a], c[a]) : __dsub_rn(widen(xp[a]), d);
+        const double ey = INTSUB ? sub_exact(yp[a], c[a]) : __dsub_rn(widen(yp[a]), d);
+        const double ez = INTSUB ? sub_exact(zp[a], c[a]) : __dsub_rn(widen(zp[a]), d);
         acc[kGrad] = __fma_rn(ez, ez, __fma_rn(ey, ey, __fma_rn(ex, ex, acc[kGrad])));
-        acc[kSum + a] = __dadd_rn(acc[kSum + a], c[a]);
-        acc[kSum + NC + a] = __fma_rn(c[a], c[a], acc[kSum + NC + a]);
+        acc[kSum + a] = __dadd_rn(acc[kSum + a], d);
+        acc[kSum + NC + a] = __fma_rn(d, d, acc[kSum + NC + a]);
     }
-    acc[kPot] = __fma_rn(w, w, acc[kPot]);
 }
 
 // Block sum of acc, left in sh[j][0].  A pairwise tree whose additions at each level are packed
@@ -179,7 +280,7 @@ __device__ __forceinline__ Nbr neighbours(const SiteWalk &w, const Geom &g) {
 }
 
 template <typename R, int NC>
-__global__ void __launch_bounds__(kEnergyThreads) k_energy(const R *__restrict__ phi, const R *__restrict__ pi, Geom g,
+__global__ void __launch_bounds__(kEnergyThreads, kEnergyResident<NC>) k_energy(const R *__restrict__ phi, const R *__restrict__ pi, Geom g,
                                                            Stride3 d, CoefE k, double *__restrict__ scratch,
                                                            double *__restrict__ record) {
     __shared__ double sh[kNs<NC>][kEnergyThreads];
@@ -189,18 +290,17 @@ __global__ void __launch_bounds__(kEnergyThreads) k_energy(const R *__restrict__
     for (SiteWalk w((long long)blockIdx.x * blockDim.x + threadIdx.x, g); w.s < g.sites; w.advance(d, g)) {
         const Nbr n = neighbours(w, g);
         const long long s = w.s;
-        double c[NC], xm[NC], xp[NC], ym[NC], yp[NC], zm[NC], zp[NC], p[NC];
-        load_d<R, NC>(phi, s, g.sites, c);
-        load_d<R, NC>(phi, n.xm, g.sites, xm);
-        load_d<R, NC>(phi, n.xp, g.sites, xp);
-        load_d<R, NC>(phi, n.ym, g.sites, ym);
-        load_d<R, NC>(phi, n.yp, g.sites, yp);
-        load_d<R, NC>(phi, n.zm, g.sites, zm);
-        load_d<R, NC>(phi, n.zp, g.sites, zp);
-        load_d<R, NC>(pi, s, g.sites, p);
+        R c[NC], xm[NC], xp[NC], ym[NC], yp[NC], zm[NC], zp[NC], p[NC];
+        load_site<R, NC>(phi, s, g.sites, c);
+        load_site<R, NC>(phi, n.xm, g.sites, xm);
+        load_site<R, NC>(phi, n.xp, g.sites, xp);
+        load_site<R, NC>(phi, n.ym, g.sites, ym);
+        load_site<R, NC>(phi, n.yp, g.sites, yp);
+        load_site<R, NC>(phi, n.zm, g.sites, zm);
+        load_site<R, NC>(phi, n.zp, g.sites, zp);
+        load_site<R, NC>(pi, s, g.sites, p);
         double nb[NC];
-        neighbour_sums<NC>(xm, xp, ym, yp, zm, zp, nb);
-        energy_site<NC>(c, xp, yp, zp, nb, p, acc, k);
+        energy_site<R, NC, true>(c, xm, xp, ym, yp, zm, zp, p, nb, acc, k);
     }
     finish_energy<NC>(acc, sh, scratch, k, record);
 }
@@ -214,19 +314,18 @@ __device__ __forceinline__ void site_step_energy_f64(const double *__restrict__ 
     const Nbr n = neighbours(w, g);
     const long long s = w.s;
     double c[NC], xm[NC], xp[NC], ym[NC], yp[NC], zm[NC], zp[NC], p[NC], out[NC];
-    load_d<double, NC, COHERENT>(phi, s, g.sites, c);
-    load_d<double, NC, COHERENT>(phi, n.xm, g.sites, xm);
-    load_d<double, NC, COHERENT>(phi, n.xp, g.sites, xp);
-    load_d<double, NC, COHERENT>(phi, n.ym, g.sites, ym);
-    load_d<double, NC, COHERENT>(phi, n.yp, g.sites, yp);
-    load_d<double, NC, COHERENT>(phi, n.zm, g.sites, zm);
-    load_d<double, NC, COHERENT>(phi, n.zp, g.sites, zp);
+    load_site<double, NC, COHERENT>(phi, s, g.sites, c);
+    load_site<double, NC, COHERENT>(phi, n.xm, g.sites, xm);
+    load_site<double, NC, COHERENT>(phi, n.xp, g.sites, xp);
+    load_site<double, NC, COHERENT>(phi, n.ym, g.sites, ym);
+    load_site<double, NC, COHERENT>(phi, n.yp, g.sites, yp);
+    load_site<double, NC, COHERENT>(phi, n.zm, g.sites, zm);
+    load_site<double, NC, COHERENT>(phi, n.zp, g.sites, zp);
     const long long o = checked(s * NC, NC, g.sites * NC);
 #pragma unroll
     for (int a = 0; a < NC; ++a) p[a] = pi[o + a];
     double nb[NC];
-    neighbour_sums<NC>(xm, xp, ym, yp, zm, zp, nb);
-    energy_site<NC>(c, xp, yp, zp, nb, p, acc, ke);
+    energy_site<double, NC, !COHERENT>(c, xm, xp, ym, yp, zm, zp, p, nb, acc, ke);
     update_f64_nb<NC>(c, nb, p, out, k);
 #pragma unroll
     for (int a = 0; a < NC; ++a) {
@@ -261,21 +360,8 @@ __device__ __forceinline__ void site_step_energy_f32(const float *__restrict__ p
         p[a] = pi[o + a];
         cm[a] = KAHAN ? comp[o + a] : 0.0f;
     }
-    double dc[NC], dxm[NC], dxp[NC], dym[NC], dyp[NC], dzm[NC], dzp[NC], dp[NC];
-#pragma unroll
-    for (int a = 0; a < NC; ++a) {
-        dc[a] = widen(c[a]);
-        dxm[a] = widen(xm[a]);
-        dxp[a] = widen(xp[a]);
-        dym[a] = widen(ym[a]);
-        dyp[a] = widen(yp[a]);
-        dzm[a] = widen(zm[a]);
-        dzp[a] = widen(zp[a]);
-        dp[a] = widen(p[a]);
-    }
     double nb[NC];
-    neighbour_sums<NC>(dxm, dxp, dym, dyp, dzm, dzp, nb);
-    energy_site<NC>(dc, dxp, dyp, dzp, nb, dp, acc, ke);
+    energy_site<float, NC, true>(c, xm, xp, ym, yp, zm, zp, p, nb, acc, ke);
     update_f32<NC, KAHAN>(c, xm, xp, ym, yp, zm, zp, p, cm, out, k);
 #pragma unroll
     for (int a = 0; a < NC; ++a) {
@@ -287,7 +373,7 @@ __device__ __forceinline__ void site_step_energy_f32(const float *__restrict__ p
 
 // Fused step + energy, one step per launch.
 template <int NC>
-__global__ void __launch_bounds__(kEnergyThreads)
+__global__ void __launch_bounds__(kEnergyThreads, kEnergyResident<NC>)
     k_step_energy_f64(const double *__restrict__ phi, double *__restrict__ phi_out, double *__restrict__ pi, Geom g,
                       Stride3 d, Coef64 k, CoefE ke, double *__restrict__ scratch, double *__restrict__ record) {
     __shared__ double sh[kNs<NC>][kEnergyThreads];
@@ -300,7 +386,7 @@ __global__ void __launch_bounds__(kEnergyThreads)
 }
 
 template <int NC, bool KAHAN>
-__global__ void __launch_bounds__(kEnergyThreads)
+__global__ void __launch_bounds__(kEnergyThreads, NC <= 2 ? 4 : 2)
     k_step_energy_f32(const float *__restrict__ phi, float *__restrict__ phi_out, float *__restrict__ pi,
                       float *__restrict__ comp, Geom g, Stride3 d, Coef32 k, CoefE ke,
                       double *__restrict__ scratch, double *__restrict__ record) {
@@ -436,7 +522,7 @@ __device__ __forceinline__ void steps_energy_loop(R *phi_a, R *phi_b, Geom g, co
 }
 
 template <int NC>
-__global__ void __launch_bounds__(kEnergyThreads)
+__global__ void __launch_bounds__(kEnergyThreads, 2)
     k_steps_energy_f64(double *phi_a, double *phi_b, double *__restrict__ pi, Geom g, Stride3 d, Coef64 k, CoefE ke, int nsteps,
                        double *__restrict__ scratch, double *__restrict__ records, unsigned polls) {
     __shared__ double sh[kNs<NC>][kEnergyThreads];
@@ -447,7 +533,7 @@ __global__ void __launch_bounds__(kEnergyThreads)
 }
 
 template <int NC, bool KAHAN>
-__global__ void __launch_bounds__(kEnergyThreads)
+__global__ void __launch_bounds__(kEnergyThreads, 2)
     k_steps_energy_f32(float *phi_a, float *phi_b, float *__restrict__ pi, float *__restrict__ comp, Geom g, Stride3 d,
                        Coef32 k, CoefE ke, int nsteps, double *__restrict__ scratch, double *__restrict__ records,
                        unsigned polls) {

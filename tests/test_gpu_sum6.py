@@ -89,3 +89,35 @@ def test_infinities_and_nan_reach_the_result(lf2):
     assert np.array_equal(got[np.isinf(got)], want[np.isinf(want)])
     fine = np.isfinite(want)
     assert np.allclose(got[fine], want[fine], rtol=1e-14, atol=1e-13)
+
+
+@pytest.mark.parametrize("prec", ["f64", "f32k"])
+@pytest.mark.parametrize("kind", ["near", "spread", "ties"])
+def test_gradient_energy_differences_against_exact_rationals(lf2, kind, prec):
+    """The forward differences, subtracted as integers, at the edges of their fast ranges: exponents
+    7 to 11 (FP64) or 26 to 31 (FP32) binary orders apart, neighbours equal to the last bit, zeros.
+    Bound: each difference is rounded once (u), squared and added in FP64: a sum of N terms, added
+    in any order, is off by at most (N + 3) u of the sum of the (non-negative) terms."""
+    rng = np.random.default_rng(8)
+    n = SHAPE[::-1] + (1,)
+    v = rng.standard_normal(n)
+    if kind == "spread":
+        span = (7, 12) if prec == "f64" else (26, 32)
+        v = np.where(np.indices(n).sum(0) % 2 == 0, v, np.ldexp(v, -rng.integers(*span, n)))
+    elif kind == "ties":
+        v = np.where(rng.random(n) < 0.3, 0.0, 1.0) * (1.0 + 2.0 ** (-52 if prec == "f64" else -23) * rng.integers(-2, 3, n))
+    if prec != "f64":
+        v = v.astype(np.float32).astype(np.float64)
+    p = lf2.params(dx=1.0, dt=0.1, lam=0.0, eta=0.0, m2=0.0)
+    with lf2.System(SHAPE, 1, prec) as s:
+        s.upload(v, np.zeros_like(v))
+        e = lf2.lf2_energy(s.phi, s.pi, p, ncomp=1)
+    f = v[..., 0]
+    exact, terms = Fraction(0), 0
+    for ax in range(3):
+        up = np.roll(f, -1, ax)
+        for at in np.ndindex(f.shape):
+            exact += (Fraction(up[at]) - Fraction(f[at])) ** 2
+            terms += 1
+    got = 2 * Fraction(e["gradient"])
+    assert abs(got - exact) <= (terms + 3) * Fraction(1, 2 ** 53) * exact, float(abs(got - exact) / exact)
