@@ -470,7 +470,8 @@ lf2_status lf2_leapfrog_ex(lf2_field phi, lf2_field pi, const lf2_params *p, int
         const StepArgs a = step_args(phi, pi, p, p->dt, true);
         cudaError_t e = use_stream ? launch_stream_step(a, kernel == LF2_KERNEL_STREAM ? tile_y : 0,
                                                         kernel == LF2_KERNEL_STREAM ? zchunk : 0, 1, s)
-                                   : launch_site_step(a, s);
+                        : kernel == LF2_KERNEL_SITE ? launch_site_step(a, s)
+                                                    : launch_general_step(a, s);
         if (e != cudaSuccess) return cuda_fail(e, "leapfrog launch");
         phi->front = 1 - phi->front;
         return LF2_OK;

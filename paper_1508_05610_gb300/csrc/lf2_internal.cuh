@@ -23,6 +23,10 @@ struct StepArgs {
 
 cudaError_t launch_site_step(const StepArgs &a, cudaStream_t s);
 
+// One step (kick and drift) on any lattice shape: the column-walking kernel for real FP32 fields,
+// else the one-thread-per-site kernel.
+cudaError_t launch_general_step(const StepArgs &a, cudaStream_t s);
+
 // Streaming kernel (x-y tile, z-streaming); returns cudaErrorNotSupported when the shape
 // does not fit its constraints.
 bool stream_supported(const StepArgs &a, int tile_y, int zchunk);

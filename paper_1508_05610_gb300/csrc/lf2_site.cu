@@ -15,11 +15,75 @@ namespace {
 
 constexpr int kThreads = 256;
 
+// A site's NC components as accesses of the largest of 16, 8 and 4 bytes that divides them (field
+// buffers are 16-byte aligned): whole sites of 2, 4 and 6 FP32 or 2 FP64 components take one to
+// three vector accesses instead of one per component, each of which touched every line of the warp
+// (133x121x112 FP32+Kahan step, k_site: 4 components 55.9 -> 31.4 us, 6 components 112 -> 51 us).
+template <typename R, int BYTES>
+struct Chunk;
+template <>
+struct Chunk<float, 4> {
+    using T = float;
+};
+template <>
+struct Chunk<float, 8> {
+    using T = float2;
+};
+template <>
+struct Chunk<float, 16> {
+    using T = float4;
+};
+template <>
+struct Chunk<double, 8> {
+    using T = double;
+};
+template <>
+struct Chunk<double, 16> {
+    using T = double2;
+};
+template <typename R, int NC>
+struct SiteChunks {
+    static constexpr int BYTES = NC * (int)sizeof(R);
+    static constexpr int CH = BYTES % 16 == 0 ? 16 : (BYTES % 8 == 0 ? 8 : 4);
+    static constexpr int COUNT = BYTES / CH, E = CH / (int)sizeof(R);
+    using V = typename Chunk<R, CH>::T;
+};
+template <typename R, int NC>
+__device__ __forceinline__ void load_at(const R *__restrict__ p, R (&v)[NC]) {
+    using C = SiteChunks<R, NC>;
+#pragma unroll
+    for (int q = 0; q < C::COUNT; ++q) {
+        const typename C::V t = __ldg(reinterpret_cast<const typename C::V *>(p) + q);
+        memcpy(&v[q * C::E], &t, C::CH);
+    }
+}
+// Data the kernel also writes.  FP64 by L2 loads, which may be issued ahead of earlier stores (the
+// punned pointers lose __restrict__; 257x193x161 complex FP64: 1.96 against 1.46 times the start);
+// FP32 by plain ones, since the chunks of a site share L1 lines (5 components 1.7 against 1.55).
+template <typename R, int NC>
+__device__ __forceinline__ void load_own(const R *p, R (&v)[NC]) {
+    using C = SiteChunks<R, NC>;
+    const typename C::V *c = reinterpret_cast<const typename C::V *>(p);
+#pragma unroll
+    for (int q = 0; q < C::COUNT; ++q) {
+        const typename C::V t = sizeof(R) == 8 ? __ldcg(c + q) : c[q];
+        memcpy(&v[q * C::E], &t, C::CH);
+    }
+}
+template <typename R, int NC>
+__device__ __forceinline__ void store_own(R *p, const R (&v)[NC]) {
+    using C = SiteChunks<R, NC>;
+#pragma unroll
+    for (int q = 0; q < C::COUNT; ++q) {
+        typename C::V t;
+        memcpy(&t, &v[q * C::E], C::CH);
+        reinterpret_cast<typename C::V *>(p)[q] = t;
+    }
+}
+
 template <typename R, int NC>
 __device__ __forceinline__ void load_site(const R *__restrict__ f, long long s, long long sites, R (&v)[NC]) {
-    const long long i = checked(s * NC, NC, sites * NC);
-#pragma unroll
-    for (int a = 0; a < NC; ++a) v[a] = __ldg(f + i + a);
+    load_at<R, NC>(f + checked(s * NC, NC, sites * NC), v);
 }
 
 template <int NC>
@@ -40,14 +104,10 @@ __global__ void __launch_bounds__(kThreads) k_site_f64(const double *__restrict_
         load_site<double, NC>(phi, s + (wrap_up(y, g.ny) - y) * row, g.sites, yp);
         load_site<double, NC>(phi, s + (wrap_dn(z, g.nz) - z) * plane, g.sites, zm);
         load_site<double, NC>(phi, s + (wrap_up(z, g.nz) - z) * plane, g.sites, zp);
-#pragma unroll
-        for (int a = 0; a < NC; ++a) p[a] = pi[o + a];
+        load_own<double, NC>(pi + o, p);
         update_f64<NC>(c, xm, xp, ym, yp, zm, zp, p, out, k);
-#pragma unroll
-        for (int a = 0; a < NC; ++a) {
-            pi[o + a] = p[a];
-            if (drift) phi_out[o + a] = out[a];
-        }
+        store_own<double, NC>(pi + o, p);
+        if (drift) store_own<double, NC>(phi_out + o, out);
     }
 }
 
@@ -70,23 +130,55 @@ __global__ void __launch_bounds__(kThreads) k_site_f32(const float *__restrict__
         load_site<float, NC>(phi, s + (wrap_up(y, g.ny) - y) * row, g.sites, yp);
         load_site<float, NC>(phi, s + (wrap_dn(z, g.nz) - z) * plane, g.sites, zm);
         load_site<float, NC>(phi, s + (wrap_up(z, g.nz) - z) * plane, g.sites, zp);
-#pragma unroll
-        for (int a = 0; a < NC; ++a) p[a] = pi[o + a];
+        load_own<float, NC>(pi + o, p);
         if constexpr (MODE == 2) {
             kick_f32<NC>(c, xm, xp, ym, yp, zm, zp, p, k);
-#pragma unroll
-            for (int a = 0; a < NC; ++a) pi[o + a] = p[a];
+            store_own<float, NC>(pi + o, p);
         } else {
-#pragma unroll
-            for (int a = 0; a < NC; ++a) cm[a] = (MODE == 1) ? comp[o + a] : 0.0f;
+            if (MODE == 1) load_own<float, NC>(comp + o, cm);
             update_f32<NC, MODE == 1>(c, xm, xp, ym, yp, zm, zp, p, cm, out, k);
-#pragma unroll
-            for (int a = 0; a < NC; ++a) {
-                pi[o + a] = p[a];
-                phi_out[o + a] = out[a];
-                if (MODE == 1) comp[o + a] = cm[a];
-            }
+            store_own<float, NC>(pi + o, p);
+            store_own<float, NC>(phi_out + o, out);
+            if (MODE == 1) store_own<float, NC>(comp + o, cm);
         }
+    }
+}
+
+// One step of a real FP32 field on any lattice shape: a thread owns one (x, y) column of sites and
+// walks a chunk of z-planes with planes z-1, z, z+1 of its column in registers; the x and y
+// neighbours come from L1 and L2 (threads are numbered along the plane's rows, so a block's rows
+// overlap).  Against k_site it has no index arithmetic per site and loads each column once
+// instead of three times.  FP32+Kahan step, 133x121x112: k_site 12.8 us, k_march 10.7 (14.8 before
+// k_site's divisions went); 515x77x99: 21.6 and 17.9 us (27.2); 257x193x161: 47.6 and 46.7 (53.8).
+// With 2 or more components k_site is as fast or faster (its vector accesses are aligned along the
+// whole lattice), and in FP64 both wait for the FP64 pipe.
+constexpr int kMarchThreads = 512;
+constexpr int kMarchPlanes = 8;  // per chunk: two planes more to load than to compute; 4 to 32 within 5 %
+
+template <bool KAHAN>
+__global__ void __launch_bounds__(kMarchThreads) k_march(const float *__restrict__ phi, float *__restrict__ phi_out,
+                                                         float *__restrict__ pi, float *__restrict__ comp, Geom g,
+                                                         Coef32 k, int zchunk) {
+    const int plane = g.nx * g.ny;
+    const int i = blockIdx.x * kMarchThreads + threadIdx.x;
+    if (i >= plane) return;
+    const int y = i / g.nx, x = i - y * g.nx;
+    const int ixm = x == 0 ? i + g.nx - 1 : i - 1, ixp = x == g.nx - 1 ? i + 1 - g.nx : i + 1;
+    const int iym = y == 0 ? i + plane - g.nx : i - g.nx, iyp = y == g.ny - 1 ? x : i + g.nx;
+    const int z0 = blockIdx.y * zchunk, z1 = min(z0 + zchunk, g.nz);
+    auto load = [&](long long at) { return __ldg(phi + checked(at, 1, g.sites)); };
+    float below[1] = {load((long long)wrap_dn(z0, g.nz) * plane + i)}, cur[1] = {load((long long)z0 * plane + i)};
+    for (int z = z0; z < z1; ++z) {
+        const long long pz = (long long)z * plane, at = checked(pz + i, 1, g.sites);
+        float above[1] = {load((long long)wrap_up(z, g.nz) * plane + i)}, out[1];
+        float xm[1] = {load(pz + ixm)}, xp[1] = {load(pz + ixp)}, ym[1] = {load(pz + iym)}, yp[1] = {load(pz + iyp)};
+        float p[1] = {pi[at]}, cm[1] = {KAHAN ? comp[at] : 0.0f};
+        update_f32<1, KAHAN>(cur, xm, xp, ym, yp, below, above, p, cm, out, k);
+        pi[at] = p[0];
+        phi_out[at] = out[0];
+        if (KAHAN) comp[at] = cm[0];
+        below[0] = cur[0];
+        cur[0] = above[0];
     }
 }
 
@@ -143,6 +235,26 @@ cudaError_t launch_site_step(const StepArgs &a, cudaStream_t s) {
         case 6: site_launch<6>(a, grid, s); break;
         default: return cudaErrorInvalidValue;
     }
+    return cudaGetLastError();
+}
+
+cudaError_t launch_general_step(const StepArgs &a, cudaStream_t s) {
+    const long long plane = (long long)a.g.nx * a.g.ny, bx = (plane + kMarchThreads - 1) / kMarchThreads;
+    // chunks as long as they leave four blocks per SM, and 16-bit grid and 32-bit plane indices
+    int zchunk = kMarchPlanes;
+    while (zchunk > 1 && bx * ((a.g.nz + zchunk - 1) / zchunk) < 4LL * device_sm_count()) zchunk /= 2;
+    const long long bz = (a.g.nz + zchunk - 1) / zchunk;
+    if (a.g.sites == 0 || a.prec == LF2_F64 || a.ncomp != 1 || !a.drift || plane + kMarchThreads >= (1LL << 31) ||
+        bz > 65535)
+        return launch_site_step(a, s);
+    const dim3 grid((unsigned)bx, (unsigned)bz);
+    const Coef32 k = make_coef32(a.p, a.dt);
+    if (a.prec == LF2_F32_KAHAN)
+        k_march<true><<<grid, kMarchThreads, 0, s>>>((const float *)a.phi, (float *)a.phi_out, (float *)a.pi, a.comp,
+                                                     a.g, k, zchunk);
+    else
+        k_march<false><<<grid, kMarchThreads, 0, s>>>((const float *)a.phi, (float *)a.phi_out, (float *)a.pi, a.comp,
+                                                      a.g, k, zchunk);
     return cudaGetLastError();
 }
 

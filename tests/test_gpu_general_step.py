@@ -1,0 +1,44 @@
+"""GPU: the step that lattices take whose rows are no whole vectors, against the one-thread-per-site
+kernel (bitwise) and the FP64 oracle: every component count and precision, sides of 1, 2 and 3,
+planes smaller and larger than a block, z-chunks of one plane and with a remainder."""
+import numpy as np
+import pytest
+
+from paper_1508_05610_gb300 import inputs
+
+pytestmark = pytest.mark.gpu
+KW = dict(dx=0.9, dt=0.07, lam=1.3, eta=0.8, m2=0.1)
+
+
+@pytest.fixture(scope="module")
+def lf2():
+    import torch
+    if not torch.cuda.is_available():
+        pytest.skip("needs a GPU")
+    from paper_1508_05610_gb300 import build, lf2 as binding
+    build.build()
+    binding.load()
+    return binding
+
+
+@pytest.mark.parametrize("prec", ["f64", "f32k", "f32"])
+@pytest.mark.parametrize("shape,ncomp", [((1, 1, 1), 1), ((2, 1, 3), 1), ((3, 2, 1), 2), ((1, 5, 67), 1),
+                                         ((513, 1, 9), 1), ((33, 31, 19), 1), ((257, 21, 10), 1), ((33, 5, 7), 2),
+                                         ((17, 9, 5), 3), ((9, 7, 5), 4), ((19, 6, 5), 5), ((7, 9, 5), 6)])
+def test_default_step_equals_site_kernel_and_oracle(lf2, ora, monkeypatch, shape, ncomp, prec):
+    monkeypatch.setenv("LF2_TUNE", "off")
+    nx, ny, nz = shape
+    phi0 = inputs.gaussian_field(nx, ny, nz, ncomp, sigma=0.4, seed=901)
+    pi0 = inputs.gaussian_field(nx, ny, nz, ncomp, sigma=0.2, seed=902)
+    p = lf2.params(**KW)
+    with lf2.System(shape, ncomp, prec) as a, lf2.System(shape, ncomp, prec) as b:
+        for s in (a, b):
+            s.upload(phi0, pi0)
+        lf2.lf2_leapfrog(a.phi, a.pi, p, 5)
+        lf2.lf2_leapfrog_ex(b.phi, b.pi, p, 5, kernel=lf2.LF2_KERNEL_SITE)
+        got, ref = a.download(), b.download()
+    assert np.array_equal(got[0], ref[0]) and np.array_equal(got[1], ref[1])
+    ophi, opi = ora.evolve(phi0, pi0, 5, **KW)
+    tol = 1e-12 if prec == "f64" else 1e-5  # as in test_gpu_parity.py, there for 10 steps
+    assert np.max(np.abs(got[0] - ophi)) <= tol * np.max(np.abs(ophi))
+    assert np.max(np.abs(got[1] - opi)) <= tol * np.max(np.abs(opi))
