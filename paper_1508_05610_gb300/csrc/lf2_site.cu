@@ -261,134 +261,165 @@ cudaError_t launch_general_step(const StepArgs &a, cudaStream_t s) {
 // ------------------------------------------------------------ symmetric difference
 namespace {
 
+// Any row length: a thread per element of the grid stride, so that neighbouring threads read
+// neighbouring elements whatever the dimension.  g: the lattice in units of `inner` elements (1, and
+// the row nx * ncomp units with x-neighbours `dist` = ncomp units apart; for rows of 2^31 elements and
+// more in sites, with inner = ncomp and dist = 1); the coordinates advance by additions.  Bound by
+// latency: the loads of kDerivBatch<R> elements are issued together (one at a time kept 10 KB per SM
+// in flight, 1.5 TB/s): 257x193x161, the three dimensions, 3 components FP32 386 -> 231 us, FP64
+// (two elements; four leave small lattices with a ragged last round) 410 -> 347 us.
+template <typename R>
+constexpr int kDerivBatch = sizeof(R) == 8 ? 2 : 4;
+
 template <typename R>
 __global__ void __launch_bounds__(kThreads) k_derivative(const R *__restrict__ src, R *__restrict__ dst, Geom g,
-                                                         int ncomp, int dim, R inv2dx) {
-    // one thread per element (site, component): neighbouring threads read neighbouring
-    // elements, so every access is coalesced whatever the dimension
-    const long long n = g.sites * ncomp;
-    const long long stride = (long long)gridDim.x * blockDim.x;
-    for (long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x; e < n; e += stride) {
-        const long long s = e / ncomp;
-        const int a = (int)(e - s * ncomp);
-        const int x = (int)(s % g.nx);
-        const long long r = s / g.nx;
-        const int y = (int)(r % g.ny);
-        const int z = (int)(r / g.ny);
-        long long up, dn;
-        if (dim == 0) {
-            up = s - x + wrap_up(x, g.nx);
-            dn = s - x + wrap_dn(x, g.nx);
-        } else if (dim == 1) {
-            up = s + (long long)(wrap_up(y, g.ny) - y) * g.nx;
-            dn = s + (long long)(wrap_dn(y, g.ny) - y) * g.nx;
-        } else {
-            const long long plane = (long long)g.nx * g.ny;
-            up = s + (long long)(wrap_up(z, g.nz) - z) * plane;
-            dn = s + (long long)(wrap_dn(z, g.nz) - z) * plane;
+                                                         Stride3 d, int inner, int dist, int dim, R inv2dx) {
+    const long long row = g.nx, plane = row * g.ny;
+    SiteWalk w((long long)blockIdx.x * blockDim.x + threadIdx.x, g);
+    while (w.s < g.sites) {
+        const long long s0 = w.s;
+        long long up[kDerivBatch<R>], dn[kDerivBatch<R>];
+        int n = 0;
+#pragma unroll
+        for (int u = 0; u < kDerivBatch<R>; ++u) {
+            up[u] = dn[u] = s0;  // past the end: an element of the lattice, not used
+            if (w.s >= g.sites) continue;
+            if (dim == 0) {
+                up[u] = w.s + (w.x >= g.nx - dist ? dist - row : dist);
+                dn[u] = w.s + (w.x < dist ? row - dist : -dist);
+            } else if (dim == 1) {
+                up[u] = w.s + (wrap_up(w.y, g.ny) - w.y) * row;
+                dn[u] = w.s + (wrap_dn(w.y, g.ny) - w.y) * row;
+            } else {
+                up[u] = w.s + (wrap_up(w.z, g.nz) - w.z) * plane;
+                dn[u] = w.s + (wrap_dn(w.z, g.nz) - w.z) * plane;
+            }
+            ++n;
+            w.advance(d, g);
         }
-        dst[e] = (__ldg(src + up * ncomp + a) - __ldg(src + dn * ncomp + a)) * inv2dx;
+        for (int a = 0; a < inner; ++a) {
+            R hi[kDerivBatch<R>], lo[kDerivBatch<R>];
+#pragma unroll
+            for (int u = 0; u < kDerivBatch<R>; ++u) {
+                hi[u] = __ldg(src + up[u] * inner + a);
+                lo[u] = __ldg(src + dn[u] * inner + a);
+            }
+#pragma unroll
+            for (int u = 0; u < kDerivBatch<R>; ++u)
+                if (u < n) dst[(s0 + u * d.sites) * inner + a] = (hi[u] - lo[u]) * inv2dx;
+        }
     }
 }
 
-}  // namespace
+// Rows made of whole 16-byte vectors: a thread takes one vector (E elements) of kDerivRows rows of a
+// plane, all loads before the first use.  Bound: HBM, one read and one write of the field.  Along y
+// and z the two neighbours are vectors of other rows.  Along x they are NC elements away: within the
+// thread's vector or in the adjacent lane's (warp shuffle; the first lane of a warp and the last of
+// a row load theirs) for the component counts of at most E (DIM 0), single loads from L1 otherwise
+// (DIM 3).  256^3, the three dimensions together: 3 components FP32 390 -> 191 us (one, two, four
+// rows per thread: 195, 191, 201), 1 component 113 -> 70, 6 components 740 -> 368; FP64 is bound by
+// its subtraction and product on the FP64 pipe (3 components 662 -> 591).
+constexpr int kDerivRows = 2;
 
-namespace {
-
-// Row-vectorised symmetric difference for rows made of whole 16-byte vectors.  Blocks are
-// (x-chunk, y, z), so there is no division; each lane holds E = 16 / sizeof(R) elements of a
-// row.  Along y and z the two neighbours are whole-row vector loads.  Along x (template NC,
-// which must divide E) they are within the lane's vector or in the adjacent lane's (warp
-// shuffle); the first lane of a warp and the last lane of a row read the wrapped neighbour
-// from memory.
-template <typename R, int NC>
-__global__ void __launch_bounds__(128) k_derivative_rows(const R *__restrict__ src, R *__restrict__ dst, Geom g,
-                                                         int dim, R inv2dx) {
+template <typename R, int NC, int DIM>
+__global__ void __launch_bounds__(256) k_derivative_rows(const R *__restrict__ src, R *__restrict__ dst, Geom g,
+                                                         int ncomp, R inv2dx) {
     constexpr int E = 16 / sizeof(R);
-    static_assert(E % NC == 0, "components must divide the vector");
+    static_assert(NC <= E, "the x-neighbours of a vector lie in the vectors next to it");
     using V = typename std::conditional<sizeof(R) == 8, double2, float4>::type;
-    const long long rowE = (long long)g.nx * NC;
-    const int y = blockIdx.y, z = blockIdx.z;
+    const long long rowE = (long long)g.nx * ncomp, planeE = rowE * g.ny;
+    const int y0 = blockIdx.y * kDerivRows, z = blockIdx.z;
     const long long e0 = ((long long)blockIdx.x * blockDim.x + threadIdx.x) * E;
     const bool active = e0 < rowE;
-    const long long base = ((long long)z * g.ny + y) * rowE;
-    R up[E], dn[E];
-    if (dim == 0) {
-        R v[E];
-        V t{};
-        if (active) t = __ldg(reinterpret_cast<const V *>(src + base + e0));
-        memcpy(v, &t, 16);
-        R left[NC], right[NC];
-        const int lane = threadIdx.x & 31;
+    R up[kDerivRows][E], dn[kDerivRows][E];
 #pragma unroll
-        for (int a = 0; a < NC; ++a) {
-            left[a] = __shfl_up_sync(0xffffffffu, v[E - NC + a], 1);
-            right[a] = __shfl_down_sync(0xffffffffu, v[a], 1);
-        }
-        if (active && lane == 0) {
+    for (int r = 0; r < kDerivRows; ++r) {
+        const int y = y0 + r;
+        const bool on = active && y < g.ny;  // y is the same for the whole block
+        const long long base = (long long)z * planeE + (long long)y * rowE;
+        if constexpr (DIM == 0) {
+            R v[E];
+            V t{};
+            if (on) t = __ldg(reinterpret_cast<const V *>(src + base + e0));
+            memcpy(v, &t, 16);
+            R left[NC], right[NC];
+            const int lane = threadIdx.x & 31;
 #pragma unroll
             for (int a = 0; a < NC; ++a) {
-                long long e = e0 - NC + a;
-                if (e < 0) e += rowE;
-                left[a] = __ldg(src + base + e);
+                left[a] = __shfl_up_sync(0xffffffffu, v[E - NC + a], 1);
+                right[a] = __shfl_down_sync(0xffffffffu, v[a], 1);
             }
-        }
-        if (active && (lane == 31 || e0 + E >= rowE)) {
+            if (on && lane == 0) {
 #pragma unroll
-            for (int a = 0; a < NC; ++a) {
-                long long e = e0 + E + a;
-                if (e >= rowE) e -= rowE;
-                right[a] = __ldg(src + base + e);
+                for (int a = 0; a < NC; ++a) {
+                    const long long e = e0 - NC + a;
+                    left[a] = __ldg(src + base + (e < 0 ? e + rowE : e));
+                }
             }
-        }
+            if (on && (lane == 31 || e0 + E >= rowE)) {
 #pragma unroll
-        for (int j = 0; j < E; ++j) {
-            dn[j] = j < NC ? left[j] : v[j - NC];
-            up[j] = j + NC < E ? v[j + NC] : right[j + NC - E];
+                for (int a = 0; a < NC; ++a) {
+                    const long long e = e0 + E + a;
+                    right[a] = __ldg(src + base + (e >= rowE ? e - rowE : e));
+                }
+            }
+#pragma unroll
+            for (int j = 0; j < E; ++j) {
+                dn[r][j] = j < NC ? left[j] : v[j < NC ? 0 : j - NC];
+                up[r][j] = j + NC < E ? v[j + NC < E ? j + NC : 0] : right[j + NC < E ? 0 : j + NC - E];
+            }
+        } else if constexpr (DIM == 3) {
+#pragma unroll
+            for (int j = 0; j < E; ++j) {
+                const long long u = e0 + j + ncomp, d = e0 + j - ncomp;
+                up[r][j] = on ? __ldg(src + base + (u >= rowE ? u - rowE : u)) : R(0);
+                dn[r][j] = on ? __ldg(src + base + (d < 0 ? d + rowE : d)) : R(0);
+            }
+        } else if (on) {
+            const long long du = DIM == 1 ? (long long)(wrap_up(y, g.ny) - y) * rowE : (long long)(wrap_up(z, g.nz) - z) * planeE;
+            const long long dd = DIM == 1 ? (long long)(wrap_dn(y, g.ny) - y) * rowE : (long long)(wrap_dn(z, g.nz) - z) * planeE;
+            const V a = __ldg(reinterpret_cast<const V *>(src + base + du + e0));
+            const V b = __ldg(reinterpret_cast<const V *>(src + base + dd + e0));
+            memcpy(up[r], &a, 16);
+            memcpy(dn[r], &b, 16);
         }
-    } else {
-        if (!active) return;
-        long long du, dd;
-        if (dim == 1) {
-            du = (long long)(wrap_up(y, g.ny) - y) * rowE;
-            dd = (long long)(wrap_dn(y, g.ny) - y) * rowE;
-        } else {
-            const long long plane = rowE * g.ny;
-            du = (long long)(wrap_up(z, g.nz) - z) * plane;
-            dd = (long long)(wrap_dn(z, g.nz) - z) * plane;
-        }
-        V a = __ldg(reinterpret_cast<const V *>(src + base + du + e0));
-        V b = __ldg(reinterpret_cast<const V *>(src + base + dd + e0));
-        memcpy(up, &a, 16);
-        memcpy(dn, &b, 16);
     }
-    if (!active) return;
-    R out[E];
 #pragma unroll
-    for (int j = 0; j < E; ++j) out[j] = (up[j] - dn[j]) * inv2dx;
-    V o;
-    memcpy(&o, out, 16);
-    __stcs(reinterpret_cast<V *>(dst + base + e0), o);
+    for (int r = 0; r < kDerivRows; ++r) {
+        if (!active || y0 + r >= g.ny) continue;
+        R out[E];
+#pragma unroll
+        for (int j = 0; j < E; ++j) out[j] = (up[r][j] - dn[r][j]) * inv2dx;
+        V o;
+        memcpy(&o, out, 16);
+        __stcs(reinterpret_cast<V *>(dst + (long long)z * planeE + (long long)(y0 + r) * rowE + e0), o);
+    }
 }
 
 template <typename R>
 cudaError_t launch_rows(const void *src, void *dst, const Geom &g, int ncomp, int dim, R inv2dx, cudaStream_t s) {
-    const long long vecs = (long long)g.nx * ncomp * sizeof(R) / 16;
-    dim3 grid((unsigned)((vecs + 127) / 128), g.ny, g.nz);
-    // along y and z the component count does not matter (whole rows): use the NC = 1 instance
-    const int nc = dim == 0 ? ncomp : 1;
-    const Geom gg = dim == 0 ? g : Geom{g.nx * ncomp, g.ny, g.nz, g.sites * ncomp};
-    switch (nc) {
-        case 1: k_derivative_rows<R, 1><<<grid, 128, 0, s>>>((const R *)src, (R *)dst, gg, dim, inv2dx); break;
-        case 2: k_derivative_rows<R, 2><<<grid, 128, 0, s>>>((const R *)src, (R *)dst, gg, dim, inv2dx); break;
-        case 4:
-            if constexpr (sizeof(R) == 4) {
-                k_derivative_rows<R, 4><<<grid, 128, 0, s>>>((const R *)src, (R *)dst, gg, dim, inv2dx);
-                break;
-            }
-            return cudaErrorNotSupported;
-        default: return cudaErrorNotSupported;
-    }
+    constexpr int E = 16 / (int)sizeof(R);
+    const long long vecs = (long long)g.nx * ncomp / E;
+    // whole warps of about equal blocks along a row, at most 256 threads (192 vectors: 192 threads)
+    const long long nb = (vecs + 255) / 256;
+    const int threads = (int)(((vecs + nb - 1) / nb + 31) / 32 * 32);
+    const dim3 grid((unsigned)((vecs + threads - 1) / threads), (unsigned)((g.ny + kDerivRows - 1) / kDerivRows), g.nz);
+    const R *a = (const R *)src;
+    R *d = (R *)dst;
+    if (dim == 1)
+        k_derivative_rows<R, 1, 1><<<grid, threads, 0, s>>>(a, d, g, ncomp, inv2dx);
+    else if (dim == 2)
+        k_derivative_rows<R, 1, 2><<<grid, threads, 0, s>>>(a, d, g, ncomp, inv2dx);
+    else if (ncomp == 1)
+        k_derivative_rows<R, 1, 0><<<grid, threads, 0, s>>>(a, d, g, ncomp, inv2dx);
+    else if (ncomp == 2)
+        k_derivative_rows<R, 2, 0><<<grid, threads, 0, s>>>(a, d, g, ncomp, inv2dx);
+    else if (ncomp == 3 && E >= 3)
+        k_derivative_rows<R, E < 3 ? 1 : 3, 0><<<grid, threads, 0, s>>>(a, d, g, ncomp, inv2dx);
+    else if (ncomp == 4 && E >= 4)
+        k_derivative_rows<R, E < 4 ? 1 : 4, 0><<<grid, threads, 0, s>>>(a, d, g, ncomp, inv2dx);
+    else
+        k_derivative_rows<R, 1, 3><<<grid, threads, 0, s>>>(a, d, g, ncomp, inv2dx);
     return cudaGetLastError();
 }
 
@@ -398,18 +429,21 @@ cudaError_t launch_derivative(const void *src, void *dst, const Geom &g, int nco
                               double dx, cudaStream_t s) {
     if (g.sites == 0) return cudaSuccess;
     const int esz = prec == LF2_F64 ? 8 : 4;
-    const int E = 16 / esz;
     const bool rows_ok = ((long long)g.nx * ncomp * esz) % 16 == 0 && ((uintptr_t)src | (uintptr_t)dst) % 16 == 0 &&
-                         g.ny <= 65535 && g.nz <= 65535 && (dim != 0 || (ncomp <= E && E % ncomp == 0));
+                         g.ny <= 65535 && g.nz <= 65535;
     if (rows_ok) {
         return prec == LF2_F64 ? launch_rows<double>(src, dst, g, ncomp, dim, 0.5 / dx, s)
                                : launch_rows<float>(src, dst, g, ncomp, dim, (float)(0.5 / dx), s);
     }
-    const int grid = grid_for(g.sites * ncomp);
+    const bool elements = (long long)g.nx * ncomp < (1LL << 31);
+    const int inner = elements ? 1 : ncomp, dist = elements ? ncomp : 1;
+    const Geom u = elements ? Geom{g.nx * ncomp, g.ny, g.nz, g.sites * ncomp} : g;
+    const int grid = grid_for(u.sites);
+    const Stride3 d = make_stride3((long long)grid * kThreads, u);
     if (prec == LF2_F64)
-        k_derivative<double><<<grid, kThreads, 0, s>>>((const double *)src, (double *)dst, g, ncomp, dim, 0.5 / dx);
+        k_derivative<double><<<grid, kThreads, 0, s>>>((const double *)src, (double *)dst, u, d, inner, dist, dim, 0.5 / dx);
     else
-        k_derivative<float><<<grid, kThreads, 0, s>>>((const float *)src, (float *)dst, g, ncomp, dim,
+        k_derivative<float><<<grid, kThreads, 0, s>>>((const float *)src, (float *)dst, u, d, inner, dist, dim,
                                                       (float)(0.5 / dx));
     return cudaGetLastError();
 }

@@ -42,3 +42,23 @@ def test_default_step_equals_site_kernel_and_oracle(lf2, ora, monkeypatch, shape
     tol = 1e-12 if prec == "f64" else 1e-5  # as in test_gpu_parity.py, there for 10 steps
     assert np.max(np.abs(got[0] - ophi)) <= tol * np.max(np.abs(ophi))
     assert np.max(np.abs(got[1] - opi)) <= tol * np.max(np.abs(opi))
+
+
+@pytest.mark.parametrize("prec", ["f64", "f32"])
+@pytest.mark.parametrize("ncomp", [1, 2, 3, 4, 5, 6])
+@pytest.mark.parametrize("shape", [(1, 1, 1), (2, 3, 1), (7, 5, 3), (4, 3, 2), (12, 7, 5), (132, 3, 4), (260, 5, 2),
+                                   (1028, 3, 2), (515, 2, 3)])
+def test_derivative_of_every_row_length(lf2, shape, ncomp, prec):
+    """(phi(x+i) - phi(x-i)) * (1 / (2 dx)) in the storage type, exactly: rows shorter than a vector,
+    of whole vectors and not, within one block and over several, an odd number of rows."""
+    nx, ny, nz = shape
+    dtype = np.float64 if prec == "f64" else np.float32
+    v = inputs.gaussian_field(nx, ny, nz, ncomp, sigma=1.0, seed=903).astype(dtype)
+    inv = dtype(0.5 / 0.7)
+    with lf2.System(shape, ncomp, prec) as s:
+        lf2.lf2_field_upload(s.phi, v.astype(np.float64))
+        for dim in range(3):
+            lf2.lf2_field_derivative(s.phi, s.pi, dim, 0.7)
+            want = (np.roll(v, -1, 2 - dim) - np.roll(v, 1, 2 - dim)) * inv
+            got = lf2.lf2_field_download(s.pi, s.host_shape)
+            assert np.array_equal(got, want.astype(np.float64)), dim
