@@ -51,26 +51,6 @@ __device__ __forceinline__ R ld_field(const R *p) {
         return __ldg(p);
 }
 
-// Exact FP32 -> FP64 widening on the integer pipe, without a branch.  This GPU converts on its
-// FP64 pipe, which the FP64 sums already keep busy: the 8 conversions per component-site of
-// FP32 storage made the FP64 energy of FP32 data 1.4x slower than that of FP64 data.  Widening
-// re-biases the exponent (bias 127 -> 1023) and moves the 23-bit significand to the top of the
-// 52-bit one.  A subnormal (leading bit n places below the implicit one) is first shifted up by
-// n and its exponent lowered by n; infinities and NaN keep the all-ones exponent, a NaN comes
-// back quiet with its payload; a signed zero keeps only its sign.  The result is the one exact
-// double (IEEE 754 widening), so FP64 and FP32 storage of the same values give the same sums.
-__device__ __forceinline__ double widen(double v) { return v; }
-__device__ __forceinline__ double widen(float v) {
-    const unsigned u = __float_as_uint(v), mag = u & 0x7fffffffu;
-    const int n = max(__clz(mag) - 8, 0);  // 0 for normal numbers, infinities and NaN
-    const unsigned m = mag << n;
-    unsigned hi = (m >> 3) + ((896u - (unsigned)n) << 20);
-    hi += mag >= 0x7f800000u ? 896u << 20 : 0u;
-    hi |= mag > 0x7f800000u ? 1u << 19 : 0u;
-    hi = (mag ? hi : 0u) | (u & 0x80000000u);
-    return __hiloint2double((int)hi, (int)(m << 29));
-}
-
 template <typename R, int NC, bool COHERENT = false>
 __device__ __forceinline__ void load_site(const R *__restrict__ f, long long s, long long sites, R (&v)[NC]) {
     const long long i = checked(s * NC, NC, sites * NC);

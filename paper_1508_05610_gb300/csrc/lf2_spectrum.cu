@@ -29,53 +29,123 @@ __global__ void k_extract(const R *__restrict__ f, R *__restrict__ out, long lon
         out[s] = f[s * ncomp + comp];
 }
 
-__device__ __forceinline__ int isqrt_exact(long long s) {
-    long long b = (long long)sqrt((double)s);
-    while (b * b > s) --b;
-    while ((b + 1) * (b + 1) <= s) ++b;
-    return (int)b;
+// The largest x >= 0 with x^2 <= v, exactly.
+__device__ __forceinline__ int floor_sqrt(long long v) {
+    long long x = (long long)sqrtf((float)v);
+    while (x * x > v) --x;
+    while ((x + 1) * (x + 1) <= v) ++x;
+    return (int)x;
 }
 
+__device__ __forceinline__ void add_mode(double2 c, double &acc) { acc = __fma_rn(c.y, c.y, __fma_rn(c.x, c.x, acc)); }
+__device__ __forceinline__ void add_mode(float2 c, double &acc) {
+    const double re = widen(c.x), im = widen(c.y);
+    acc = __fma_rn(im, im, __fma_rn(re, re, acc));
+}
+
+// Sums of the modes of each shell.  The rows (ky, kz), (+-ky, +-kz) and with ky and kz exchanged, up
+// to eight, have the same |k| at every kx, so a warp adds the modes of all of them, lane for kx,
+// before it looks at shells: one square root and one shell per eight modes, and eight independent
+// coalesced loads in flight.  Along kx the shells are runs of neighbouring lanes, which are summed
+// by shuffles, so that the block's histogram in shared memory gets one addition per shell and warp.
+// 256^3 FP32: 75 us, against 438 us with an atomic for each of power, |k| and count per mode.
+// Bound: the FP64 pipe (two products per mode, then the square roots).
 // add_power: add this component's power to the rows a previous component's binning wrote,
 // leaving the |k| sums and mode counts (the same for every component) as they are.
 template <typename C>
 __global__ void __launch_bounds__(kBinThreads) k_bin(const C *__restrict__ spec, int n, int nbins, double kunit,
                                                      double inv_volume, double *__restrict__ partials, int add_power) {
-    extern __shared__ double hist[];  // 3 * nbins: power, |k| sum, count
-    for (int i = threadIdx.x; i < 3 * nbins; i += blockDim.x) hist[i] = 0.0;
+    extern __shared__ double hist[];  // nbins powers, nbins |k| sums, nbins counts (64-bit integers)
+    unsigned long long *cnt = reinterpret_cast<unsigned long long *>(hist + 2 * nbins);
+    for (int i = threadIdx.x; i < 2 * nbins; i += kBinThreads) hist[i] = 0.0;
+    for (int i = threadIdx.x; i < nbins; i += kBinThreads) cnt[i] = 0ull;
     __syncthreads();
-    const int hx = n / 2 + 1;
-    const long long total = (long long)n * n * hx;
-    for (long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x; e < total; e += (long long)gridDim.x * blockDim.x) {
-        const int kx = (int)(e % hx);
-        const long long r = e / hx;
-        const int ky = (int)(r % n);
-        const int kz = (int)(r / n);
-        const int mx = kx, my = ky <= n / 2 ? ky : ky - n, mz = kz <= n / 2 ? kz : kz - n;
-        const long long s2 = (long long)mx * mx + (long long)my * my + (long long)mz * mz;
-        const int b = isqrt_exact(s2);
-        if (b >= nbins) continue;
-        const double w = (kx == 0 || (n % 2 == 0 && kx == n / 2)) ? 1.0 : 2.0;
-        const double re = (double)spec[e].x, im = (double)spec[e].y;
-        atomicAdd(&hist[b], w * (re * re + im * im) * inv_volume);
-        atomicAdd(&hist[nbins + b], w * kunit * sqrt((double)s2));
-        atomicAdd(&hist[2 * nbins + b], w);
+    const int hx = n / 2 + 1, half = n / 2, lane = threadIdx.x & 31;
+    const bool even = n % 2 == 0;
+    auto self = [&](int k) { return k == 0 || (even && k == half); };  // its own mirror image
+    const long long pairs = (long long)hx * (hx + 1) / 2;  // 0 <= ky <= kz <= half
+    const int segs = (hx + 31) / 32;
+    const long long items = pairs * segs;
+    const long long warp0 = ((long long)blockIdx.x * kBinThreads + threadIdx.x) / 32;
+    for (long long it = warp0; it < items; it += (long long)gridDim.x * (kBinThreads / 32)) {
+        const long long p = it / segs;
+        const int x = (int)(it - p * segs) * 32 + lane;
+        // p = kz (kz + 1) / 2 + ky
+        int kz = (floor_sqrt(8 * p + 1) - 1) / 2;
+        const int ky = (int)(p - (long long)kz * (kz + 1) / 2);
+        const long long q = (long long)ky * ky + (long long)kz * kz;
+        if (floor_sqrt(q) >= nbins) continue;  // the whole row lies beyond the shells asked for
+        C v[8];
+        bool have[8];
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+            have[j] = !((j & 1) && self(ky)) && !((j & 2) && self(kz)) && !((j & 4) && ky == kz);
+            const int a = (j & 1) ? n - ky : ky, b = (j & 2) ? n - kz : kz;
+            const long long row = (j & 4) ? (long long)a * n + b : (long long)b * n + a;
+            if (have[j] && x < hx) v[j] = __ldg(spec + row * hx + x);
+        }
+        const long long s2 = q + (long long)x * x;
+        const int shell = x < hx ? floor_sqrt(s2) : 0x7fffffff;
+        const bool in = shell < nbins;
+        double power = 0.0, ksum = 0.0;
+        int images = 0;
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+            if (!have[j]) continue;  // the same for the whole warp
+            ++images;
+            if (in) add_mode(v[j], power);
+        }
+        unsigned count = 0u;
+        if (in) {
+            const int w = self(x) ? 1 : 2;  // kx and -kx
+            power *= (double)w;
+            count = (unsigned)(w * images);
+            if (!add_power) ksum = (double)count * sqrt((double)s2);
+        }
+        // sums over runs of equal shells, left in the run's first lane
+        for (int off = 1; off < 32; off *= 2) {
+            const int other = __shfl_down_sync(0xffffffffu, shell, off);
+            const bool same = lane + off < 32 && other == shell;
+            if (!__any_sync(0xffffffffu, same)) break;  // no run is longer
+            const double dp = __shfl_down_sync(0xffffffffu, power, off), dk = __shfl_down_sync(0xffffffffu, ksum, off);
+            const unsigned dc = __shfl_down_sync(0xffffffffu, count, off);
+            if (same) {
+                power += dp;
+                ksum += dk;
+                count += dc;
+            }
+        }
+        const int before = __shfl_up_sync(0xffffffffu, shell, 1);
+        if (in && (lane == 0 || before != shell)) {
+            atomicAdd(&hist[shell], power);
+            if (!add_power) {
+                atomicAdd(&hist[nbins + shell], ksum);
+                atomicAdd(&cnt[shell], (unsigned long long)count);
+            }
+        }
     }
     __syncthreads();
-    double *row = partials + (size_t)blockIdx.x * 3 * nbins;
-    if (add_power) {
-        for (int i = threadIdx.x; i < nbins; i += blockDim.x) row[i] += hist[i];
-    } else {
-        for (int i = threadIdx.x; i < 3 * nbins; i += blockDim.x) row[i] = hist[i];
+    double *out = partials + (size_t)blockIdx.x * 3 * nbins;
+    for (int i = threadIdx.x; i < nbins; i += kBinThreads) {
+        if (add_power) {
+            out[i] += hist[i] * inv_volume;
+        } else {
+            out[i] = hist[i] * inv_volume;
+            out[nbins + i] = hist[nbins + i] * kunit;
+            out[2 * nbins + i] = (double)cnt[i];
+        }
     }
 }
 
-__global__ void k_bin_final(const double *__restrict__ partials, int nblocks, int nbins, double *__restrict__ out) {
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < 3 * nbins; i += gridDim.x * blockDim.x) {
-        double s = 0.0;
-        for (int b = 0; b < nblocks; ++b) s += partials[(size_t)b * 3 * nbins + i];
-        out[i] = s;
-    }
+// A warp per sum over the blocks' rows: lanes in steps of 32 rows, then pairwise (a fixed order).
+__global__ void __launch_bounds__(kBinThreads) k_bin_final(const double *__restrict__ partials, int nblocks, int nbins,
+                                                           double *__restrict__ out) {
+    const int i = (blockIdx.x * kBinThreads + threadIdx.x) / 32, lane = threadIdx.x % 32;
+    if (i >= 3 * nbins) return;
+    double s = 0.0;
+    for (int b = lane; b < nblocks; b += 32) s += partials[(size_t)b * 3 * nbins + i];
+    for (int w = 16; w > 0; w >>= 1) s += __shfl_down_sync(0xffffffffu, s, w);
+    if (lane == 0) out[i] = s;
 }
 
 }  // namespace
@@ -100,7 +170,7 @@ extern "C" lf2_status lf2_power_spectrum(lf2_field f, int comp, int nbins, doubl
     cufftHandle plan = 0;
     bool have_plan = false;
     lf2_status st = LF2_OK;
-    const int kBinBlocks = 2 * device_sm_count();  // two histogram blocks per SM
+    const int kBinBlocks = 4 * device_sm_count();  // four histogram blocks per SM
     cudaError_t e = cudaMalloc(&real, (size_t)sites * rsz);
     if (e == cudaSuccess) e = cudaMalloc(&spec, (size_t)n * n * (n / 2 + 1) * csz);
     if (e == cudaSuccess) e = cudaMalloc(&partials, (size_t)kBinBlocks * 3 * nbins * sizeof(double));
@@ -137,16 +207,14 @@ extern "C" lf2_status lf2_power_spectrum(lf2_field f, int comp, int nbins, doubl
         }
         const int add = c > c0;
         if (dbl)
-            k_bin<double2><<<kBinBlocks, kBinThreads, smem, s>>>((const double2 *)spec, n, nbins, kunit, inv_volume, partials,
-                                                                 add);
+            k_bin<double2><<<kBinBlocks, kBinThreads, smem, s>>>((const double2 *)spec, n, nbins, kunit, inv_volume, partials, add);
         else
-            k_bin<float2><<<kBinBlocks, kBinThreads, smem, s>>>((const float2 *)spec, n, nbins, kunit, inv_volume, partials,
-                                                                add);
+            k_bin<float2><<<kBinBlocks, kBinThreads, smem, s>>>((const float2 *)spec, n, nbins, kunit, inv_volume, partials, add);
         e = cudaGetLastError();
         if (e != cudaSuccess) st = cuda_error(e, "binning");
     }
     if (st == LF2_OK) {
-        k_bin_final<<<(3 * nbins + 255) / 256, 256, 0, s>>>(partials, kBinBlocks, nbins, out);
+        k_bin_final<<<(3 * nbins * 32 + kBinThreads - 1) / kBinThreads, kBinThreads, 0, s>>>(partials, kBinBlocks, nbins, out);
         e = cudaGetLastError();
         if (e == cudaSuccess) e = cudaMemcpyAsync(power, out, nbins * sizeof(double), cudaMemcpyDeviceToHost, s);
         if (e == cudaSuccess) e = cudaMemcpyAsync(kmean, out + nbins, nbins * sizeof(double), cudaMemcpyDeviceToHost, s);

@@ -74,3 +74,27 @@ def test_grf_initial_condition_has_the_requested_spectrum(lf2):
     assert P[0] < 1e-20 * np.max(P[inside])  # the k = 0 mode is removed
     del phi
     torch.cuda.empty_cache()
+
+
+@pytest.mark.parametrize("n", [1, 2, 3, 31, 33, 64])
+@pytest.mark.parametrize("nbins", [1, 9, 1024])
+def test_spectrum_at_edges_of_rows_and_shells(lf2, n, nbins):
+    """Rows of less than, about and more than a warp of modes, odd and even sides (self-mirrored
+    planes), fewer and more shells than the lattice has: mode counts exactly, power and |k| to 1e-12
+    of numpy's FFT of the same FP64 values (the transform errs by some ten units of 1e-16)."""
+    phi = inputs.gaussian_field(n, n, n, 1, sigma=1.0, seed=142)
+    with lf2.System((n, n, n), 1, "f64") as s:
+        lf2.lf2_field_upload(s.phi, phi)
+        P, K, C = lf2.lf2_power_spectrum(s.phi, comp=0, nbins=nbins, dx=0.8)
+    m = np.rint(np.fft.fftfreq(n) * n).astype(np.int64)
+    m2 = m[:, None, None] ** 2 + m[None, :, None] ** 2 + m[None, None, :] ** 2
+    shell = np.array([math.isqrt(int(v)) for v in m2.ravel()])
+    keep = shell < nbins
+    count = np.bincount(shell[keep], minlength=nbins).astype(float)
+    power = np.abs(np.fft.fftn(phi[..., 0])).ravel() ** 2 / n ** 3
+    some = np.maximum(count, 1)
+    want = np.bincount(shell[keep], weights=power[keep], minlength=nbins) / some
+    k = np.bincount(shell[keep], weights=np.sqrt(m2.ravel()[keep].astype(float)), minlength=nbins) / some
+    assert np.array_equal(C, count)
+    assert np.max(np.abs(P - want)) <= 1e-12 * np.max(want)
+    assert np.max(np.abs(K - k * 2 * math.pi / (n * 0.8))) <= 1e-12 * max(np.max(K), 1e-300)
