@@ -196,8 +196,8 @@ lf2_status lf2_field_derivative(lf2_field src, lf2_field dst, int dim, double dx
  * / N^3, since the cross terms cancel between k and -k).  Mode (m_x, m_y, m_z) (signed integer frequencies)
  * belongs to shell b = floor(sqrt(m_x^2 + m_y^2 + m_z^2)); shells b < nbins (<= 1024) are
  * returned as host arrays of nbins doubles: mean power, mean |k|, mode count.  The transform is
- * cuFFT (single or double precision after the storage type); buffers and the plan are
- * allocated per call.  LF2_ERR_UNSUPPORTED for non-cubic lattices.  Synchronises `stream`. */
+ * cuFFT (single or double precision after the storage type); buffers are allocated per call, plans
+ * (without work areas, at most two idle ones) are kept by the lattice until it is destroyed.  LF2_ERR_UNSUPPORTED for non-cubic lattices.  Synchronises `stream`. */
 lf2_status lf2_power_spectrum(lf2_field f, int comp, int nbins, double dx, double *power, double *kmean,
                               double *count, void *stream);
 

@@ -240,6 +240,7 @@ lf2_status lf2_lattice_create(int dim, const int *sizes, int halo, lf2_lattice *
 lf2_status lf2_lattice_destroy(lf2_lattice lat) {
     if (!lat) return fail(LF2_ERR_INVALID, "lattice is NULL");
     if (lat->users.load() != 0) return fail(LF2_ERR_STATE, "lattice still used by %d field(s)", lat->users.load());
+    release_fft_plans(lat);
     delete lat;
     return LF2_OK;
 }

@@ -3,9 +3,19 @@
 #pragma once
 
 #include <atomic>
+#include <mutex>
 #include <string>
+#include <vector>
 
 #include "lf2_internal.cuh"
+
+// A cuFFT plan of a lattice without its work area (lf2_spectrum.cu).
+struct FftPlan {
+    int device;
+    bool dbl;
+    int handle;        // cufftHandle
+    size_t work_bytes;
+};
 
 struct lf2_lattice_s {
     int dim;
@@ -13,6 +23,10 @@ struct lf2_lattice_s {
     int halo;
     long long sites;
     std::atomic<int> users{0};  // fields and ensembles still attached
+    // FFT plans not in use, at most kIdleFftPlans: a call takes one out (or makes one) and gives it
+    // back when its stream is done, so threads never share a plan; destroyed with the lattice
+    std::mutex fft_mu;
+    std::vector<FftPlan> fft_idle;
 };
 
 struct lf2_field_s {
@@ -52,6 +66,9 @@ TbArgs tb_args(lf2_field phi, lf2_field pi, const lf2_params *p);
 
 // Tuned kernel plan for a lattice shape (filled by lf2_tune); false if none.
 bool plan_lookup(const int n[3], int ncomp, lf2_precision prec, lf2_step_config *out);
+
+// Destroys the lattice's idle FFT plans (lf2_spectrum.cu).
+void release_fft_plans(lf2_lattice lat);
 
 inline Geom geom_of(const lf2_lattice_s *lat) { return Geom{lat->n[0], lat->n[1], lat->n[2], lat->sites}; }
 

@@ -13,6 +13,9 @@
 #include <cufft.h>
 
 #include <cmath>
+#include <cstring>
+#include <new>
+#include <vector>
 
 #include "lf2_handles.h"
 
@@ -148,7 +151,61 @@ __global__ void __launch_bounds__(kBinThreads) k_bin_final(const double *__restr
     if (lane == 0) out[i] = s;
 }
 
+// The lattice keeps its plans: making one took over half of a 256^3 call.
+constexpr size_t kIdleFftPlans = 2;
+
+lf2_status take_plan(lf2_lattice lat, bool dbl, FftPlan *out) {
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return cuda_error(e, "cudaGetDevice");
+    {
+        std::lock_guard<std::mutex> lock(lat->fft_mu);
+        for (size_t i = 0; i < lat->fft_idle.size(); ++i) {
+            if (lat->fft_idle[i].device != dev || lat->fft_idle[i].dbl != dbl) continue;
+            *out = lat->fft_idle[i];
+            lat->fft_idle.erase(lat->fft_idle.begin() + i);
+            return LF2_OK;
+        }
+    }
+    const int n = lat->n[0];
+    cufftHandle h = 0;
+    size_t work = 0;
+    cufftResult r = cufftCreate(&h);
+    if (r != CUFFT_SUCCESS)
+        return set_error(r == CUFFT_ALLOC_FAILED ? LF2_ERR_NOMEM : LF2_ERR_CUDA, "cuFFT error %d", (int)r);
+    r = cufftSetAutoAllocation(h, 0);
+    if (r == CUFFT_SUCCESS) r = cufftMakePlan3d(h, n, n, n, dbl ? CUFFT_D2Z : CUFFT_R2C, &work);
+    if (r != CUFFT_SUCCESS) {
+        cufftDestroy(h);
+        return set_error(r == CUFFT_ALLOC_FAILED ? LF2_ERR_NOMEM : LF2_ERR_CUDA, "cuFFT error %d", (int)r);
+    }
+    *out = FftPlan{dev, dbl, (int)h, work};
+    return LF2_OK;
+}
+
+// Keeps a plan whose work is done, unless the call failed or enough are kept.
+void give_plan(lf2_lattice lat, const FftPlan &p, bool good) {
+    if (good) {
+        std::lock_guard<std::mutex> lock(lat->fft_mu);
+        if (lat->fft_idle.size() < kIdleFftPlans) {
+            try {
+                lat->fft_idle.push_back(p);
+                return;
+            } catch (const std::bad_alloc &) {
+            }
+        }
+    }
+    cufftDestroy((cufftHandle)p.handle);
+}
+
 }  // namespace
+
+namespace lf2 {
+void release_fft_plans(lf2_lattice lat) {
+    for (const FftPlan &p : lat->fft_idle) cufftDestroy((cufftHandle)p.handle);
+    lat->fft_idle.clear();
+}
+}  // namespace lf2
 
 extern "C" lf2_status lf2_power_spectrum(lf2_field f, int comp, int nbins, double dx, double *power, double *kmean,
                                          double *count, void *stream) {
@@ -165,22 +222,26 @@ extern "C" lf2_status lf2_power_spectrum(lf2_field f, int comp, int nbins, doubl
     const size_t rsz = dbl ? sizeof(double) : sizeof(float);
     const size_t csz = 2 * rsz;
     cudaStream_t s = (cudaStream_t)stream;
-    void *real = nullptr, *spec = nullptr;
-    double *partials = nullptr, *out = nullptr;
-    cufftHandle plan = 0;
-    bool have_plan = false;
-    lf2_status st = LF2_OK;
     const int kBinBlocks = 4 * device_sm_count();  // four histogram blocks per SM
-    cudaError_t e = cudaMalloc(&real, (size_t)sites * rsz);
-    if (e == cudaSuccess) e = cudaMalloc(&spec, (size_t)n * n * (n / 2 + 1) * csz);
-    if (e == cudaSuccess) e = cudaMalloc(&partials, (size_t)kBinBlocks * 3 * nbins * sizeof(double));
-    if (e == cudaSuccess) e = cudaMalloc(&out, (size_t)3 * nbins * sizeof(double));
+    FftPlan plan{};
+    lf2_status st = take_plan(f->lat, dbl, &plan);
+    if (st != LF2_OK) return st;
+    // one allocation: a component's values (a one-component field is read where it is), its half
+    // spectrum, the transform's work area, the partial rows and the sums
+    auto aligned = [](size_t b) { return (b + 255) / 256 * 256; };
+    const bool copy = f->ncomp > 1;
+    const size_t real_b = copy ? aligned((size_t)sites * rsz) : 0, spec_b = aligned((size_t)n * n * (n / 2 + 1) * csz),
+                 work_b = aligned(plan.work_bytes), part_b = aligned((size_t)kBinBlocks * 3 * nbins * sizeof(double)),
+                 out_b = (size_t)3 * nbins * sizeof(double);
+    char *arena = nullptr;
+    cudaError_t e = cudaMalloc(&arena, real_b + spec_b + work_b + part_b + out_b);
     if (e != cudaSuccess) st = cuda_error(e, "spectrum buffers");
+    void *real = arena, *spec = arena + real_b, *work = arena + real_b + spec_b;
+    double *partials = (double *)(arena + real_b + spec_b + work_b), *out = partials + part_b / sizeof(double);
     if (st == LF2_OK) {
-        cufftResult r = cufftPlan3d(&plan, n, n, n, dbl ? CUFFT_D2Z : CUFFT_R2C);
-        have_plan = r == CUFFT_SUCCESS;
-        if (r == CUFFT_SUCCESS) r = cufftSetStream(plan, s);
-        if (r != CUFFT_SUCCESS) st = set_error(r == CUFFT_ALLOC_FAILED ? LF2_ERR_NOMEM : LF2_ERR_CUDA, "cuFFT error %d", (int)r);
+        cufftResult r = cufftSetStream(plan.handle, s);
+        if (r == CUFFT_SUCCESS) r = cufftSetWorkArea(plan.handle, work);
+        if (r != CUFFT_SUCCESS) st = set_error(LF2_ERR_CUDA, "cuFFT error %d", (int)r);
     }
     // one component, or every component in order with their powers added bin by bin
     const int c0 = comp < 0 ? 0 : comp, c1 = comp < 0 ? f->ncomp : comp + 1;
@@ -190,7 +251,9 @@ extern "C" lf2_status lf2_power_spectrum(lf2_field f, int comp, int nbins, doubl
     for (int c = c0; c < c1 && st == LF2_OK; ++c) {
         const long long cap = 16LL * device_sm_count();
         const int g = (int)((sites + 255) / 256 < cap ? (sites + 255) / 256 : cap);
-        if (dbl)
+        if (!copy)
+            real = f->val[f->front];
+        else if (dbl)
             k_extract<double><<<g, 256, 0, s>>>((const double *)f->val[f->front], (double *)real, sites, f->ncomp, c);
         else
             k_extract<float><<<g, 256, 0, s>>>((const float *)f->val[f->front], (float *)real, sites, f->ncomp, c);
@@ -199,8 +262,8 @@ extern "C" lf2_status lf2_power_spectrum(lf2_field f, int comp, int nbins, doubl
             st = cuda_error(e, "component copy");
             break;
         }
-        const cufftResult r = dbl ? cufftExecD2Z(plan, (cufftDoubleReal *)real, (cufftDoubleComplex *)spec)
-                                  : cufftExecR2C(plan, (cufftReal *)real, (cufftComplex *)spec);
+        const cufftResult r = dbl ? cufftExecD2Z(plan.handle, (cufftDoubleReal *)real, (cufftDoubleComplex *)spec)
+                                  : cufftExecR2C(plan.handle, (cufftReal *)real, (cufftComplex *)spec);
         if (r != CUFFT_SUCCESS) {
             st = set_error(LF2_ERR_CUDA, "cuFFT error %d", (int)r);
             break;
@@ -216,17 +279,18 @@ extern "C" lf2_status lf2_power_spectrum(lf2_field f, int comp, int nbins, doubl
     if (st == LF2_OK) {
         k_bin_final<<<(3 * nbins * 32 + kBinThreads - 1) / kBinThreads, kBinThreads, 0, s>>>(partials, kBinBlocks, nbins, out);
         e = cudaGetLastError();
-        if (e == cudaSuccess) e = cudaMemcpyAsync(power, out, nbins * sizeof(double), cudaMemcpyDeviceToHost, s);
-        if (e == cudaSuccess) e = cudaMemcpyAsync(kmean, out + nbins, nbins * sizeof(double), cudaMemcpyDeviceToHost, s);
-        if (e == cudaSuccess) e = cudaMemcpyAsync(count, out + 2 * nbins, nbins * sizeof(double), cudaMemcpyDeviceToHost, s);
+        double host[3 * kMaxBins];
+        if (e == cudaSuccess) e = cudaMemcpyAsync(host, out, out_b, cudaMemcpyDeviceToHost, s);
         if (e == cudaSuccess) e = cudaStreamSynchronize(s);
         if (e != cudaSuccess) st = cuda_error(e, "binning");
+        if (st == LF2_OK) {
+            memcpy(power, host, nbins * sizeof(double));
+            memcpy(kmean, host + nbins, nbins * sizeof(double));
+            memcpy(count, host + 2 * nbins, nbins * sizeof(double));
+        }
     }
-    if (have_plan) cufftDestroy(plan);
-    if (real) cudaFree(real);
-    if (spec) cudaFree(spec);
-    if (partials) cudaFree(partials);
-    if (out) cudaFree(out);
+    give_plan(f->lat, plan, st == LF2_OK);
+    if (arena) cudaFree(arena);
     if (st != LF2_OK) return st;
     for (int b = 0; b < nbins; ++b) {  // sums -> means
         if (count[b] > 0) {
