@@ -20,6 +20,7 @@
 // arithmetic, give bitwise the record of the stand-alone reduction.
 #include <mutex>
 
+#include "lf2_barrier.cuh"
 #include "lf2_bounds.cuh"
 #include "lf2_internal.cuh"
 
@@ -397,60 +398,11 @@ __global__ void __launch_bounds__(kEnergyThreads, NC <= 2 ? 4 : 2)
 // which the reducing block joins only after it has read the rows of step k.
 
 // The row sets (at most kStepsMaxBlocks rows each) start at kStepsRowsOffset of a field's
-// scratch; the barrier slots (arrivals, generation, error) fill the row after them.
+// scratch; the barrier word (lf2_barrier.cuh) is in the row after them.
 constexpr int kRowSets = kEnergyStepsRowSets;
 constexpr int kStepsMaxBlocks = kEnergyStepsBlocks;
 constexpr size_t kBarrierOffset = (size_t)kStepsRowsOffset + (size_t)kRowSets * kStepsMaxBlocks * kEnergySlots;
 static_assert(kBarrierOffset + kEnergySlots == (size_t)kFieldScratchDoubles, "multi-step scratch layout");
-// A barrier waits at most about a second (2^24 polls of >= 64 ns); co-residency, which the
-// cooperative launch guarantees, keeps real waits to microseconds.
-constexpr unsigned kBarrierPolls = 1u << 24;
-
-// Arrival half of the grid barrier: once every thread of the block has made its writes,
-// thread 0 publishes them (fence) and counts the block in; the last block to arrive resets
-// the count and advances the generation.  Returns, in thread 0, the generation before the
-// arrival, which grid_wait compares against.
-__device__ __forceinline__ unsigned grid_arrive(unsigned *bar) {
-    __syncthreads();
-    unsigned g = 0u;
-    if (threadIdx.x == 0) {
-        g = *(volatile unsigned *)(bar + 1);
-        __threadfence();
-        if (atomicAdd(bar, 1u) == gridDim.x - 1) {
-            atomicExch(bar, 0u);
-            __threadfence();
-            atomicAdd(bar + 1, 1u);
-        }
-    }
-    return g;
-}
-
-// Waiting half: returns true once the generation has moved past g (every block arrived),
-// false when the wait ran out after polls_max polls, here or in another block (error flag).
-// The generation can move by one at most while a block waits, since no barrier completes
-// without this block's next arrival.
-__device__ __forceinline__ bool grid_wait(unsigned *bar, unsigned g, unsigned polls_max) {
-    __shared__ int s_ok;
-    if (threadIdx.x == 0) {
-        int ok = 1;
-        volatile unsigned *gen = bar + 1;
-        unsigned polls = 0;
-        while (*gen == g) {
-            if (++polls > polls_max) {
-                atomicExch(bar + 2, 1u);
-                ok = 0;
-                break;
-            }
-            __nanosleep(64);
-        }
-        __threadfence();
-        if (*(volatile unsigned *)(bar + 2) != 0u) ok = 0;
-        s_ok = ok;
-    }
-    __syncthreads();
-    return s_ok != 0;
-}
-
 // A run cut short by a barrier that did not complete leaves NaN records from `from` on (the
 // record of a step is finished during the next step, so `from` is the step before that barrier).
 __device__ __forceinline__ void poison_records(double *records, int from, int nsteps) {
@@ -487,12 +439,12 @@ __device__ __forceinline__ void steps_energy_loop(R *phi_a, R *phi_b, Geom g, co
             R *dst = (step & 1) ? phi_a : phi_b;
             for (SiteWalk w = first; w.s < g.sites; w.advance(d, g)) site(src, dst, w, acc);
         }
-        const unsigned gen = grid_arrive(bar);  // step's fields published (the final pass: rows only)
+        grid_arrive(bar);  // step's fields published (the final pass: rows only)
         if (!reducer && step < nsteps) {
             block_sum<NS>(acc, sh);
             if (threadIdx.x < NS) rows_of(step, blockIdx.x, 1)[threadIdx.x] = sh[threadIdx.x][0];
         }
-        if (!grid_wait(bar, gen, polls)) {
+        if (!grid_wait(bar, (unsigned)(step + 1) * gridDim.x, polls)) {
             poison_records(records, step > 0 ? step - 1 : 0, nsteps);
             return;
         }
@@ -724,8 +676,8 @@ cudaError_t launch_steps_energy(const StepArgs &a, int nsteps, double *scratch, 
                                 cudaStream_t s) {
     const int nb = energy_grid(a.g.sites);  // site blocks, as for one launch per step
     if (!a.drift || nsteps < 2 || nb > kStepsMaxBlocks) return cudaErrorNotSupported;
-    // the barrier's arrival count, generation and error flag start at zero
-    cudaError_t e = cudaMemsetAsync(scratch + kBarrierOffset, 0, 4 * sizeof(unsigned), s);
+    // the barrier's arrival count and error flag start at zero
+    cudaError_t e = cudaMemsetAsync(scratch + kBarrierOffset, 0, 2 * sizeof(unsigned), s);
     if (e != cudaSuccess) return e;
     const CoefE ke = make_coefE(a.p);
     const unsigned polls = no_wait ? 0u : kBarrierPolls;
@@ -741,11 +693,11 @@ cudaError_t launch_steps_energy(const StepArgs &a, int nsteps, double *scratch, 
 }
 
 cudaError_t steps_energy_timed_out(double *scratch, bool *out, cudaStream_t s) {
-    unsigned word[4] = {0, 0, 0, 0};
+    unsigned word[2] = {0, 0};  // arrivals, error flag
     cudaError_t e = cudaMemcpyAsync(word, scratch + kBarrierOffset, sizeof word, cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     if (e != cudaSuccess) return e;
-    *out = word[2] != 0u;
+    *out = word[1] != 0u;
     if (*out) {
         e = cudaMemsetAsync(scratch + kBarrierOffset, 0, sizeof word, s);  // reported once
         if (e == cudaSuccess) e = cudaStreamSynchronize(s);
