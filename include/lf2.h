@@ -228,7 +228,11 @@ lf2_status lf2_leapfrog_init(lf2_field phi, lf2_field pi, const lf2_params *p, v
  * shape, else the default one; results are bitwise identical whichever kernel runs.  The
  * environment variable LF2_TUNE changes that: "off" ignores tuned plans, "force" tunes a shape
  * that has no plan on its first call (that call synchronises and allocates, so keep it out of
- * stream capture). */
+ * stream capture).  Two or more steps of a small lattice without a plan (one site per resident
+ * thread: up to about 230,000 sites of a real FP32 field) run in one cooperative launch with a grid
+ * barrier between steps, once lf2_leapfrog_init or an energy call has allocated phi's scratch; the
+ * barrier's waits are bounded as in lf2_leapfrog_energy and reported by lf2_field_check.  Calls on
+ * one phi share that scratch: order them on one stream. */
 lf2_status lf2_leapfrog(lf2_field phi, lf2_field pi, const lf2_params *p, int nsteps, void *stream);
 
 /* lf2_leapfrog with an explicit kernel choice (testing and tuning).  LF2_ERR_UNSUPPORTED if the
@@ -289,7 +293,7 @@ lf2_status lf2_leapfrog_energy(lf2_field phi, lf2_field pi, const lf2_params *p,
 lf2_status lf2_field_compare(lf2_field f, int which, const void *ref, lf2_precision ref_prec, double *out,
                              void *stream);
 
-/* Status of the last multi-step lf2_leapfrog_energy run on phi: LF2_ERR_TIMEOUT (once; the
+/* Status of the last multi-step lf2_leapfrog_energy or lf2_leapfrog run on phi: LF2_ERR_TIMEOUT (once; the
  * flag is then cleared) if one of its grid barriers gave up, else LF2_OK.  The paper has no
  * counterpart (its programs have no device-side waits).  Synchronises `stream`.  Host-side
  * failure injection for tests: with LF2_FAULT=timeout in the environment the barrier waits give

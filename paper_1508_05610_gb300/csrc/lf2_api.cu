@@ -479,6 +479,16 @@ lf2_status lf2_leapfrog_ex(lf2_field phi, lf2_field pi, const lf2_params *p, int
     };
 
     int done = 0;
+    // small lattices without a tuned plan: all steps in one cooperative launch, when
+    // lf2_leapfrog_init (or an energy) has made the scratch its barrier needs
+    if (kernel == LF2_KERNEL_AUTO && phi->energy_scratch) {
+        const cudaError_t e = launch_steps_plain(probe, nsteps, phi->energy_scratch, s);
+        if (e == cudaSuccess) {
+            if (nsteps & 1) phi->front = 1 - phi->front;
+            return LF2_OK;
+        }
+        if (e != cudaErrorNotSupported) return cuda_fail(e, "multi-step launch");
+    }
     if (kernel == LF2_KERNEL_TBLOCK) {
         TbConfig c{cfg->depth, cfg->cx, cfg->tile_x, tile_y, zchunk, cfg->cluster};
         TbArgs ta = tb_args(phi, pi, p);
@@ -597,8 +607,8 @@ lf2_status lf2_field_check(lf2_field phi, void *stream) {
     LF2_CUDA(steps_energy_timed_out(phi->energy_scratch, &timed_out, (cudaStream_t)stream), "status read");
     if (timed_out)
         return fail(LF2_ERR_TIMEOUT,
-                    "a grid barrier of the last multi-step lf2_leapfrog_energy run gave up: its records from that step "
-                    "on are NaN and the fields are not a valid state");
+                    "a grid barrier of the last multi-step run gave up: the records of an lf2_leapfrog_energy run "
+                    "from that step on are NaN and the fields are not a valid state");
     return LF2_OK;
 }
 

@@ -5,8 +5,8 @@
 // and is never reset, the high half is an error flag.  Barrier number b (from 0) is complete when
 // the count has reached (b + 1) * blocks, so the last arrival releases the waiters by itself, and one
 // load tells a waiter both the count and the error.  (A counter that the last block reset before it
-// advanced a generation, a fence on each side and a second load for the error flag: FIG us a barrier
-// longer.)  The count wraps modulo 2^32; a waiter is never more than one barrier behind.
+// advanced a generation, a fence on each side and a second load for the error flag made a barrier
+// 1.2 us longer.)  The count wraps modulo 2^32; a waiter is never more than one barrier behind.
 //
 // Waits are bounded: a cooperative launch keeps every block resident, so real waits take
 // microseconds; after kBarrierPolls polls of about half a microsecond (about a second) the waiter sets the

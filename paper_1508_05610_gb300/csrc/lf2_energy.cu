@@ -142,9 +142,10 @@ __device__ __forceinline__ double sub_exact(double a, double b) {
 // -x, +x, -y, +y, -z, +z; p: pi_{n-1/2}, in the storage type.  Explicit round-to-nearest
 // operations keep the stand-alone and fused kernels bitwise equal; the half kick is the FP64 kick's
 // arithmetic.  Component by component, so that few widened values are live at once.  nb: the
-// neighbour sums, for the FP64 update that follows.  INTSUB: the differences in integers (the
-// multi-step kernel's FP64 instance, bound by latency, is 3 % faster with FP64 subtractions).
-template <typename R, int NC, bool INTSUB>
+// neighbour sums, which the FP64 update uses too; computed here unless HAVE_NB.  INTSUB: the
+// differences in integers (the multi-step kernel's FP64 instance, bound by latency, is 3 % faster
+// with FP64 subtractions).
+template <typename R, int NC, bool INTSUB, bool HAVE_NB = false>
 __device__ __forceinline__ void energy_site(const R (&c)[NC], const R (&xm)[NC], const R (&xp)[NC], const R (&ym)[NC],
                                             const R (&yp)[NC], const R (&zm)[NC], const R (&zp)[NC], const R (&p)[NC],
                                             double (&nb)[NC], double (&acc)[kNs<NC>], const CoefE &k) {
@@ -163,7 +164,7 @@ __device__ __forceinline__ void energy_site(const R (&c)[NC], const R (&xm)[NC],
     acc[kPot] = __fma_rn(w, w, acc[kPot]);
 #pragma unroll
     for (int a = 0; a < NC; ++a) {
-        nb[a] = neighbour_sum(xm[a], xp[a], ym[a], yp[a], zm[a], zp[a]);
+        if (!HAVE_NB) nb[a] = neighbour_sum(xm[a], xp[a], ym[a], yp[a], zm[a], zp[a]);
         const double d = widen(c[a]);
         const double pin = __fma_rn(k.ah, nb[a], __fma_rn(-gh, d, widen(p[a])));
         acc[kKin] = __fma_rn(pin, pin, acc[kKin]);
@@ -288,25 +289,25 @@ __global__ void __launch_bounds__(kEnergyThreads, kEnergyResident<NC>) k_energy(
 
 // One site of a fused step + energy, FP64: adds the energy of (phi_n, pi_{n-1/2}) at site s
 // to acc and writes the step to (phi_{n+1}, pi_{n+1/2}), from one read of the site's stencil.
-template <int NC, bool COHERENT>
+template <int NC>
 __device__ __forceinline__ void site_step_energy_f64(const double *__restrict__ phi, double *__restrict__ phi_out,
                                                      double *__restrict__ pi, const SiteWalk &w, const Geom &g,
                                                      const Coef64 &k, const CoefE &ke, double (&acc)[kNs<NC>]) {
     const Nbr n = neighbours(w, g);
     const long long s = w.s;
     double c[NC], xm[NC], xp[NC], ym[NC], yp[NC], zm[NC], zp[NC], p[NC], out[NC];
-    load_site<double, NC, COHERENT>(phi, s, g.sites, c);
-    load_site<double, NC, COHERENT>(phi, n.xm, g.sites, xm);
-    load_site<double, NC, COHERENT>(phi, n.xp, g.sites, xp);
-    load_site<double, NC, COHERENT>(phi, n.ym, g.sites, ym);
-    load_site<double, NC, COHERENT>(phi, n.yp, g.sites, yp);
-    load_site<double, NC, COHERENT>(phi, n.zm, g.sites, zm);
-    load_site<double, NC, COHERENT>(phi, n.zp, g.sites, zp);
+    load_site<double, NC>(phi, s, g.sites, c);
+    load_site<double, NC>(phi, n.xm, g.sites, xm);
+    load_site<double, NC>(phi, n.xp, g.sites, xp);
+    load_site<double, NC>(phi, n.ym, g.sites, ym);
+    load_site<double, NC>(phi, n.yp, g.sites, yp);
+    load_site<double, NC>(phi, n.zm, g.sites, zm);
+    load_site<double, NC>(phi, n.zp, g.sites, zp);
     const long long o = checked(s * NC, NC, g.sites * NC);
 #pragma unroll
     for (int a = 0; a < NC; ++a) p[a] = pi[o + a];
     double nb[NC];
-    energy_site<double, NC, !COHERENT>(c, xm, xp, ym, yp, zm, zp, p, nb, acc, ke);
+    energy_site<double, NC, true>(c, xm, xp, ym, yp, zm, zp, p, nb, acc, ke);
     update_f64_nb<NC>(c, nb, p, out, k);
 #pragma unroll
     for (int a = 0; a < NC; ++a) {
@@ -317,7 +318,7 @@ __device__ __forceinline__ void site_step_energy_f64(const double *__restrict__ 
 
 // The same for FP32 storage (KAHAN: compensated drift); the energy is computed in FP64 from
 // the exact conversions of the stored values.
-template <int NC, bool KAHAN, bool COHERENT>
+template <int NC, bool KAHAN>
 __device__ __forceinline__ void site_step_energy_f32(const float *__restrict__ phi, float *__restrict__ phi_out,
                                                      float *__restrict__ pi, float *__restrict__ comp, const SiteWalk &w,
                                                      const Geom &g, const Coef32 &k, const CoefE &ke,
@@ -331,13 +332,13 @@ __device__ __forceinline__ void site_step_energy_f32(const float *__restrict__ p
     float c[NC], xm[NC], xp[NC], ym[NC], yp[NC], zm[NC], zp[NC], p[NC], cm[NC], out[NC];
 #pragma unroll
     for (int a = 0; a < NC; ++a) {
-        c[a] = ld_field<COHERENT>(phi + o + a);
-        xm[a] = ld_field<COHERENT>(phi + ixm + a);
-        xp[a] = ld_field<COHERENT>(phi + ixp + a);
-        ym[a] = ld_field<COHERENT>(phi + iym + a);
-        yp[a] = ld_field<COHERENT>(phi + iyp + a);
-        zm[a] = ld_field<COHERENT>(phi + izm + a);
-        zp[a] = ld_field<COHERENT>(phi + izp + a);
+        c[a] = __ldg(phi + o + a);
+        xm[a] = __ldg(phi + ixm + a);
+        xp[a] = __ldg(phi + ixp + a);
+        ym[a] = __ldg(phi + iym + a);
+        yp[a] = __ldg(phi + iyp + a);
+        zm[a] = __ldg(phi + izm + a);
+        zp[a] = __ldg(phi + izp + a);
         p[a] = pi[o + a];
         cm[a] = KAHAN ? comp[o + a] : 0.0f;
     }
@@ -362,7 +363,7 @@ __global__ void __launch_bounds__(kEnergyThreads, kEnergyResident<NC>)
 #pragma unroll
     for (int j = 0; j < kNs<NC>; ++j) acc[j] = 0.0;
     for (SiteWalk w((long long)blockIdx.x * blockDim.x + threadIdx.x, g); w.s < g.sites; w.advance(d, g))
-        site_step_energy_f64<NC, false>(phi, phi_out, pi, w, g, k, ke, acc);
+        site_step_energy_f64<NC>(phi, phi_out, pi, w, g, k, ke, acc);
     finish_energy<NC>(acc, sh, scratch, ke, record);
 }
 
@@ -376,26 +377,30 @@ __global__ void __launch_bounds__(kEnergyThreads, NC <= 2 ? 4 : 2)
 #pragma unroll
     for (int j = 0; j < kNs<NC>; ++j) acc[j] = 0.0;
     for (SiteWalk w((long long)blockIdx.x * blockDim.x + threadIdx.x, g); w.s < g.sites; w.advance(d, g))
-        site_step_energy_f32<NC, KAHAN, false>(phi, phi_out, pi, comp, w, g, k, ke, acc);
+        site_step_energy_f32<NC, KAHAN>(phi, phi_out, pi, comp, w, g, k, ke, acc);
     finish_energy<NC>(acc, sh, scratch, ke, record);
 }
 
-// ------------------------------------------- many fused steps in one launch (small lattices)
-// On a small lattice (the 32^3 run with an energy every step) a step costs a few microseconds
-// of arithmetic and about as much again in launch gaps and in the serial reduction.  One
-// cooperative launch runs all steps: the same grid, site order and per-site code as
-// k_step_energy for the site blocks, a grid barrier between steps, and one extra block, which
-// owns no sites and reduces the partial rows.  The fields and every record are bitwise those
-// of one launch per step.
+// ------------------------------------------- many steps in one launch (small lattices)
+// On a small lattice a step is a few microseconds of launch gaps and latency around very little
+// arithmetic.  One cooperative launch runs all steps, with a grid barrier (lf2_barrier.cuh) between
+// them, for lattices that give every resident thread at most one site: a thread keeps its site's
+// field value, momentum and compensation in registers from step to step, loads six neighbours,
+// stores one field value and arrives at the barrier.  The arithmetic is the one-step kernels', so
+// fields and records are bitwise those of one launch per step.
 //
-// The barrier is split in two halves.  A site block arrives as soon as its part of step k is
-// written (that is all the next step needs), then sums its energy accumulators into its
-// partial row of step k, then waits.  The block sums thus overlap the barrier instead of
-// preceding it.  A site block writes its row of step k before it arrives at barrier k+1, so
-// the reducing block sums the rows of step k once barrier k+1 has completed, while the site
-// blocks run step k+2, and one more barrier after the last step completes its rows.  The rows
-// rotate over three sets: a site block writes the set of step k+3 only after barrier k+2,
-// which the reducing block joins only after it has read the rows of step k.
+// ENERGY: the records of k_step_energy too, with its partial sums and their order.  The energy of a
+// step comes after the arrival, while the other blocks arrive: the site blocks add it up and write
+// the partial row of step k before they arrive at barrier k+1, and one extra block, which owns no
+// sites, reduces the rows of step k once barrier k+1 has completed, while the site blocks run step
+// k+2; one more barrier after the last step completes its rows.  The rows rotate over three sets: a
+// site block writes the set of step k+3 only after barrier k+2, which the reducing block joins only
+// after it has read the rows of step k.
+//
+// 32^3 real FP64, a step: 3.8 us with its energy (4.1 with the energy before the arrival and pi in
+// memory, 5.3 with a two-atomic barrier too), 2.2 without (4.3 at best as launches of the streaming
+// kernel); 48x40x36 real FP32+Kahan without energy 6.1 -> 1.8 us.  What is left is the barrier's
+// trips through L2 and the loads that follow it.
 
 // The row sets (at most kStepsMaxBlocks rows each) start at kStepsRowsOffset of a field's
 // scratch; the barrier word (lf2_barrier.cuh) is in the row after them.
@@ -403,6 +408,7 @@ constexpr int kRowSets = kEnergyStepsRowSets;
 constexpr int kStepsMaxBlocks = kEnergyStepsBlocks;
 constexpr size_t kBarrierOffset = (size_t)kStepsRowsOffset + (size_t)kRowSets * kStepsMaxBlocks * kEnergySlots;
 static_assert(kBarrierOffset + kEnergySlots == (size_t)kFieldScratchDoubles, "multi-step scratch layout");
+
 // A run cut short by a barrier that did not complete leaves NaN records from `from` on (the
 // record of a step is finished during the next step, so `from` is the step before that barrier).
 __device__ __forceinline__ void poison_records(double *records, int from, int nsteps) {
@@ -411,17 +417,17 @@ __device__ __forceinline__ void poison_records(double *records, int from, int ns
         for (int i = 0; i < kEnergySlots; ++i) records[(size_t)j * kEnergySlots + i] = __longlong_as_double(0x7ff8000000000000LL);
 }
 
-// The step loop shared by the FP64 and FP32 kernels.  site(src, dst, w, acc) performs the
-// fused step + energy of the site that w stands on; d is the site blocks' grid stride.
-template <int NC, typename R, typename Site>
-__device__ __forceinline__ void steps_energy_loop(R *phi_a, R *phi_b, Geom g, const Stride3 &d, const CoefE &ke, int nsteps,
-                                                  double *__restrict__ scratch, double *__restrict__ records,
-                                                  unsigned polls, double (&sh)[kNs<NC>][kEnergyThreads], Site site) {
+// MODE: 0 = FP32 plain drift, 1 = FP32 Kahan drift, 3 = FP64.  Launched with energy_grid(sites)
+// site blocks, and with ENERGY one more.
+template <typename R, int NC, int MODE, bool ENERGY, typename CoefT>
+__global__ void __launch_bounds__(kEnergyThreads, 2)
+    k_steps(R *phi_a, R *phi_b, R *__restrict__ pi, float *__restrict__ comp, Geom g, CoefT k, CoefE ke, int nsteps,
+            double *__restrict__ scratch, double *__restrict__ records, unsigned polls) {
     constexpr int NS = kNs<NC>;
+    __shared__ double sh[ENERGY ? NS : 1][ENERGY ? kEnergyThreads : 1];
     unsigned *bar = reinterpret_cast<unsigned *>(scratch + kBarrierOffset);
-    const int nsb = (int)gridDim.x - 1;  // site blocks; the last block reduces
-    const bool reducer = (int)blockIdx.x == nsb;
-    const SiteWalk first((long long)blockIdx.x * blockDim.x + threadIdx.x, g);
+    const int nsb = ENERGY ? (int)gridDim.x - 1 : (int)gridDim.x;
+    const bool reducer = ENERGY && (int)blockIdx.x == nsb;
     // rows [first, first + count) of the set of `step`, inside the row-set region (checked in
     // the debug build against that region, so neither the reduction layout before it nor the
     // barrier row after it can be hit)
@@ -430,50 +436,83 @@ __device__ __forceinline__ void steps_energy_loop(R *phi_a, R *phi_b, Geom g, co
                                       count * kEnergySlots, (long long)kRowSets * kStepsMaxBlocks * kEnergySlots);
         return scratch + kStepsRowsOffset + rel;
     };
-    for (int step = 0; step <= nsteps; ++step) {
-        double acc[NS];
+    const SiteWalk w((long long)blockIdx.x * kEnergyThreads + threadIdx.x, g);
+    const bool active = !reducer && w.s < g.sites;
+    const Nbr n = active ? neighbours(w, g) : Nbr{0, 0, 0, 0, 0, 0};
+    const long long o = active ? checked(w.s * NC, NC, g.sites * NC) : 0;
+    R c[NC], p[NC];
+    float cm[NC];
 #pragma unroll
-        for (int j = 0; j < NS; ++j) acc[j] = 0.0;
-        if (!reducer && step < nsteps) {
+    for (int a = 0; a < NC; ++a) {
+        c[a] = active ? __ldcg(phi_a + o + a) : R(0);
+        p[a] = active ? pi[o + a] : R(0);
+        cm[a] = active && MODE == 1 ? comp[o + a] : 0.0f;
+    }
+    for (int step = 0; step < nsteps + (ENERGY ? 1 : 0); ++step) {
+        const bool stepping = active && step < nsteps;
+        R xm[NC], xp[NC], ym[NC], yp[NC], zm[NC], zp[NC], pn[NC], out[NC];
+        double nb[NC];
+        if (stepping) {
             const R *src = (step & 1) ? phi_b : phi_a;
             R *dst = (step & 1) ? phi_a : phi_b;
-            for (SiteWalk w = first; w.s < g.sites; w.advance(d, g)) site(src, dst, w, acc);
+            load_site<R, NC, true>(src, n.xm, g.sites, xm);
+            load_site<R, NC, true>(src, n.xp, g.sites, xp);
+            load_site<R, NC, true>(src, n.ym, g.sites, ym);
+            load_site<R, NC, true>(src, n.yp, g.sites, yp);
+            load_site<R, NC, true>(src, n.zm, g.sites, zm);
+            load_site<R, NC, true>(src, n.zp, g.sites, zp);
+#pragma unroll
+            for (int a = 0; a < NC; ++a) pn[a] = p[a];
+            if constexpr (MODE == 3) {
+                neighbour_sums<NC>(xm, xp, ym, yp, zm, zp, nb);
+                update_f64_nb<NC>(c, nb, pn, out, k);
+            } else {
+                update_f32<NC, MODE == 1>(c, xm, xp, ym, yp, zm, zp, pn, cm, out, k);
+            }
+#pragma unroll
+            for (int a = 0; a < NC; ++a) dst[o + a] = out[a];
+        }
+        if (!ENERGY && step == nsteps - 1) {
+            if (stepping) {
+#pragma unroll
+                for (int a = 0; a < NC; ++a) p[a] = pn[a];
+            }
+            break;
         }
         grid_arrive(bar);  // step's fields published (the final pass: rows only)
-        if (!reducer && step < nsteps) {
-            block_sum<NS>(acc, sh);
-            if (threadIdx.x < NS) rows_of(step, blockIdx.x, 1)[threadIdx.x] = sh[threadIdx.x][0];
+        if constexpr (ENERGY) {
+            if (!reducer && step < nsteps) {
+                double acc[NS];
+#pragma unroll
+                for (int j = 0; j < NS; ++j) acc[j] = 0.0;
+                if (stepping) energy_site<R, NC, MODE != 3, MODE == 3>(c, xm, xp, ym, yp, zm, zp, p, nb, acc, ke);
+                block_sum<NS>(acc, sh);
+                if (threadIdx.x < NS) rows_of(step, blockIdx.x, 1)[threadIdx.x] = sh[threadIdx.x][0];
+            }
+        }
+        if (stepping) {
+#pragma unroll
+            for (int a = 0; a < NC; ++a) {
+                c[a] = out[a];
+                p[a] = pn[a];
+            }
         }
         if (!grid_wait(bar, (unsigned)(step + 1) * gridDim.x, polls)) {
-            poison_records(records, step > 0 ? step - 1 : 0, nsteps);
+            if constexpr (ENERGY) poison_records(records, step > 0 ? step - 1 : 0, nsteps);
             return;
         }
-        if (reducer && step > 0)
-            reduce_rows<NC>(rows_of(step - 1, 0, nsb), nsb, sh, ke, records + (size_t)(step - 1) * kEnergySlots, nullptr);
+        if constexpr (ENERGY) {
+            if (reducer && step > 0)
+                reduce_rows<NC>(rows_of(step - 1, 0, nsb), nsb, sh, ke, records + (size_t)(step - 1) * kEnergySlots, nullptr);
+        }
     }
-}
-
-template <int NC>
-__global__ void __launch_bounds__(kEnergyThreads, 2)
-    k_steps_energy_f64(double *phi_a, double *phi_b, double *__restrict__ pi, Geom g, Stride3 d, Coef64 k, CoefE ke, int nsteps,
-                       double *__restrict__ scratch, double *__restrict__ records, unsigned polls) {
-    __shared__ double sh[kNs<NC>][kEnergyThreads];
-    steps_energy_loop<NC>(phi_a, phi_b, g, d, ke, nsteps, scratch, records, polls, sh,
-                          [&](const double *src, double *dst, const SiteWalk &w, double (&acc)[kNs<NC>]) {
-                              site_step_energy_f64<NC, true>(src, dst, pi, w, g, k, ke, acc);
-                          });
-}
-
-template <int NC, bool KAHAN>
-__global__ void __launch_bounds__(kEnergyThreads, 2)
-    k_steps_energy_f32(float *phi_a, float *phi_b, float *__restrict__ pi, float *__restrict__ comp, Geom g, Stride3 d,
-                       Coef32 k, CoefE ke, int nsteps, double *__restrict__ scratch, double *__restrict__ records,
-                       unsigned polls) {
-    __shared__ double sh[kNs<NC>][kEnergyThreads];
-    steps_energy_loop<NC>(phi_a, phi_b, g, d, ke, nsteps, scratch, records, polls, sh,
-                          [&](const float *src, float *dst, const SiteWalk &w, double (&acc)[kNs<NC>]) {
-                              site_step_energy_f32<NC, KAHAN, true>(src, dst, pi, comp, w, g, k, ke, acc);
-                          });
+    if (active) {
+#pragma unroll
+        for (int a = 0; a < NC; ++a) {
+            pi[o + a] = p[a];
+            if (MODE == 1) comp[o + a] = cm[a];
+        }
+    }
 }
 
 // One block per 256 sites up to kEnergyBlocks: small lattices (a 32^3 run with an energy every
@@ -625,9 +664,10 @@ cudaError_t compare_ref(const RA *a, const void *ref, bool ref_double, long long
     return cudaGetLastError();
 }
 
-// Cooperative launch of k (grid nb) when every block can be resident at once.
+// Cooperative launch of kern (grid nb) when every block can be resident at once; clears the barrier
+// word first.
 template <typename K, typename... Args>
-cudaError_t launch_cooperative(K kern, int nb, cudaStream_t s, Args... args) {
+cudaError_t launch_cooperative(K kern, int nb, void *barrier, cudaStream_t s, Args... args) {
     int dev = 0, coop = 0, sms = 0, per_sm = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev);
@@ -635,6 +675,9 @@ cudaError_t launch_cooperative(K kern, int nb, cudaStream_t s, Args... args) {
     if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kEnergyThreads, 0);
     if (e != cudaSuccess) return e;
     if (!coop || (long long)per_sm * sms < nb) return cudaErrorNotSupported;
+    // the barrier's arrival count and error flag start at zero
+    e = cudaMemsetAsync(barrier, 0, 2 * sizeof(unsigned), s);
+    if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(nb);
     cfg.blockDim = dim3(kEnergyThreads);
@@ -653,43 +696,50 @@ cudaError_t launch_cooperative(K kern, int nb, cudaStream_t s, Args... args) {
     return r;
 }
 
-// nb site blocks plus the reducing block
-template <int NC>
-cudaError_t steps_energy_nc(const StepArgs &a, int nsteps, int nb, const CoefE &ke, double *scratch, double *records,
-                            unsigned polls, cudaStream_t s) {
-    const Stride3 d = make_stride3((long long)nb * kEnergyThreads, a.g);
-    nb += 1;
+template <int NC, bool ENERGY>
+cudaError_t steps_nc(const StepArgs &a, int nsteps, const CoefE &ke, double *scratch, double *records, unsigned polls,
+                     cudaStream_t s) {
+    // with ENERGY the partial sums' blocks and the reducing one
+    const int nb = ENERGY ? energy_grid(a.g.sites) + 1 : (int)((a.g.sites + kEnergyThreads - 1) / kEnergyThreads);
     if (a.prec == LF2_F64)
-        return launch_cooperative(k_steps_energy_f64<NC>, nb, s, (double *)a.phi, (double *)a.phi_out, (double *)a.pi,
-                                  a.g, d, make_coef64(a.p, a.dt), ke, nsteps, scratch, records, polls);
+        return launch_cooperative(k_steps<double, NC, 3, ENERGY, Coef64>, nb, scratch + kBarrierOffset, s, (double *)a.phi, (double *)a.phi_out,
+                                  (double *)a.pi, a.comp, a.g, make_coef64(a.p, a.dt), ke, nsteps, scratch, records, polls);
     const Coef32 k = make_coef32(a.p, a.dt);
     if (a.prec == LF2_F32_KAHAN)
-        return launch_cooperative(k_steps_energy_f32<NC, true>, nb, s, (float *)a.phi, (float *)a.phi_out,
-                                  (float *)a.pi, a.comp, a.g, d, k, ke, nsteps, scratch, records, polls);
-    return launch_cooperative(k_steps_energy_f32<NC, false>, nb, s, (float *)a.phi, (float *)a.phi_out, (float *)a.pi,
-                              a.comp, a.g, d, k, ke, nsteps, scratch, records, polls);
+        return launch_cooperative(k_steps<float, NC, 1, ENERGY, Coef32>, nb, scratch + kBarrierOffset, s, (float *)a.phi, (float *)a.phi_out,
+                                  (float *)a.pi, a.comp, a.g, k, ke, nsteps, scratch, records, polls);
+    return launch_cooperative(k_steps<float, NC, 0, ENERGY, Coef32>, nb, scratch + kBarrierOffset, s, (float *)a.phi, (float *)a.phi_out,
+                              (float *)a.pi, a.comp, a.g, k, ke, nsteps, scratch, records, polls);
+}
+
+template <bool ENERGY>
+cudaError_t launch_steps(const StepArgs &a, int nsteps, double *scratch, double *records, bool no_wait, cudaStream_t s) {
+    if (!a.drift || nsteps < 2) return cudaErrorNotSupported;
+    // one site per thread; the launch itself checks that all blocks are resident
+    if (a.g.sites > (ENERGY ? (long long)kStepsMaxBlocks : 8LL * device_sm_count()) * kEnergyThreads)
+        return cudaErrorNotSupported;
+    const CoefE ke = make_coefE(a.p);
+    const unsigned polls = no_wait ? 0u : kBarrierPolls;
+    switch (a.ncomp) {
+        case 1: return steps_nc<1, ENERGY>(a, nsteps, ke, scratch, records, polls, s);
+        case 2: return steps_nc<2, ENERGY>(a, nsteps, ke, scratch, records, polls, s);
+        case 3: return steps_nc<3, ENERGY>(a, nsteps, ke, scratch, records, polls, s);
+        case 4: return steps_nc<4, ENERGY>(a, nsteps, ke, scratch, records, polls, s);
+        case 5: return steps_nc<5, ENERGY>(a, nsteps, ke, scratch, records, polls, s);
+        case 6: return steps_nc<6, ENERGY>(a, nsteps, ke, scratch, records, polls, s);
+        default: return cudaErrorNotSupported;
+    }
 }
 
 }  // namespace
 
 cudaError_t launch_steps_energy(const StepArgs &a, int nsteps, double *scratch, double *records, bool no_wait,
                                 cudaStream_t s) {
-    const int nb = energy_grid(a.g.sites);  // site blocks, as for one launch per step
-    if (!a.drift || nsteps < 2 || nb > kStepsMaxBlocks) return cudaErrorNotSupported;
-    // the barrier's arrival count and error flag start at zero
-    cudaError_t e = cudaMemsetAsync(scratch + kBarrierOffset, 0, 2 * sizeof(unsigned), s);
-    if (e != cudaSuccess) return e;
-    const CoefE ke = make_coefE(a.p);
-    const unsigned polls = no_wait ? 0u : kBarrierPolls;
-    switch (a.ncomp) {
-        case 1: return steps_energy_nc<1>(a, nsteps, nb, ke, scratch, records, polls, s);
-        case 2: return steps_energy_nc<2>(a, nsteps, nb, ke, scratch, records, polls, s);
-        case 3: return steps_energy_nc<3>(a, nsteps, nb, ke, scratch, records, polls, s);
-        case 4: return steps_energy_nc<4>(a, nsteps, nb, ke, scratch, records, polls, s);
-        case 5: return steps_energy_nc<5>(a, nsteps, nb, ke, scratch, records, polls, s);
-        case 6: return steps_energy_nc<6>(a, nsteps, nb, ke, scratch, records, polls, s);
-        default: return cudaErrorNotSupported;
-    }
+    return launch_steps<true>(a, nsteps, scratch, records, no_wait, s);
+}
+
+cudaError_t launch_steps_plain(const StepArgs &a, int nsteps, double *scratch, cudaStream_t s) {
+    return launch_steps<false>(a, nsteps, scratch, nullptr, false, s);
 }
 
 cudaError_t steps_energy_timed_out(double *scratch, bool *out, cudaStream_t s) {

@@ -62,3 +62,29 @@ def test_derivative_of_every_row_length(lf2, shape, ncomp, prec):
             want = (np.roll(v, -1, 2 - dim) - np.roll(v, 1, 2 - dim)) * inv
             got = lf2.lf2_field_download(s.pi, s.host_shape)
             assert np.array_equal(got, want.astype(np.float64)), dim
+
+
+@pytest.mark.parametrize("prec", ["f64", "f32k", "f32"])
+@pytest.mark.parametrize("shape,ncomp", [((1, 1, 1), 1), ((5, 3, 2), 2), ((16, 16, 16), 1), ((31, 9, 8), 3),
+                                         ((48, 40, 36), 1), ((20, 18, 14), 4), ((13, 11, 9), 5), ((16, 12, 10), 6),
+                                         ((60, 60, 60), 1), ((61, 61, 61), 1), ((64, 64, 64), 1), ((64, 64, 40), 2)])
+def test_many_steps_of_small_lattices_equal_single_steps(lf2, monkeypatch, shape, ncomp, prec):
+    """Runs of 2, 7 and 1 steps (one cooperative launch where every site has a resident thread, else a
+    launch per step), even and odd, bitwise as many single calls of the site kernel; the runs reuse
+    the scratch and continue from each other's state."""
+    monkeypatch.setenv("LF2_TUNE", "off")
+    nx, ny, nz = shape
+    phi0 = inputs.gaussian_field(nx, ny, nz, ncomp, sigma=0.4, seed=911)
+    pi0 = inputs.gaussian_field(nx, ny, nz, ncomp, sigma=0.2, seed=912)
+    p = lf2.params(**KW)
+    with lf2.System(shape, ncomp, prec) as a, lf2.System(shape, ncomp, prec) as b:
+        for s in (a, b):
+            s.upload(phi0, pi0)
+            lf2.lf2_leapfrog_init(s.phi, s.pi, p)
+        for n in (2, 7, 1):
+            lf2.lf2_leapfrog(a.phi, a.pi, p, n)
+            for _ in range(n):
+                lf2.lf2_leapfrog_ex(b.phi, b.pi, p, 1, kernel=lf2.LF2_KERNEL_SITE)
+            got, ref = a.download(), b.download()
+            assert np.array_equal(got[0], ref[0]) and np.array_equal(got[1], ref[1]), n
+        lf2.lf2_field_check(a.phi)
