@@ -459,20 +459,15 @@ lf2_status lf2_leapfrog_ex(lf2_field phi, lf2_field pi, const lf2_params *p, int
     st = (kernel == LF2_KERNEL_TBLOCK) ? ensure_tblock(phi, pi, s) : ensure_dynamic(phi, s);
     if (st != LF2_OK) return st;
 
-    // one-step kernel used for single steps (and for what temporal blocking leaves over)
     const StepArgs probe = step_args(phi, pi, p, p->dt, true);
-    const bool stream_ok = stream_supported(probe, kernel == LF2_KERNEL_STREAM ? tile_y : 0,
-                                            kernel == LF2_KERNEL_STREAM ? zchunk : 0);
-    if (kernel == LF2_KERNEL_STREAM && !stream_ok)
+    if (kernel == LF2_KERNEL_STREAM && !stream_supported(probe, tile_y, zchunk))
         return fail(LF2_ERR_UNSUPPORTED, "streaming kernel does not fit this lattice/config");
-    const bool use_stream = (kernel == LF2_KERNEL_STREAM || kernel == LF2_KERNEL_AUTO || kernel == LF2_KERNEL_TBLOCK) &&
-                            stream_ok;
+    // single steps, and what temporal blocking leaves over
     auto one_step = [&]() -> lf2_status {
         const StepArgs a = step_args(phi, pi, p, p->dt, true);
-        cudaError_t e = use_stream ? launch_stream_step(a, kernel == LF2_KERNEL_STREAM ? tile_y : 0,
-                                                        kernel == LF2_KERNEL_STREAM ? zchunk : 0, 1, s)
+        cudaError_t e = kernel == LF2_KERNEL_STREAM ? launch_stream_step(a, tile_y, zchunk, 1, s)
                         : kernel == LF2_KERNEL_SITE ? launch_site_step(a, s)
-                                                    : launch_general_step(a, s);
+                                                    : launch_default_step(a, s);
         if (e != cudaSuccess) return cuda_fail(e, "leapfrog launch");
         phi->front = 1 - phi->front;
         return LF2_OK;

@@ -156,7 +156,7 @@ lf2_status enqueue_run(lf2_ensemble e, int nsteps, const TbMember *d_members, cu
             a.phi_out = phi->val[1 - fphi];
             a.pi = pi->val[fpi];
             a.comp = phi->comp[fc];
-            cudaError_t err = stream_supported(a, 0, 0) ? launch_stream_step(a, 0, 0, 1, s) : launch_general_step(a, s);
+            cudaError_t err = launch_default_step(a, s);
             if (err != cudaSuccess) return cuda_error(err, "ensemble single step");
             fphi ^= 1;
         }

@@ -32,6 +32,9 @@ cudaError_t launch_general_step(const StepArgs &a, cudaStream_t s);
 bool stream_supported(const StepArgs &a, int tile_y, int zchunk);
 cudaError_t launch_stream_step(const StepArgs &a, int tile_y, int zchunk, int nsteps_hint, cudaStream_t s);
 
+// One step with the kernel that fits the lattice: streaming, else launch_general_step.
+cudaError_t launch_default_step(const StepArgs &a, cudaStream_t s);
+
 // Multiprocessors of the current device (queried once per device, then cached); grid sizes
 // and the temporal-blocking wave model are derived from it.
 int device_sm_count();
