@@ -76,9 +76,18 @@ __host__ __device__ constexpr int stream_nv() {
     return (16 / (int)sizeof(R)) % NC == 0 ? 1 : ((32 / (int)sizeof(R)) % NC == 0 ? 2 : 3);
 }
 
+// Warps per SM that the registers of an FP64 instance are held to (0: the compiler's choice, which
+// is the best for FP32 and for 3 FP64 components).  The integer sums need warps to hide their
+// latency behind: 256^2 x 128, a step, 2 components 158 -> 156 us, 4 components 349 -> 318, 6
+// components 564 -> 492.
+template <int NC, int MODE>
+constexpr int stream_warps() {
+    return MODE != 3 ? 0 : (NC <= 2 ? 32 : (NC == 4 ? 20 : (NC == 6 ? 16 : 0)));
+}
+
 // MODE: 0 = FP32 plain drift, 1 = FP32 Kahan drift, 3 = FP64.
 template <typename R, int NC, int MODE, int BY, typename CoefT>
-__global__ void __launch_bounds__(32 * BY) k_stream(const R *__restrict__ phi, R *__restrict__ phi_out,
+__global__ void __launch_bounds__(32 * BY, (stream_warps<NC, MODE>() / BY)) k_stream(const R *__restrict__ phi, R *__restrict__ phi_out,
                                                     R *__restrict__ pi, float *__restrict__ comp, Geom g, CoefT k,
                                                     int zchunk) {
     constexpr int NV = stream_nv<R, NC>();
