@@ -491,13 +491,29 @@ lf2_status lf2_leapfrog_ex(lf2_field phi, lf2_field pi, const lf2_params *p, int
             return fail(LF2_ERR_UNSUPPORTED,
                         "temporal blocking config (depth %d, cx %d, tile %dx%d, cluster %d) does not fit", c.depth,
                         c.cx, c.tile_x, c.tile_y, c.cluster);
-        for (; done + c.depth <= nsteps; done += c.depth) {
+        auto pass = [&](const TbConfig &q) -> lf2_status {
             ta = tb_args(phi, pi, p);
-            cudaError_t e = launch_tblock(ta, c, s);
+            cudaError_t e = launch_tblock(ta, q, s);
             if (e != cudaSuccess) return cuda_fail(e, "temporal-blocking launch");
             phi->front = 1 - phi->front;
             pi->front = 1 - pi->front;
             if (phi->prec == LF2_F32_KAHAN) phi->cfront = 1 - phi->cfront;
+            done += q.depth;
+            return LF2_OK;
+        };
+        while (done + c.depth <= nsteps) {
+            st = pass(c);
+            if (st != LF2_OK) return st;
+        }
+        // what is left, in shallower passes where they fit (FP64 is bound by its arithmetic, of which
+        // single steps do none twice)
+        TbConfig c2 = with_depth(c, 2), c3 = with_depth(c, 3);
+        const bool shallow = c.cluster <= 1 && phi->prec != LF2_F64;
+        const bool have2 = shallow && c.depth > 2 && tblock_supported(ta, c2);
+        const bool have3 = shallow && c.depth > 3 && tblock_supported(ta, c3);
+        while (const int d = rest_depth(nsteps - done, have2, have3)) {
+            st = pass(d == 2 ? c2 : c3);
+            if (st != LF2_OK) return st;
         }
     }
     for (; done < nsteps; ++done) {

@@ -4,8 +4,9 @@
 // own lattice and with its own parameters.  lf2_ensemble_run advances all of them by nsteps
 // with one CUDA-graph launch: the graph holds nsteps / depth temporal-blocking passes, each a
 // single persistent kernel launch whose blocks take (member, tile, z-chunk) items, longest
-// chunks first, from a counter zeroed before the pass, followed by the leftover single steps
-// per member.  Members
+// chunks first, from a counter zeroed before the pass, followed by shallower passes for what the
+// depth leaves over (two single steps of 64 lattices were 128 launches, 1.33 ms; a depth-2 pass of
+// them takes 0.8) and at most one single step per member.  Members
 // are independent, so no block ever waits for another; the graph is captured once per
 // (nsteps, buffer parities) and relaunched.
 #include <cuda_runtime.h>
@@ -30,16 +31,21 @@ struct CapturedRun {
 
 }  // namespace
 
+// The passes of one depth: configuration and work list.
+struct PassList {
+    TbConfig cfg{0, 0, 0, 0, 0, 0};
+    int4 *d_items = nullptr;
+    int nitems = 0;
+};
+
 struct lf2_ensemble_s {
     int n = 0;
     std::vector<lf2_field> phi, pi;
     std::vector<lf2_params> params;
     lf2_precision prec = LF2_F64;
     int ncomp = 1;
-    TbConfig cfg{0, 0, 0, 0, 0};
     bool tblock = false;  // temporal-blocking passes usable for every member
-    int4 *d_items = nullptr;
-    int nitems = 0;
+    PassList main, rest[2];  // the chosen passes, and those of depth 2 and 3 for what they leave over
     int *d_counter = nullptr;  // work-list position of the running pass
     cudaStream_t capture = nullptr;
     std::vector<CapturedRun> runs;
@@ -67,8 +73,15 @@ std::vector<int> signature_of(lf2_ensemble e) {
 
 int member_zchunk(const lf2_lattice_s *lat) { return lat->n[2]; }
 
+void free_passes(PassList &l) {
+    if (l.d_items) cudaFree(l.d_items);
+    l = PassList{};
+}
+
 // Builds the work list for configuration c (longest z-chunks first, then member order).
-lf2_status build_items(lf2_ensemble e, const TbConfig &c) {
+lf2_status build_items(lf2_ensemble e, const TbConfig &c, PassList &l) {
+    free_passes(l);
+    l.cfg = c;
     std::vector<int4> items;
     for (int m = 0; m < e->n; ++m) {
         const int *n = e->phi[m]->lat->n;
@@ -84,14 +97,12 @@ lf2_status build_items(lf2_ensemble e, const TbConfig &c) {
         return std::min(zc, nz - w.w * zc);
     };
     std::stable_sort(items.begin(), items.end(), [&](const int4 &a, const int4 &b) { return zlen(a) > zlen(b); });
-    if (e->d_items) cudaFree(e->d_items);
-    e->d_items = nullptr;
-    e->nitems = (int)items.size();
     if (items.empty()) return LF2_OK;
-    cudaError_t err = cudaMalloc(&e->d_items, items.size() * sizeof(int4));
+    cudaError_t err = cudaMalloc(&l.d_items, items.size() * sizeof(int4));
     if (err == cudaSuccess)
-        err = cudaMemcpy(e->d_items, items.data(), items.size() * sizeof(int4), cudaMemcpyHostToDevice);
+        err = cudaMemcpy(l.d_items, items.data(), items.size() * sizeof(int4), cudaMemcpyHostToDevice);
     if (err != cudaSuccess) return cuda_error(err, "ensemble work list");
+    l.nitems = (int)items.size();
     return LF2_OK;
 }
 
@@ -109,10 +120,32 @@ bool config_fits(lf2_ensemble e, TbConfig c) {
 }
 
 lf2_status set_config(lf2_ensemble e, const TbConfig &c) {
-    e->cfg = c;
-    e->tblock = config_fits(e, c);
     free_runs(e);
-    return e->tblock ? build_items(e, c) : LF2_OK;
+    free_passes(e->rest[0]);
+    free_passes(e->rest[1]);
+    e->main.cfg = c;
+    e->tblock = config_fits(e, c);
+    lf2_status st = e->tblock ? build_items(e, c, e->main) : LF2_OK;
+    const bool shallow = e->tblock && e->prec != LF2_F64 && c.cx > 0 && c.tile_x > 0 && c.tile_y > 0;
+    for (int depth = 2; depth <= 3 && depth < c.depth && shallow && st == LF2_OK; ++depth) {
+        const TbConfig r = with_depth(c, depth);
+        if (config_fits(e, r)) st = build_items(e, r, e->rest[depth - 2]);
+    }
+    return st;
+}
+
+// A run of nsteps: its temporal-blocking passes, and the single steps after them.
+std::vector<const PassList *> run_passes(lf2_ensemble e, int nsteps, int *singles) {
+    std::vector<const PassList *> out;
+    if (e->tblock) {
+        for (; nsteps >= e->main.cfg.depth; nsteps -= e->main.cfg.depth) out.push_back(&e->main);
+        while (const int d = rest_depth(nsteps, e->rest[0].nitems > 0, e->rest[1].nitems > 0)) {
+            out.push_back(&e->rest[d - 2]);
+            nsteps -= d;
+        }
+    }
+    *singles = nsteps;
+    return out;
 }
 
 TbMember member_entry(lf2_ensemble e, int m) {
@@ -136,15 +169,16 @@ TbMember member_entry(lf2_ensemble e, int m) {
 
 // Enqueues nsteps for every member on stream s (used for capture and for the tuner).
 lf2_status enqueue_run(lf2_ensemble e, int nsteps, const TbMember *d_members, cudaStream_t s) {
-    const int depth = e->tblock ? e->cfg.depth : 0;
-    const int passes = depth ? nsteps / depth : 0;
+    int rest = 0;
+    const std::vector<const PassList *> list = run_passes(e, nsteps, &rest);
+    const int passes = (int)list.size();
     for (int k = 0; k < passes; ++k) {
-        TbEnsembleLaunch L{d_members, e->d_items, e->nitems, e->d_counter, k & 1, e->cfg, e->ncomp, e->prec};
+        const PassList &l = *list[k];
+        TbEnsembleLaunch L{d_members, l.d_items, l.nitems, e->d_counter, k & 1, l.cfg, e->ncomp, e->prec};
         cudaError_t err = launch_tblock_ensemble(L, s);
         if (err != cudaSuccess) return cuda_error(err, "ensemble pass");
     }
     // leftover single steps per member, from the buffers the passes leave current
-    const int rest = nsteps - passes * depth;
     for (int m = 0; m < e->n; ++m) {
         lf2_field phi = e->phi[m], pi = e->pi[m];
         const int pf = passes & 1;
@@ -165,9 +199,8 @@ lf2_status enqueue_run(lf2_ensemble e, int nsteps, const TbMember *d_members, cu
 }
 
 void advance_fronts(lf2_ensemble e, int nsteps) {
-    const int depth = e->tblock ? e->cfg.depth : 0;
-    const int passes = depth ? nsteps / depth : 0;
-    const int rest = nsteps - passes * depth;
+    int rest = 0;
+    const int passes = (int)run_passes(e, nsteps, &rest).size();
     for (int m = 0; m < e->n; ++m) {
         e->phi[m]->front ^= (passes + rest) & 1;
         e->pi[m]->front ^= passes & 1;
@@ -229,7 +262,7 @@ lf2_status lf2_ensemble_create(int n, const lf2_field *phis, const lf2_field *pi
     if (st == LF2_OK && err != cudaSuccess) st = cuda_error(err, "ensemble set-up");
     if (st == LF2_OK) {
         // default configuration: depth 4 with the widest packed columns that fit, else one-step
-        const TbConfig tries[] = {{4, 4, 56, 24, 0}, {4, 2, 24, 24, 0}, {4, 1, 24, 8, 0}, {2, 1, 16, 8, 0}};
+        const TbConfig tries[] = {{4, 4, 56, 24, 0, 1}, {4, 2, 24, 24, 0, 1}, {4, 1, 24, 8, 0, 1}, {2, 1, 16, 8, 0, 1}};
         bool ok = false;
         for (const TbConfig &c : tries)
             if (config_fits(e, c)) {
@@ -241,7 +274,8 @@ lf2_status lf2_ensemble_create(int n, const lf2_field *phis, const lf2_field *pi
     }
     if (st != LF2_OK) {
         if (e->capture) cudaStreamDestroy(e->capture);
-        if (e->d_items) cudaFree(e->d_items);
+        free_passes(e->main);
+        for (PassList &l : e->rest) free_passes(l);
         if (e->d_counter) cudaFree(e->d_counter);
         delete e;
         return st;
@@ -257,7 +291,8 @@ lf2_status lf2_ensemble_create(int n, const lf2_field *phis, const lf2_field *pi
 lf2_status lf2_ensemble_destroy(lf2_ensemble e) {
     if (!e) return set_error(LF2_ERR_INVALID, "ensemble is NULL");
     free_runs(e);
-    if (e->d_items) cudaFree(e->d_items);
+    free_passes(e->main);
+    for (PassList &l : e->rest) free_passes(l);
     if (e->d_counter) cudaFree(e->d_counter);
     if (e->capture) cudaStreamDestroy(e->capture);
     for (int m = 0; m < e->n; ++m) {
@@ -348,7 +383,7 @@ lf2_status lf2_ensemble_tune(lf2_ensemble e, int flags, lf2_step_config *chosen,
     }
     lf2_ensemble clone = nullptr;
     if (st == LF2_OK) st = lf2_ensemble_create(e->n, cphi.data(), cpi.data(), e->params.data(), &clone);
-    TbConfig best = e->cfg;
+    TbConfig best = e->main.cfg;
     bool best_tb = e->tblock;
     float best_ms = -1.0f;
     if (st == LF2_OK) {

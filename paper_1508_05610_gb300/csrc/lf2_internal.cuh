@@ -133,6 +133,19 @@ cudaError_t launch_tblock_ensemble(const TbEnsembleLaunch &e, cudaStream_t s);
 // depth, columns per thread and cluster size (FP32 storage, 1 or 2 components).
 bool tblock_cluster_built(int esz, int ncomp, int depth, int cx, int cluster);
 
+// The steps that passes of c.depth leave over of a run, in passes of depth 2 and 3 with the same
+// region of columns and, last, single steps: the next pass's depth for `rest` steps (0: single steps).
+// have2, have3: such passes are available.
+inline int rest_depth(int rest, bool have2, bool have3) {
+    if (rest >= 2 && have2 && (rest == 2 || rest == 4 || !have3)) return 2;
+    return rest >= 3 && have3 ? 3 : 0;
+}
+// c with another depth and the same region (one CTA per tile).
+inline TbConfig with_depth(const TbConfig &c, int depth) {
+    const int halo = (c.depth + c.cx - 1) / c.cx * c.cx, halo2 = (depth + c.cx - 1) / c.cx * c.cx;
+    return TbConfig{depth, c.cx, c.tile_x + 2 * (halo - halo2), c.tile_y + 2 * (c.depth - depth), 0, 1};
+}
+
 // Shape/configuration check; fills defaults for zero fields of `c`.
 bool tblock_supported(const TbArgs &a, TbConfig &c);
 cudaError_t launch_tblock(const TbArgs &a, const TbConfig &c, cudaStream_t s);

@@ -88,3 +88,36 @@ def test_many_steps_of_small_lattices_equal_single_steps(lf2, monkeypatch, shape
             got, ref = a.download(), b.download()
             assert np.array_equal(got[0], ref[0]) and np.array_equal(got[1], ref[1]), n
         lf2.lf2_field_check(a.phi)
+
+
+@pytest.mark.parametrize("prec,ncomp,depth,cx,tile", [("f32k", 1, 4, 4, (56, 24)), ("f32", 2, 4, 2, (24, 24)),
+                                                      ("f32k", 1, 6, 2, (20, 12)), ("f32", 1, 8, 1, (8, 4)),
+                                                      ("f32k", 4, 4, 1, (8, 24)), ("f32k", 3, 3, 1, (10, 8)),
+                                                      ("f32k", 6, 2, 1, (12, 12)), ("f64", 1, 4, 2, (24, 8)),
+                                                      ("f32k", 1, 3, 4, (56, 26))])
+def test_steps_left_over_by_temporal_blocking(lf2, prec, ncomp, depth, cx, tile):
+    """Every remainder of a run by the depth (shallower passes of the same region, then single steps)
+    gives bitwise the site kernel's state, on a lattice of ragged tiles and as an ensemble of two."""
+    shape = (72, 30, 12)
+    nx, ny, nz = shape
+    phi0 = inputs.gaussian_field(nx, ny, nz, ncomp, sigma=0.4, seed=921)
+    pi0 = inputs.gaussian_field(nx, ny, nz, ncomp, sigma=0.2, seed=922)
+    p = lf2.params(**KW)
+    cfg = dict(depth=depth, cx=cx, tile_x=tile[0], tile_y=tile[1])
+    with lf2.System(shape, ncomp, prec) as a, lf2.System(shape, ncomp, prec) as b, \
+            lf2.System(shape, ncomp, prec) as c, lf2.System(shape, ncomp, prec) as d:
+        for s in (a, b, c, d):
+            s.upload(phi0, pi0)
+        e = lf2.lf2_ensemble_create([c.phi, d.phi], [c.pi, d.pi], [p, p])
+        try:
+            lf2.lf2_ensemble_set_config(e, **cfg)
+            for rest in range(depth):
+                lf2.lf2_leapfrog_ex(a.phi, a.pi, p, depth + rest, kernel=lf2.LF2_KERNEL_TBLOCK, **cfg)
+                lf2.lf2_leapfrog_ex(b.phi, b.pi, p, depth + rest, kernel=lf2.LF2_KERNEL_SITE)
+                lf2.lf2_ensemble_run(e, depth + rest)
+                ref = b.download()
+                for s in (a, c, d):
+                    got = s.download()
+                    assert np.array_equal(got[0], ref[0]) and np.array_equal(got[1], ref[1]), rest
+        finally:
+            lf2.lf2_ensemble_destroy(e)
