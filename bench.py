@@ -50,9 +50,10 @@ WORKLOAD = ("phi4 complex {n}^3 periodic lattice, dt=0.05, lambda=eta=1, sigma=0
 # Kahan compensation read + write
 BYTES_PER_SITE = {"f64": 8 * NCOMP * 4, "f32k": 4 * NCOMP * 6, "f32": 4 * NCOMP * 4}
 FALLBACK_HBM_GBS = 6800.0
-# The FP64 step issues 10 DP instructions per real site and 19 per complex site (the folded
-# update of lf2_arith.cuh); the FP64 pipe issues 2 DFMA per SM per clock.
-DP_INSTR_PER_SITE = {1: 10, 2: 19}
+# The FP64 step issues 5 DP instructions per real site and 9 per complex site (the folded update of
+# lf2_arith.cuh; the neighbour sums run on the integer pipes); the FP64 pipe issues 2 DFMA per SM
+# per clock.
+DP_INSTR_PER_SITE = {1: 5, 2: 9}
 ERROR_STEP = 50        # error against FP64 and energy drift are taken at this step
 ENERGY_EVERY = 10
 TIMED_REGIONS = 5      # the headline is the median of this many timed regions
@@ -218,12 +219,29 @@ class WrappedPair:
         return keep
 
 
+def rest_launches(rest, depth, cfg):
+    """Launches of lf2_leapfrog_ex for the steps that FP32 passes of `depth` leave over: the rule of
+    rest_depth in lf2_internal.cuh, passes of one CTA per tile."""
+    launches = 0
+    shallow = (cfg.get("cluster") or 1) <= 1
+    while rest:
+        if rest >= 2 and shallow and depth > 2 and (rest in (2, 4) or depth <= 3):
+            rest -= 2
+        elif rest >= 3 and shallow and depth > 3:
+            rest -= 3
+        else:
+            rest -= 1
+        launches += 1
+    return launches
+
+
 def time_regions(torch, lf2, pair, p, steps, warmup, stream, cfg, regions):
     """Half-kick, `warmup` untimed steps, then `regions` timed regions of EXACTLY `steps` leapfrog
     steps, each between CUDA events on the launch stream with a synchronisation on both sides.
     A step pass is one launch (`depth` steps under temporal blocking, one otherwise); remainder
-    steps run as single-step launches.  Each pass launch is also bracketed by its own events, so
-    the dominant kernel's average launch duration is measured live.  Returns (region seconds,
+    steps run in passes of depth 3 and 2 and single steps (rest_launches).  Each pass launch is also
+    bracketed by its own events, so the dominant kernel's average launch duration is measured live.
+    Returns (region seconds,
     average seconds of one full pass, passes per region, launches per region)."""
     lf2.lf2_leapfrog_init(pair.fphi, pair.fpi, p, stream)
     depth = cfg.get("depth", 0) if cfg.get("kernel") == lf2.LF2_KERNEL_TBLOCK else 1
@@ -251,7 +269,7 @@ def time_regions(torch, lf2, pair, p, steps, warmup, stream, cfg, regions):
         times.append(start.elapsed_time(stop) / 1e3)
     per_pass = statistics.mean(a.elapsed_time(b) / 1e3 for a, b in pass_events) if pass_events else None
     passes = steps // depth
-    return times, per_pass, passes, passes + steps % depth
+    return times, per_pass, passes, passes + rest_launches(steps % depth, depth, cfg)
 
 
 def error_block(torch, lf2, inputs, n, p, plan32, stream, seed):
