@@ -101,7 +101,10 @@ lf2_status build_items(lf2_ensemble e, const TbConfig &c, PassList &l) {
     cudaError_t err = cudaMalloc(&l.d_items, items.size() * sizeof(int4));
     if (err == cudaSuccess)
         err = cudaMemcpy(l.d_items, items.data(), items.size() * sizeof(int4), cudaMemcpyHostToDevice);
-    if (err != cudaSuccess) return cuda_error(err, "ensemble work list");
+    if (err != cudaSuccess) {
+        free_passes(l);
+        return cuda_error(err, "ensemble work list");
+    }
     l.nitems = (int)items.size();
     return LF2_OK;
 }
@@ -125,27 +128,34 @@ lf2_status set_config(lf2_ensemble e, const TbConfig &c) {
     free_passes(e->rest[1]);
     e->main.cfg = c;
     e->tblock = config_fits(e, c);
-    lf2_status st = e->tblock ? build_items(e, c, e->main) : LF2_OK;
+    const lf2_status st = e->tblock ? build_items(e, c, e->main) : LF2_OK;
+    if (st != LF2_OK) e->tblock = false;  // no work list: the members step one by one
     const bool shallow = e->tblock && e->prec != LF2_F64 && c.cx > 0 && c.tile_x > 0 && c.tile_y > 0;
-    for (int depth = 2; depth <= 3 && depth < c.depth && shallow && st == LF2_OK; ++depth) {
+    for (int depth = 2; depth <= 3 && depth < c.depth && shallow; ++depth) {
         const TbConfig r = with_depth(c, depth);
-        if (config_fits(e, r)) st = build_items(e, r, e->rest[depth - 2]);
+        // without memory for its list the steps it would take are single ones
+        if (config_fits(e, r)) (void)build_items(e, r, e->rest[depth - 2]);
     }
     return st;
 }
 
-// A run of nsteps: its temporal-blocking passes, and the single steps after them.
-std::vector<const PassList *> run_passes(lf2_ensemble e, int nsteps, int *singles) {
-    std::vector<const PassList *> out;
+// The temporal-blocking passes of a run of nsteps in order, pass(index, list) for each until one fails;
+// then the passes' number, and the single steps after them.
+template <typename F>
+lf2_status run_passes(lf2_ensemble e, int nsteps, int *passes, int *singles, F pass) {
+    lf2_status st = LF2_OK;
+    *passes = 0;
     if (e->tblock) {
-        for (; nsteps >= e->main.cfg.depth; nsteps -= e->main.cfg.depth) out.push_back(&e->main);
-        while (const int d = rest_depth(nsteps, e->rest[0].nitems > 0, e->rest[1].nitems > 0)) {
-            out.push_back(&e->rest[d - 2]);
+        for (; nsteps >= e->main.cfg.depth && st == LF2_OK; nsteps -= e->main.cfg.depth) st = pass((*passes)++, e->main);
+        while (st == LF2_OK) {
+            const int d = rest_depth(nsteps, e->rest[0].nitems > 0, e->rest[1].nitems > 0);
+            if (!d) break;
+            st = pass((*passes)++, e->rest[d - 2]);
             nsteps -= d;
         }
     }
     *singles = nsteps;
-    return out;
+    return st;
 }
 
 TbMember member_entry(lf2_ensemble e, int m) {
@@ -169,15 +179,13 @@ TbMember member_entry(lf2_ensemble e, int m) {
 
 // Enqueues nsteps for every member on stream s (used for capture and for the tuner).
 lf2_status enqueue_run(lf2_ensemble e, int nsteps, const TbMember *d_members, cudaStream_t s) {
-    int rest = 0;
-    const std::vector<const PassList *> list = run_passes(e, nsteps, &rest);
-    const int passes = (int)list.size();
-    for (int k = 0; k < passes; ++k) {
-        const PassList &l = *list[k];
+    int passes = 0, rest = 0;
+    const lf2_status st = run_passes(e, nsteps, &passes, &rest, [&](int k, const PassList &l) {
         TbEnsembleLaunch L{d_members, l.d_items, l.nitems, e->d_counter, k & 1, l.cfg, e->ncomp, e->prec};
         cudaError_t err = launch_tblock_ensemble(L, s);
-        if (err != cudaSuccess) return cuda_error(err, "ensemble pass");
-    }
+        return err == cudaSuccess ? LF2_OK : cuda_error(err, "ensemble pass");
+    });
+    if (st != LF2_OK) return st;
     // leftover single steps per member, from the buffers the passes leave current
     for (int m = 0; m < e->n; ++m) {
         lf2_field phi = e->phi[m], pi = e->pi[m];
@@ -199,8 +207,8 @@ lf2_status enqueue_run(lf2_ensemble e, int nsteps, const TbMember *d_members, cu
 }
 
 void advance_fronts(lf2_ensemble e, int nsteps) {
-    int rest = 0;
-    const int passes = (int)run_passes(e, nsteps, &rest).size();
+    int passes = 0, rest = 0;
+    (void)run_passes(e, nsteps, &passes, &rest, [](int, const PassList &) { return LF2_OK; });
     for (int m = 0; m < e->n; ++m) {
         e->phi[m]->front ^= (passes + rest) & 1;
         e->pi[m]->front ^= passes & 1;
