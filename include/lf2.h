@@ -97,7 +97,8 @@ typedef enum {
     LF2_KERNEL_AUTO = 0,     /* tuned choice (the one lf2_leapfrog uses) */
     LF2_KERNEL_SITE = 1,     /* one thread per site, any lattice shape */
     LF2_KERNEL_STREAM = 2,   /* x-y tile streaming along z, one step per pass */
-    LF2_KERNEL_TBLOCK = 3    /* temporal blocking: `depth` steps per pass */
+    LF2_KERNEL_TBLOCK = 3    /* temporal blocking: `depth` steps per pass; FP32 steps left over in
+                              * passes of depth 3 and 2 of the same region, then one by one */
 } lf2_kernel;
 
 typedef struct {
@@ -272,9 +273,9 @@ lf2_status lf2_energy_device(lf2_field phi, lf2_field pi, const lf2_params *p, d
  * either way.  A barrier that does not complete within about a second (all blocks of a
  * cooperative launch are resident, so it always completes) ends the run and leaves NaN in the
  * records from the step before that barrier on (a step's record is finished during the next
- * step); lf2_field_check(phi) then returns LF2_ERR_TIMEOUT.  Enqueues on `stream` without waiting; after the first call on phi (which may
- * allocate its back buffer and energy scratch, so make it outside a stream capture) calls
- * allocate nothing and can be captured into a CUDA graph.  Calls on one phi share its energy
+ * step); lf2_field_check(phi) then returns LF2_ERR_TIMEOUT.  Enqueues on `stream` without waiting;
+ * after the first call on phi (which may allocate its back buffer and energy scratch, so make it
+ * outside a stream capture) calls allocate nothing and can be captured into a CUDA graph.  Calls on one phi share its energy
  * scratch with lf2_energy and lf2_energy_device: order them on one stream.
  * LF2_ERR_INVALID for nsteps < 0 or dev_records NULL with nsteps > 0. */
 lf2_status lf2_leapfrog_energy(lf2_field phi, lf2_field pi, const lf2_params *p, int nsteps, double *dev_records,
@@ -293,9 +294,9 @@ lf2_status lf2_leapfrog_energy(lf2_field phi, lf2_field pi, const lf2_params *p,
 lf2_status lf2_field_compare(lf2_field f, int which, const void *ref, lf2_precision ref_prec, double *out,
                              void *stream);
 
-/* Status of the last multi-step lf2_leapfrog_energy or lf2_leapfrog run on phi: LF2_ERR_TIMEOUT (once; the
- * flag is then cleared) if one of its grid barriers gave up, else LF2_OK.  The paper has no
- * counterpart (its programs have no device-side waits).  Synchronises `stream`.  Host-side
+/* Status of the last multi-step lf2_leapfrog_energy or lf2_leapfrog run on phi: LF2_ERR_TIMEOUT
+ * (once; the flag is then cleared) if one of its grid barriers gave up, else LF2_OK.  The paper has
+ * no counterpart (its programs have no device-side waits).  Synchronises `stream`.  Host-side
  * failure injection for tests: with LF2_FAULT=timeout in the environment the barrier waits give
  * up at once; with LF2_FAULT=launch, lf2_leapfrog and lf2_leapfrog_energy return LF2_ERR_CUDA
  * without launching; with LF2_FAULT=alloc, the library's allocations fail with LF2_ERR_NOMEM. */
@@ -340,7 +341,7 @@ lf2_status lf2_ensemble_create(int n, const lf2_field *phis, const lf2_field *pi
 /* Advances every member by nsteps (each member's phi_n / pi_{n-1/2} convention as in
  * lf2_leapfrog) with ONE CUDA-graph launch on `stream`: nsteps/depth temporal-blocking passes,
  * each a persistent kernel over a work list of (member, tile, z-chunk) items ordered longest
- * first, then the leftover single steps.  The graph is captured on first use for a given
+ * first, then passes of depth 3 and 2 and single steps for what is left.  The graph is captured on first use for a given
  * nsteps and buffer state (this first call must not itself be inside a stream capture) and
  * relaunched afterwards.  Results are bitwise those of running each member alone. */
 lf2_status lf2_ensemble_run(lf2_ensemble e, int nsteps, void *stream);

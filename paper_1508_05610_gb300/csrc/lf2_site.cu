@@ -1,7 +1,8 @@
-// lf2_site.cu -- one thread per site: the shape-agnostic leapfrog kernel (any Nx, Ny, Nz),
-// plus the precision conversions used by upload/download.
+// lf2_site.cu -- the shape-agnostic leapfrog kernels (any Nx, Ny, Nz): one thread per site, and a
+// column walk for real FP32 fields; the first derivative; the precision conversions used by
+// upload/download.
 //
-// Each thread owns one site (x, y, z) of the row-major lattice and reads its six periodic
+// In the per-site kernel each thread owns one site (x, y, z) of the row-major lattice and reads its six periodic
 // neighbours x+-i (the Site jumps of Sec. 3.4 with the torus wrap of Sec. 3.3.1 done by
 // index arithmetic instead of a stored halo).
 #include <atomic>
@@ -58,8 +59,8 @@ __device__ __forceinline__ void load_at(const R *__restrict__ p, R (&v)[NC]) {
     }
 }
 // Data the kernel also writes.  FP64 by L2 loads, which may be issued ahead of earlier stores (the
-// punned pointers lose __restrict__; 257x193x161 complex FP64: 1.96 against 1.46 times the start);
-// FP32 by plain ones, since the chunks of a site share L1 lines (5 components 1.7 against 1.55).
+// punned pointers lose __restrict__; 257x193x161 complex FP64 runs 1.34 times as fast with them);
+// FP32 by plain ones, since the chunks of a site share L1 lines (5 components: 1.1 times as fast).
 template <typename R, int NC>
 __device__ __forceinline__ void load_own(const R *p, R (&v)[NC]) {
     using C = SiteChunks<R, NC>;

@@ -9,8 +9,8 @@
 // shuffle, with only the two edge lanes of a warp reading one site from global memory.
 // Periodic wrap (the torus of Sec. 3.3.1) is index arithmetic on plane, row and column.
 //
-// Requirements (else the one-thread-per-site kernel runs): rows of 16-byte multiples
-// (Nx * ncomp * sizeof(R) % 16 == 0) and Ny a multiple of the tile height.
+// Requirements (else the kernels for any shape run, launch_general_step): rows of 16-byte multiples
+// (Nx * ncomp * sizeof(R) % 16 == 0) and Ny a multiple of the tile height, two by default.
 #include "lf2_bounds.cuh"
 #include "lf2_internal.cuh"
 

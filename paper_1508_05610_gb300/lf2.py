@@ -239,14 +239,14 @@ def lf2_energy_device(phi, pi, p: lf2_params, dev_out_ptr, stream=None):
 
 
 def lf2_leapfrog_energy(phi, pi, p: lf2_params, nsteps, dev_records_ptr, stream=None):
-    """nsteps leapfrog steps, one kernel each, that also write the energy record of the state at
-    the start of every step (nsteps x 16 doubles of device memory at dev_records_ptr)."""
+    """nsteps leapfrog steps that also write the energy record of the state at the start of every
+    step, in one launch for a small lattice and one launch per step otherwise (nsteps x 16 doubles of device memory at dev_records_ptr)."""
     _call("lf2_leapfrog_energy", phi, pi, ctypes.byref(p), int(nsteps), dev_records_ptr, _stream_ptr(stream))
 
 
 def lf2_field_check(f, stream=None):
     """Raises LF2Error (LF2_ERR_TIMEOUT) if a grid barrier of the last multi-step
-    lf2_leapfrog_energy run on f gave up."""
+    lf2_leapfrog_energy or lf2_leapfrog run on f gave up."""
     _call("lf2_field_check", f, _stream_ptr(stream))
 
 
