@@ -2,8 +2,8 @@
 // column walk for real FP32 fields; the first derivative; the precision conversions used by
 // upload/download.
 //
-// In the per-site kernel each thread owns one site (x, y, z) of the row-major lattice and reads its six periodic
-// neighbours x+-i (the Site jumps of Sec. 3.4 with the torus wrap of Sec. 3.3.1 done by
+// In the per-site kernel each thread owns one site (x, y, z) of the row-major lattice and reads its
+// six periodic neighbours x+-i (the Site jumps of Sec. 3.4 with the torus wrap of Sec. 3.3.1 done by
 // index arithmetic instead of a stored halo).
 #include <atomic>
 #include <type_traits>
@@ -149,14 +149,19 @@ __global__ void __launch_bounds__(kThreads) k_site_f32(const float *__restrict__
 // walks a chunk of z-planes with planes z-1, z, z+1 of its column in registers; the x and y
 // neighbours come from L1 and L2 (threads are numbered along the plane's rows, so a block's rows
 // overlap).  Against k_site it has no index arithmetic per site and loads each column once
-// instead of three times.  FP32+Kahan step, 133x121x112: k_site 12.8 us, k_march 10.7 (14.8 before
+// instead of three times.  FP32+Kahan step, a plane at a time, 133x121x112: k_site 12.8 us, k_march 10.7 (14.8 before
 // k_site's divisions went); 515x77x99: 21.6 and 17.9 us (27.2); 257x193x161: 47.6 and 46.7 (53.8).
 // With 2 or more components k_site is as fast or faster (its vector accesses are aligned along the
 // whole lattice), and in FP64 both wait for the FP64 pipe.
-constexpr int kMarchThreads = 512;
+// Bound by the latency of the loads, so BATCH planes are loaded before the first is computed: two
+// with the compensated drift, 257x193x161 45.4 -> 41.3 us, 521x509x301 385 -> 365, 515x77x99 17.3 ->
+// 16.6 (in blocks of 512: 42.5, 371, 16.6; four planes: 52, 516, 20, too few warps for their
+// registers), and chunks of at least two: 67x65x61 6.0 -> 4.1 us.  One with the plain drift, which has
+// fewer loads (two: 26.5 -> 30 us at 257x193x161).
+constexpr int kMarchThreads = 256;
 constexpr int kMarchPlanes = 8;  // per chunk: two planes more to load than to compute; 4 to 32 within 5 %
 
-template <bool KAHAN>
+template <bool KAHAN, int BATCH>
 __global__ void __launch_bounds__(kMarchThreads) k_march(const float *__restrict__ phi, float *__restrict__ phi_out,
                                                          float *__restrict__ pi, float *__restrict__ comp, Geom g,
                                                          Coef32 k, int zchunk) {
@@ -169,17 +174,33 @@ __global__ void __launch_bounds__(kMarchThreads) k_march(const float *__restrict
     const int z0 = blockIdx.y * zchunk, z1 = min(z0 + zchunk, g.nz);
     auto load = [&](long long at) { return __ldg(phi + checked(at, 1, g.sites)); };
     float below[1] = {load((long long)wrap_dn(z0, g.nz) * plane + i)}, cur[1] = {load((long long)z0 * plane + i)};
-    for (int z = z0; z < z1; ++z) {
-        const long long pz = (long long)z * plane, at = checked(pz + i, 1, g.sites);
-        float above[1] = {load((long long)wrap_up(z, g.nz) * plane + i)}, out[1];
-        float xm[1] = {load(pz + ixm)}, xp[1] = {load(pz + ixp)}, ym[1] = {load(pz + iym)}, yp[1] = {load(pz + iyp)};
-        float p[1] = {pi[at]}, cm[1] = {KAHAN ? comp[at] : 0.0f};
-        update_f32<1, KAHAN>(cur, xm, xp, ym, yp, below, above, p, cm, out, k);
-        pi[at] = p[0];
-        phi_out[at] = out[0];
-        if (KAHAN) comp[at] = cm[0];
-        below[0] = cur[0];
-        cur[0] = above[0];
+    for (int z = z0; z < z1; z += BATCH) {
+        float next[BATCH], xm[BATCH][1], xp[BATCH][1], ym[BATCH][1], yp[BATCH][1], p[BATCH][1], cm[BATCH][1];
+        long long at[BATCH];
+#pragma unroll
+        for (int b = 0; b < BATCH; ++b) {
+            const int zb = min(z + b, z1 - 1);  // past the chunk: its last plane again, not used
+            const long long pz = (long long)zb * plane;
+            at[b] = checked(pz + i, 1, g.sites);
+            next[b] = load((long long)wrap_up(zb, g.nz) * plane + i);
+            xm[b][0] = load(pz + ixm);
+            xp[b][0] = load(pz + ixp);
+            ym[b][0] = load(pz + iym);
+            yp[b][0] = load(pz + iyp);
+            p[b][0] = pi[at[b]];
+            cm[b][0] = KAHAN ? comp[at[b]] : 0.0f;
+        }
+#pragma unroll
+        for (int b = 0; b < BATCH; ++b) {
+            if (z + b >= z1) break;
+            float above[1] = {next[b]}, out[1];
+            update_f32<1, KAHAN>(cur, xm[b], xp[b], ym[b], yp[b], below, above, p[b], cm[b], out, k);
+            pi[at[b]] = p[b][0];
+            phi_out[at[b]] = out[0];
+            if (KAHAN) comp[at[b]] = cm[b][0];
+            below[0] = cur[0];
+            cur[0] = above[0];
+        }
     }
 }
 
@@ -241,21 +262,22 @@ cudaError_t launch_site_step(const StepArgs &a, cudaStream_t s) {
 
 cudaError_t launch_general_step(const StepArgs &a, cudaStream_t s) {
     const long long plane = (long long)a.g.nx * a.g.ny, bx = (plane + kMarchThreads - 1) / kMarchThreads;
-    // chunks as long as they leave four blocks per SM, and 16-bit grid and 32-bit plane indices
+    // chunks as long as they leave eight blocks per SM, and 16-bit grid and 32-bit plane indices
+    const bool kahan = a.prec == LF2_F32_KAHAN;
     int zchunk = kMarchPlanes;
-    while (zchunk > 1 && bx * ((a.g.nz + zchunk - 1) / zchunk) < 4LL * device_sm_count()) zchunk /= 2;
+    while (zchunk > (kahan ? 2 : 1) && bx * ((a.g.nz + zchunk - 1) / zchunk) < 8LL * device_sm_count()) zchunk /= 2;
     const long long bz = (a.g.nz + zchunk - 1) / zchunk;
     if (a.g.sites == 0 || a.prec == LF2_F64 || a.ncomp != 1 || !a.drift || plane + kMarchThreads >= (1LL << 31) ||
         bz > 65535)
         return launch_site_step(a, s);
     const dim3 grid((unsigned)bx, (unsigned)bz);
     const Coef32 k = make_coef32(a.p, a.dt);
-    if (a.prec == LF2_F32_KAHAN)
-        k_march<true><<<grid, kMarchThreads, 0, s>>>((const float *)a.phi, (float *)a.phi_out, (float *)a.pi, a.comp,
-                                                     a.g, k, zchunk);
+    const float *phi = (const float *)a.phi;
+    float *out = (float *)a.phi_out, *pi = (float *)a.pi;
+    if (kahan)
+        k_march<true, 2><<<grid, kMarchThreads, 0, s>>>(phi, out, pi, a.comp, a.g, k, zchunk);
     else
-        k_march<false><<<grid, kMarchThreads, 0, s>>>((const float *)a.phi, (float *)a.phi_out, (float *)a.pi, a.comp,
-                                                      a.g, k, zchunk);
+        k_march<false, 1><<<grid, kMarchThreads, 0, s>>>(phi, out, pi, a.comp, a.g, k, zchunk);
     return cudaGetLastError();
 }
 

@@ -121,3 +121,22 @@ def test_steps_left_over_by_temporal_blocking(lf2, prec, ncomp, depth, cx, tile)
                     assert np.array_equal(got[0], ref[0]) and np.array_equal(got[1], ref[1]), rest
         finally:
             lf2.lf2_ensemble_destroy(e)
+
+
+@pytest.mark.parametrize("prec", ["f32k", "f32"])
+@pytest.mark.parametrize("shape", [(131, 121, 61), (133, 121, 111), (133, 121, 112), (257, 193, 67), (1, 515, 1201)])
+def test_column_walk_over_chunks_of_several_planes(lf2, monkeypatch, shape, prec):
+    """Chunks of 2, 4 and 8 planes, whole and with 1 or 3 planes left in the last one, bitwise the
+    site kernel; three steps, so that the buffers change places."""
+    monkeypatch.setenv("LF2_TUNE", "off")
+    nx, ny, nz = shape
+    phi0 = inputs.gaussian_field(nx, ny, nz, 1, sigma=0.4, seed=931)
+    pi0 = inputs.gaussian_field(nx, ny, nz, 1, sigma=0.2, seed=932)
+    p = lf2.params(**KW)
+    with lf2.System(shape, 1, prec) as a, lf2.System(shape, 1, prec) as b:
+        for s in (a, b):
+            s.upload(phi0, pi0)
+        lf2.lf2_leapfrog(a.phi, a.pi, p, 3)
+        lf2.lf2_leapfrog_ex(b.phi, b.pi, p, 3, kernel=lf2.LF2_KERNEL_SITE)
+        got, ref = a.download(), b.download()
+    assert np.array_equal(got[0], ref[0]) and np.array_equal(got[1], ref[1])
