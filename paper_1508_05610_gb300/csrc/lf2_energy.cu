@@ -425,7 +425,7 @@ __global__ void __launch_bounds__(kEnergyThreads, 2)
             double *__restrict__ scratch, double *__restrict__ records, unsigned polls) {
     constexpr int NS = kNs<NC>;
     __shared__ double sh[ENERGY ? NS : 1][ENERGY ? kEnergyThreads : 1];
-    unsigned *bar = reinterpret_cast<unsigned *>(scratch + kBarrierOffset);
+    unsigned long long *bar = reinterpret_cast<unsigned long long *>(scratch + kBarrierOffset);
     const int nsb = ENERGY ? (int)gridDim.x - 1 : (int)gridDim.x;
     const bool reducer = ENERGY && (int)blockIdx.x == nsb;
     // rows [first, first + count) of the set of `step`, inside the row-set region (checked in
@@ -497,7 +497,7 @@ __global__ void __launch_bounds__(kEnergyThreads, 2)
                 p[a] = pn[a];
             }
         }
-        if (!grid_wait(bar, (unsigned)(step + 1) * gridDim.x, polls)) {
+        if (!grid_wait(bar, (step + 1ull) * gridDim.x, polls)) {
             if constexpr (ENERGY) poison_records(records, step > 0 ? step - 1 : 0, nsteps);
             return;
         }
@@ -675,8 +675,8 @@ cudaError_t launch_cooperative(K kern, int nb, void *barrier, cudaStream_t s, Ar
     if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kEnergyThreads, 0);
     if (e != cudaSuccess) return e;
     if (!coop || (long long)per_sm * sms < nb) return cudaErrorNotSupported;
-    // the barrier's arrival count and error flag start at zero
-    e = cudaMemsetAsync(barrier, 0, 2 * sizeof(unsigned), s);
+    // the barrier's arrival count and flag start at zero
+    e = cudaMemsetAsync(barrier, 0, sizeof(unsigned long long), s);
     if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(nb);
@@ -743,11 +743,11 @@ cudaError_t launch_steps_plain(const StepArgs &a, int nsteps, double *scratch, c
 }
 
 cudaError_t steps_energy_timed_out(double *scratch, bool *out, cudaStream_t s) {
-    unsigned word[2] = {0, 0};  // arrivals, error flag
-    cudaError_t e = cudaMemcpyAsync(word, scratch + kBarrierOffset, sizeof word, cudaMemcpyDeviceToHost, s);
+    unsigned long long word = 0;
+    cudaError_t e = cudaMemcpyAsync(&word, scratch + kBarrierOffset, sizeof word, cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     if (e != cudaSuccess) return e;
-    *out = word[1] != 0u;
+    *out = (word & kBarrierGaveUp) != 0;
     if (*out) {
         e = cudaMemsetAsync(scratch + kBarrierOffset, 0, sizeof word, s);  // reported once
         if (e == cudaSuccess) e = cudaStreamSynchronize(s);
