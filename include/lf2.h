@@ -294,8 +294,9 @@ lf2_status lf2_leapfrog_energy(lf2_field phi, lf2_field pi, const lf2_params *p,
 lf2_status lf2_field_compare(lf2_field f, int which, const void *ref, lf2_precision ref_prec, double *out,
                              void *stream);
 
-/* Status of the last multi-step lf2_leapfrog_energy or lf2_leapfrog run on phi: LF2_ERR_TIMEOUT
- * (once; the flag is then cleared) if one of its grid barriers gave up, else LF2_OK.  The paper has
+/* Status of the multi-step lf2_leapfrog_energy and lf2_leapfrog runs on phi since the last call:
+ * LF2_ERR_TIMEOUT (once; the flag is then cleared) if a grid barrier of any of them gave up, else
+ * LF2_OK.  Later runs neither clear the flag nor stop for it.  The paper has
  * no counterpart (its programs have no device-side waits).  Synchronises `stream`.  Host-side
  * failure injection for tests: with LF2_FAULT=timeout in the environment the barrier waits give
  * up at once; with LF2_FAULT=launch, lf2_leapfrog and lf2_leapfrog_energy return LF2_ERR_CUDA

@@ -147,9 +147,12 @@ lf2_status ensure_energy_scratch(lf2_field f) {
     if (!f->energy_scratch) {
         void *d = nullptr;
         LF2_CUDA(cudaMalloc(&d, sizeof(double) * kFieldScratchDoubles), "cudaMalloc(energy scratch)");
-        // the finished-block counter must start at zero (each reduction leaves it at zero)
-        const double zero = 0.0;
-        cudaError_t e = cudaMemcpy((double *)d + kEnergyCounterOffset, &zero, sizeof zero, cudaMemcpyHostToDevice);
+        // the finished-block counter (each reduction leaves it at zero) and the row with the multi-step
+        // runs' status must start at zero
+        const double zero[kEnergySlots] = {};
+        cudaError_t e = cudaMemcpy((double *)d + kEnergyCounterOffset, zero, sizeof zero[0], cudaMemcpyHostToDevice);
+        if (e == cudaSuccess)
+            e = cudaMemcpy((double *)d + kStepsWordsOffset, zero, sizeof zero, cudaMemcpyHostToDevice);
         if (e != cudaSuccess) {
             cudaFree(d);
             return cuda_fail(e, "energy scratch counter");
@@ -618,8 +621,8 @@ lf2_status lf2_field_check(lf2_field phi, void *stream) {
     LF2_CUDA(steps_energy_timed_out(phi->energy_scratch, &timed_out, (cudaStream_t)stream), "status read");
     if (timed_out)
         return fail(LF2_ERR_TIMEOUT,
-                    "a grid barrier of the last multi-step run gave up: the records of an lf2_leapfrog_energy run "
-                    "from that step on are NaN and the fields are not a valid state");
+                    "a grid barrier of a multi-step run since the last check gave up: the records of an "
+                    "lf2_leapfrog_energy run from that step on are NaN and the fields it left are not a valid state");
     return LF2_OK;
 }
 

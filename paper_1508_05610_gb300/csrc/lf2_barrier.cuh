@@ -11,7 +11,8 @@
 //
 // Waits are bounded: a cooperative launch keeps every block resident, so real waits take
 // microseconds; after kBarrierPolls polls of about half a microsecond (about a second) the waiter sets the
-// flag, every block stops and the host reports it (lf2_field_check).
+// flag, every block stops and the host reports it (lf2_field_check).  The flag goes with the launch's
+// word; a status word beside it, which launches leave alone, keeps the event until it is reported.
 #include <cuda_runtime.h>
 
 namespace lf2 {
@@ -27,7 +28,8 @@ __device__ __forceinline__ void grid_arrive(unsigned long long *bar) {
 }
 
 // False when the wait ran out after polls_max polls, here or in another block.
-__device__ __forceinline__ bool grid_wait(unsigned long long *bar, unsigned long long target, unsigned polls_max) {
+__device__ __forceinline__ bool grid_wait(unsigned long long *bar, unsigned long long *status, unsigned long long target,
+                                          unsigned polls_max) {
     __shared__ int s_ok;
     if (threadIdx.x == 0) {
         int ok = 1;
@@ -42,6 +44,7 @@ __device__ __forceinline__ bool grid_wait(unsigned long long *bar, unsigned long
             if (v >= target && polls_max) break;
             if (++polls > polls_max) {
                 asm volatile("red.relaxed.gpu.global.or.b64 [%0], %1;" ::"l"(bar), "l"(kBarrierGaveUp) : "memory");
+                asm volatile("red.relaxed.gpu.global.or.b64 [%0], 1;" ::"l"(status) : "memory");
                 ok = 0;
                 break;
             }

@@ -403,11 +403,9 @@ __global__ void __launch_bounds__(kEnergyThreads, NC <= 2 ? 4 : 2)
 // trips through L2 and the loads that follow it.
 
 // The row sets (at most kStepsMaxBlocks rows each) start at kStepsRowsOffset of a field's
-// scratch; the barrier word (lf2_barrier.cuh) is in the row after them.
+// scratch; the barrier and status words (lf2_barrier.cuh) are in the row after them.
 constexpr int kRowSets = kEnergyStepsRowSets;
 constexpr int kStepsMaxBlocks = kEnergyStepsBlocks;
-constexpr size_t kBarrierOffset = (size_t)kStepsRowsOffset + (size_t)kRowSets * kStepsMaxBlocks * kEnergySlots;
-static_assert(kBarrierOffset + kEnergySlots == (size_t)kFieldScratchDoubles, "multi-step scratch layout");
 
 // A run cut short by a barrier that did not complete leaves NaN records from `from` on (the
 // record of a step is finished during the next step, so `from` is the step before that barrier).
@@ -425,7 +423,8 @@ __global__ void __launch_bounds__(kEnergyThreads, 2)
             double *__restrict__ scratch, double *__restrict__ records, unsigned polls) {
     constexpr int NS = kNs<NC>;
     __shared__ double sh[ENERGY ? NS : 1][ENERGY ? kEnergyThreads : 1];
-    unsigned long long *bar = reinterpret_cast<unsigned long long *>(scratch + kBarrierOffset);
+    unsigned long long *bar = reinterpret_cast<unsigned long long *>(scratch + kStepsBarrierWord);
+    unsigned long long *status = reinterpret_cast<unsigned long long *>(scratch + kStepsStatusWord);
     const int nsb = ENERGY ? (int)gridDim.x - 1 : (int)gridDim.x;
     const bool reducer = ENERGY && (int)blockIdx.x == nsb;
     // rows [first, first + count) of the set of `step`, inside the row-set region (checked in
@@ -497,7 +496,7 @@ __global__ void __launch_bounds__(kEnergyThreads, 2)
                 p[a] = pn[a];
             }
         }
-        if (!grid_wait(bar, (step + 1ull) * gridDim.x, polls)) {
+        if (!grid_wait(bar, status, (step + 1ull) * gridDim.x, polls)) {
             if constexpr (ENERGY) poison_records(records, step > 0 ? step - 1 : 0, nsteps);
             return;
         }
@@ -702,13 +701,13 @@ cudaError_t steps_nc(const StepArgs &a, int nsteps, const CoefE &ke, double *scr
     // with ENERGY the partial sums' blocks and the reducing one
     const int nb = ENERGY ? energy_grid(a.g.sites) + 1 : (int)((a.g.sites + kEnergyThreads - 1) / kEnergyThreads);
     if (a.prec == LF2_F64)
-        return launch_cooperative(k_steps<double, NC, 3, ENERGY, Coef64>, nb, scratch + kBarrierOffset, s, (double *)a.phi, (double *)a.phi_out,
+        return launch_cooperative(k_steps<double, NC, 3, ENERGY, Coef64>, nb, scratch + kStepsBarrierWord, s, (double *)a.phi, (double *)a.phi_out,
                                   (double *)a.pi, a.comp, a.g, make_coef64(a.p, a.dt), ke, nsteps, scratch, records, polls);
     const Coef32 k = make_coef32(a.p, a.dt);
     if (a.prec == LF2_F32_KAHAN)
-        return launch_cooperative(k_steps<float, NC, 1, ENERGY, Coef32>, nb, scratch + kBarrierOffset, s, (float *)a.phi, (float *)a.phi_out,
+        return launch_cooperative(k_steps<float, NC, 1, ENERGY, Coef32>, nb, scratch + kStepsBarrierWord, s, (float *)a.phi, (float *)a.phi_out,
                                   (float *)a.pi, a.comp, a.g, k, ke, nsteps, scratch, records, polls);
-    return launch_cooperative(k_steps<float, NC, 0, ENERGY, Coef32>, nb, scratch + kBarrierOffset, s, (float *)a.phi, (float *)a.phi_out,
+    return launch_cooperative(k_steps<float, NC, 0, ENERGY, Coef32>, nb, scratch + kStepsBarrierWord, s, (float *)a.phi, (float *)a.phi_out,
                               (float *)a.pi, a.comp, a.g, k, ke, nsteps, scratch, records, polls);
 }
 
@@ -744,12 +743,12 @@ cudaError_t launch_steps_plain(const StepArgs &a, int nsteps, double *scratch, c
 
 cudaError_t steps_energy_timed_out(double *scratch, bool *out, cudaStream_t s) {
     unsigned long long word = 0;
-    cudaError_t e = cudaMemcpyAsync(&word, scratch + kBarrierOffset, sizeof word, cudaMemcpyDeviceToHost, s);
+    cudaError_t e = cudaMemcpyAsync(&word, scratch + kStepsStatusWord, sizeof word, cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     if (e != cudaSuccess) return e;
-    *out = (word & kBarrierGaveUp) != 0;
+    *out = word != 0;
     if (*out) {
-        e = cudaMemsetAsync(scratch + kBarrierOffset, 0, sizeof word, s);  // reported once
+        e = cudaMemsetAsync(scratch + kStepsStatusWord, 0, sizeof word, s);  // reported once
         if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     }
     return e;

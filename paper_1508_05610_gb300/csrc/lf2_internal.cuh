@@ -62,7 +62,11 @@ static_assert(3 + 2 * kMaxComp <= kEnergySlots, "energy slots");
 constexpr int kEnergyStepsBlocks = 303;
 constexpr int kEnergyStepsRowSets = 3;
 constexpr int kStepsRowsOffset = (kEnergyScratchDoubles + kEnergySlots - 1) / kEnergySlots * kEnergySlots;
-constexpr int kFieldScratchDoubles = kStepsRowsOffset + (kEnergyStepsRowSets * kEnergyStepsBlocks + 1) * kEnergySlots;
+constexpr int kStepsWordsOffset = kStepsRowsOffset + kEnergyStepsRowSets * kEnergyStepsBlocks * kEnergySlots;
+constexpr int kFieldScratchDoubles = kStepsWordsOffset + kEnergySlots;
+// In that last row: the barrier's word, zeroed before each launch, and a word that a run whose barrier
+// gave up sets, which keeps that until it has been reported (zero before the first launch).
+constexpr int kStepsBarrierWord = kStepsWordsOffset, kStepsStatusWord = kStepsWordsOffset + 1;
 // Energy of (phi, pi) as an lf2_energy_t record: written to scratch + kEnergyRecordOffset and,
 // when `record` is not NULL, also to `record` (device).  One launch.
 cudaError_t launch_energy(const void *phi, const void *pi, const Geom &g, int ncomp, lf2_precision prec,
@@ -80,8 +84,8 @@ cudaError_t launch_steps_energy(const StepArgs &a, int nsteps, double *scratch, 
                                 cudaStream_t s);
 // The same without the records (nothing of `scratch` but the barrier word is used).
 cudaError_t launch_steps_plain(const StepArgs &a, int nsteps, double *scratch, cudaStream_t s);
-// Whether the last multi-step run on this scratch had a barrier give up (the flag is then
-// cleared); synchronises `s`.
+// Whether a multi-step run on this scratch has had a barrier give up since the last report (this one
+// clears it); synchronises `s`.
 cudaError_t steps_energy_timed_out(double *scratch, bool *out, cudaStream_t s);
 
 // Temporal blocking: `depth` fused steps per pass over x-y tiles of tile_x x tile_y output

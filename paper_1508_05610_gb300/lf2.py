@@ -245,8 +245,8 @@ def lf2_leapfrog_energy(phi, pi, p: lf2_params, nsteps, dev_records_ptr, stream=
 
 
 def lf2_field_check(f, stream=None):
-    """Raises LF2Error (LF2_ERR_TIMEOUT) if a grid barrier of the last multi-step
-    lf2_leapfrog_energy or lf2_leapfrog run on f gave up."""
+    """Raises LF2Error (LF2_ERR_TIMEOUT) if a grid barrier of a multi-step
+    lf2_leapfrog_energy or lf2_leapfrog run on f has given up since the last check."""
     _call("lf2_field_check", f, _stream_ptr(stream))
 
 
