@@ -480,7 +480,7 @@ lf2_status lf2_leapfrog_ex(lf2_field phi, lf2_field pi, const lf2_params *p, int
     // small lattices without a tuned plan: all steps in one cooperative launch, when
     // lf2_leapfrog_init (or an energy) has made the scratch its barrier needs
     if (kernel == LF2_KERNEL_AUTO && phi->energy_scratch) {
-        const cudaError_t e = launch_steps_plain(probe, nsteps, phi->energy_scratch, s);
+        const cudaError_t e = launch_steps_plain(probe, nsteps, phi->energy_scratch, fault_injected("timeout"), s);
         if (e == cudaSuccess) {
             if (nsteps & 1) phi->front = 1 - phi->front;
             return LF2_OK;

@@ -737,8 +737,8 @@ cudaError_t launch_steps_energy(const StepArgs &a, int nsteps, double *scratch, 
     return launch_steps<true>(a, nsteps, scratch, records, no_wait, s);
 }
 
-cudaError_t launch_steps_plain(const StepArgs &a, int nsteps, double *scratch, cudaStream_t s) {
-    return launch_steps<false>(a, nsteps, scratch, nullptr, false, s);
+cudaError_t launch_steps_plain(const StepArgs &a, int nsteps, double *scratch, bool no_wait, cudaStream_t s) {
+    return launch_steps<false>(a, nsteps, scratch, nullptr, no_wait, s);
 }
 
 cudaError_t steps_energy_timed_out(double *scratch, bool *out, cudaStream_t s) {

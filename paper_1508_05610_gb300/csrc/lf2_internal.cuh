@@ -82,8 +82,8 @@ cudaError_t launch_step_energy(const StepArgs &a, double *scratch, double *recor
 // no_wait: the grid barrier gives up at once (host-side timeout injection, LF2_FAULT=timeout).
 cudaError_t launch_steps_energy(const StepArgs &a, int nsteps, double *scratch, double *records, bool no_wait,
                                 cudaStream_t s);
-// The same without the records (nothing of `scratch` but the barrier word is used).
-cudaError_t launch_steps_plain(const StepArgs &a, int nsteps, double *scratch, cudaStream_t s);
+// The same without the records (of `scratch` only the barrier and status words are used).
+cudaError_t launch_steps_plain(const StepArgs &a, int nsteps, double *scratch, bool no_wait, cudaStream_t s);
 // Whether a multi-step run on this scratch has had a barrier give up since the last report (this one
 // clears it); synchronises `s`.
 cudaError_t steps_energy_timed_out(double *scratch, bool *out, cudaStream_t s);

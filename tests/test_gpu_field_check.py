@@ -59,3 +59,27 @@ def test_a_timeout_is_kept_until_it_is_reported(lf2, monkeypatch, later):
         assert np.array_equal(got[0], ref[0]) and np.array_equal(got[1], ref[1])
         assert timed_out(lf2, s.phi)
         assert not timed_out(lf2, s.phi)  # once
+
+
+@pytest.mark.parametrize("prec", ["f64", "f32k"])
+def test_injected_timeout_reaches_lf2_leapfrog(lf2, monkeypatch, prec):
+    """LF2_FAULT=timeout makes the barriers of lf2_leapfrog's one-launch runs give up as well: the
+    check reports it, and a run of freshly uploaded fields steps as the site kernel does."""
+    monkeypatch.setenv("LF2_TUNE", "off")
+    p = lf2.params(**KW)
+    phi0 = inputs.gaussian_field(*SHAPE, 1, sigma=0.1, seed=942)
+    with lf2.System(SHAPE, 1, prec) as s, lf2.System(SHAPE, 1, prec) as t:
+        for q in (s, t):
+            q.upload(phi0, np.zeros_like(phi0))
+            lf2.lf2_leapfrog_init(q.phi, q.pi, p)
+        monkeypatch.setenv("LF2_FAULT", "timeout")
+        lf2.lf2_leapfrog(s.phi, s.pi, p, 4)
+        monkeypatch.delenv("LF2_FAULT")
+        assert timed_out(lf2, s.phi)
+        s.upload(phi0, np.zeros_like(phi0))
+        lf2.lf2_leapfrog_init(s.phi, s.pi, p)
+        lf2.lf2_leapfrog(s.phi, s.pi, p, 4)
+        assert not timed_out(lf2, s.phi)
+        lf2.lf2_leapfrog_ex(t.phi, t.pi, p, 4, kernel=lf2.LF2_KERNEL_SITE)
+        got, ref = s.download(), t.download()
+        assert np.array_equal(got[0], ref[0]) and np.array_equal(got[1], ref[1])
