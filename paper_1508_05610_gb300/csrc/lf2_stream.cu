@@ -283,6 +283,20 @@ int default_zchunk(const StepArgs &a, int by) {
     return zc < a.g.nz ? zc : a.g.nz;
 }
 
+// Fills a zero tile height and a zero number of planes with the defaults.  False if the grid does not
+// fit: its y and z extents are 16-bit, so lattices of more than 131070 rows take four rows where they
+// come in fours, and more planes go to a block where a lattice has too many for its default.
+constexpr int kMaxGridYZ = 65535, kMaxDefaultPlanes = 64;
+bool stream_tile(const StepArgs &a, int &by, int &zc) {
+    if (!by) by = a.g.ny / kDefaultBY <= kMaxGridYZ || a.g.ny % kStreamRows ? kDefaultBY : kStreamRows;
+    const long long nz = a.g.nz;
+    if (!zc) {
+        zc = default_zchunk(a, by);
+        while (zc < kMaxDefaultPlanes && (nz + zc - 1) / zc > kMaxGridYZ) zc *= 2;
+    }
+    return a.g.ny / by <= kMaxGridYZ && (nz + zc - 1) / zc <= kMaxGridYZ;
+}
+
 }  // namespace
 
 cudaError_t bounds_violations_stream(unsigned long long *n, bool reset) { return bounds_violations_here(n, reset); }
@@ -299,25 +313,27 @@ bool stream_supported(const StepArgs &a, int tile_y, int zchunk) {
     if (!a.drift) return false;
     // 16-byte alignment of every buffer
     if (((uintptr_t)a.phi | (uintptr_t)a.phi_out | (uintptr_t)a.pi | (uintptr_t)a.comp) % 16) return false;
-    return true;
+    return stream_tile(a, tile_y, zchunk);
 }
 
 cudaError_t launch_default_step(const StepArgs &a, cudaStream_t s) {
     // Of the lattices whose rows come in twos but not in fours, 3-component ones take the site kernel:
     // 40x98x200 FP32 10.5 us a step, streaming 14.7 (100x102x104: 12.6 and 14.6)
-    const bool tile = stream_supported(a, kDefaultBY, 0) && (a.ncomp != 3 || a.g.ny % kStreamRows == 0);
-    return tile ? launch_stream_step(a, kDefaultBY, 0, 1, s) : launch_general_step(a, s);
+    const bool fours = a.g.ny % kStreamRows == 0;
+    int rows = 0;
+    if (a.ncomp != 3 || fours)
+        rows = stream_supported(a, kDefaultBY, 0) ? kDefaultBY : (fours && stream_supported(a, kStreamRows, 0) ? kStreamRows : 0);
+    return rows ? launch_stream_step(a, rows, 0, 1, s) : launch_general_step(a, s);
 }
 
 cudaError_t launch_stream_step(const StepArgs &a, int tile_y, int zchunk, int, cudaStream_t s) {
     if (a.g.sites == 0) return cudaSuccess;
-    const int by = tile_y ? tile_y : kDefaultBY;
-    const int zc = zchunk > 0 ? zchunk : default_zchunk(a, by);
-    switch (by) {
-        case 2: return launch_by<2>(a, zc, s);
-        case 4: return launch_by<4>(a, zc, s);
-        case 8: return launch_by<8>(a, zc, s);
-        default: return launch_by<16>(a, zc, s);
+    if (!stream_tile(a, tile_y, zchunk)) return cudaErrorNotSupported;
+    switch (tile_y) {
+        case 2: return launch_by<2>(a, zchunk, s);
+        case 4: return launch_by<4>(a, zchunk, s);
+        case 8: return launch_by<8>(a, zchunk, s);
+        default: return launch_by<16>(a, zchunk, s);
     }
 }
 
