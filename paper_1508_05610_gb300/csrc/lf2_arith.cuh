@@ -425,7 +425,7 @@ inline Stride3 make_stride3(long long stride, const Geom &g) {
 struct SiteWalk {
     int x, y, z;
     long long s;
-    __device__ __forceinline__ SiteWalk(long long first, const Geom &g) : s(first) {
+    __host__ __device__ __forceinline__ SiteWalk(long long first, const Geom &g) : s(first) {
         if (first < (1LL << 31)) {
             const unsigned f = (unsigned)first, r = f / (unsigned)g.nx;
             x = (int)(f - r * (unsigned)g.nx);
@@ -438,19 +438,21 @@ struct SiteWalk {
             y = (int)(r - (long long)z * g.ny);
         }
     }
-    __device__ __forceinline__ void advance(const Stride3 &d, const Geom &g) {
+    // Unsigned: a coordinate and its step are each below a side, which may be up to 2^31 - 1.
+    __host__ __device__ __forceinline__ void advance(const Stride3 &d, const Geom &g) {
         s += d.sites;
-        x += d.x;
-        y += d.y;
-        z += d.z;
-        if (x >= g.nx) {
-            x -= g.nx;
-            ++y;
+        unsigned ux = (unsigned)x + (unsigned)d.x, uy = (unsigned)y + (unsigned)d.y, uz = (unsigned)z + (unsigned)d.z;
+        if (ux >= (unsigned)g.nx) {
+            ux -= (unsigned)g.nx;
+            ++uy;
         }
-        if (y >= g.ny) {
-            y -= g.ny;
-            ++z;
+        if (uy >= (unsigned)g.ny) {
+            uy -= (unsigned)g.ny;
+            ++uz;
         }
+        x = (int)ux;
+        y = (int)uy;
+        z = (int)uz;  // at least nz once s is past the last site
     }
 };
 
