@@ -456,6 +456,18 @@ struct SiteWalk {
     }
 };
 
+// The x- and y-neighbours of site i of a z-plane of fewer than 2^31 sites.
+struct PlaneNbr {
+    int xm, xp, ym, yp;
+    __host__ __device__ __forceinline__ PlaneNbr(int i, const Geom &g) {
+        const int plane = g.nx * g.ny, y = i / g.nx, x = i - y * g.nx;
+        xm = x == 0 ? i - 1 + g.nx : i - 1;
+        xp = x == g.nx - 1 ? i + 1 - g.nx : i + 1;
+        ym = y == 0 ? i - g.nx + plane : i - g.nx;
+        yp = y == g.ny - 1 ? x : i + g.nx;
+    }
+};
+
 __device__ __forceinline__ int wrap_dn(int i, int n) { return i == 0 ? n - 1 : i - 1; }
 __device__ __forceinline__ int wrap_up(int i, int n) { return i == n - 1 ? 0 : i + 1; }
 

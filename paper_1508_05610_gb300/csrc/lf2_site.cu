@@ -168,9 +168,7 @@ __global__ void __launch_bounds__(kMarchThreads) k_march(const float *__restrict
     const int plane = g.nx * g.ny;
     const int i = blockIdx.x * kMarchThreads + threadIdx.x;
     if (i >= plane) return;
-    const int y = i / g.nx, x = i - y * g.nx;
-    const int ixm = x == 0 ? i + g.nx - 1 : i - 1, ixp = x == g.nx - 1 ? i + 1 - g.nx : i + 1;
-    const int iym = y == 0 ? i + plane - g.nx : i - g.nx, iyp = y == g.ny - 1 ? x : i + g.nx;
+    const PlaneNbr n(i, g);
     const int z0 = blockIdx.y * zchunk, z1 = min(z0 + zchunk, g.nz);
     auto load = [&](long long at) { return __ldg(phi + checked(at, 1, g.sites)); };
     float below[1] = {load((long long)wrap_dn(z0, g.nz) * plane + i)}, cur[1] = {load((long long)z0 * plane + i)};
@@ -183,10 +181,10 @@ __global__ void __launch_bounds__(kMarchThreads) k_march(const float *__restrict
             const long long pz = (long long)zb * plane;
             at[b] = checked(pz + i, 1, g.sites);
             next[b] = load((long long)wrap_up(zb, g.nz) * plane + i);
-            xm[b][0] = load(pz + ixm);
-            xp[b][0] = load(pz + ixp);
-            ym[b][0] = load(pz + iym);
-            yp[b][0] = load(pz + iyp);
+            xm[b][0] = load(pz + n.xm);
+            xp[b][0] = load(pz + n.xp);
+            ym[b][0] = load(pz + n.ym);
+            yp[b][0] = load(pz + n.yp);
             p[b][0] = pi[at[b]];
             cm[b][0] = KAHAN ? comp[at[b]] : 0.0f;
         }

@@ -1,4 +1,4 @@
-"""CPU: the kernels' index arithmetic on lattices with a side close to 2^31 sites, compiled
+"""CPU: the kernels' index arithmetic on lattices with a side or a plane close to 2^31 sites, compiled
 for the host with signed overflow trapped, against 64-bit divisions."""
 import os
 import subprocess
@@ -22,6 +22,19 @@ static void walk(int nx, int ny, int nz, long long stride, long long first, int 
         if (w.s != s || w.x != s % nx || w.y != r % ny || w.z != r / ny) fail("walk", s);
     }
 }
+static void plane(int nx, int ny) {
+    const Geom g{nx, ny, 1, (long long)nx * ny};
+    const long long p = (long long)nx * ny;
+    const long long at[] = {0, 1, nx - 1, nx, 2LL * nx - 1, p / 2, p - nx, p - 2, p - 1};
+    for (long long i : at) {
+        if (i < 0 || i >= p) continue;
+        const PlaneNbr n((int)i, g);
+        const long long y = i / nx, x = i % nx;
+        if (n.xm != y * nx + (x + nx - 1) % nx || n.xp != y * nx + (x + 1) % nx ||
+            n.ym != (y + ny - 1) % ny * nx + x || n.yp != (y + 1) % ny * nx + x)
+            fail("plane", i);
+    }
+}
 int main() {
     const int big = 2147483647;
     for (long long stride : {256LL, 152LL * 4 * 256, 152LL * 16 * 256, 155189LL})
@@ -33,13 +46,14 @@ int main() {
                 walk(1, 1, side, stride, first, 200000);
                 walk(5, 1, side / 5, stride, first, 200000);
             }
-    for (int s = 1; s < 12; ++s) walk(s, 13 - s, 7, 17, s, 100);
+    for (int s = 1; s < 12; ++s) walk(s, 13 - s, 7, 17, s, 100), plane(s, 13 - s), plane(1, s);
+    plane(1000, 2147483), plane(65536, 32767), plane(big - 256, 1), plane(1, big - 256), plane(1 << 20, 2047);
     puts("ok");
 }
 """
 
 
-def test_coordinates_near_2_to_the_31(tmp_path):
+def test_coordinates_and_neighbours_near_2_to_the_31(tmp_path):
     from paper_1508_05610_gb300 import build
     src, exe = tmp_path / "geometry.cu", tmp_path / "geometry"
     src.write_text(SOURCE)
