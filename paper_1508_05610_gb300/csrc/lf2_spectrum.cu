@@ -101,7 +101,7 @@ __global__ void __launch_bounds__(kBinThreads) k_bin(const C *__restrict__ spec,
         unsigned count = 0u;
         if (in) {
             const int w = self(x) ? 1 : 2;  // kx and -kx
-            power *= (double)w;
+            power *= (double)w * inv_volume;  // before the shell's sum, which could overflow where its mean does not
             count = (unsigned)(w * images);
             if (!add_power) ksum = (double)count * sqrt((double)s2);
         }
@@ -131,9 +131,9 @@ __global__ void __launch_bounds__(kBinThreads) k_bin(const C *__restrict__ spec,
     double *out = partials + (size_t)blockIdx.x * 3 * nbins;
     for (int i = threadIdx.x; i < nbins; i += kBinThreads) {
         if (add_power) {
-            out[i] += hist[i] * inv_volume;
+            out[i] += hist[i];
         } else {
-            out[i] = hist[i] * inv_volume;
+            out[i] = hist[i];
             out[nbins + i] = hist[nbins + i] * kunit;
             out[2 * nbins + i] = (double)cnt[i];
         }

@@ -101,3 +101,16 @@ def test_spectrum_at_edges_of_rows_and_shells(lf2, n, nbins):
     assert np.array_equal(C, count)
     assert np.max(np.abs(P - want)) <= 1e-12 * np.max(want)
     assert np.max(np.abs(K - k * 2 * math.pi / (n * 0.8))) <= 1e-12 * max(np.max(K), 1e-300)
+
+
+def test_spectrum_whose_unnormalised_shell_sums_overflow(lf2):
+    """Fields scaled by a power of two have the spectrum scaled by its square, up to where the sum of a
+    shell's |phi~|^2 overflows though the power, that sum over N^3 times the modes, is far below."""
+    n, nbins = 64, 32
+    phi = inputs.gaussian_field(n, n, n, 1, sigma=0.8, seed=143)
+    with lf2.System((n, n, n), 1, "f64") as s:
+        lf2.lf2_field_upload(s.phi, phi)
+        P = lf2.lf2_power_spectrum(s.phi, nbins=nbins)[0]
+        lf2.lf2_field_upload(s.phi, np.ldexp(phi, 500))
+        high = lf2.lf2_power_spectrum(s.phi, nbins=nbins)[0]
+    assert np.max(np.abs(np.ldexp(high, -1000) - P)) <= 1e-13 * np.max(P)
