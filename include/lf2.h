@@ -94,7 +94,7 @@ typedef struct {
 
 /* Kernel selection for lf2_leapfrog_ex.  Every variant computes bitwise the same result. */
 typedef enum {
-    LF2_KERNEL_AUTO = 0,     /* tuned choice (the one lf2_leapfrog uses) */
+    LF2_KERNEL_AUTO = 0,     /* tuned choice (the one lf2_leapfrog uses); in a plan: what runs without one */
     LF2_KERNEL_SITE = 1,     /* one thread per site, any lattice shape */
     LF2_KERNEL_STREAM = 2,   /* x-y tile streaming along z, one step per pass */
     LF2_KERNEL_TBLOCK = 3    /* temporal blocking: `depth` steps per pass; FP32 steps left over in
@@ -229,7 +229,7 @@ lf2_status lf2_leapfrog_init(lf2_field phi, lf2_field pi, const lf2_params *p, v
  * shape, else the default one; results are bitwise identical whichever kernel runs.  The
  * environment variable LF2_TUNE changes that: "off" ignores tuned plans, "force" tunes a shape
  * that has no plan on its first call (that call synchronises and allocates, so keep it out of
- * stream capture).  Two or more steps of a small lattice without a plan (one site per resident
+ * stream capture).  Two or more steps of a small lattice without a plan, or tuned to it (one site per resident
  * thread: up to about 230,000 sites of a real FP32 field) run in one cooperative launch with a grid
  * barrier between steps, once lf2_leapfrog_init or an energy call has allocated phi's scratch; the
  * barrier's waits are bounded as in lf2_leapfrog_energy and reported by lf2_field_check.  Calls on
@@ -369,7 +369,9 @@ lf2_status lf2_ensemble_destroy(lf2_ensemble e);
  * precision by timing candidates (one-step streaming tiles; temporal blocking of depth 2-8
  * with several tiles and column widths) on a proxy lattice of the same x-y plane and at most
  * 256 z-planes (fewer for very large planes, to stay within about 8 GB), filled with a copy
- * of the fields' first planes -- phi and pi are not modified.
+ * of the fields' first planes -- phi and pi are not modified.  On a lattice small enough for it, all
+ * steps in one launch (see lf2_leapfrog) are timed as well, on a copy of the whole lattice; where
+ * that is the fastest, the plan is LF2_KERNEL_AUTO, and phi's scratch is allocated if missing.
  * The plan is cached per process (and appended to the file named by the environment variable
  * LF2_TUNE_CACHE, which is read on first use) and used by every later lf2_leapfrog on a lattice
  * of that shape.  Results do not depend on the plan: all variants are bitwise identical.

@@ -434,32 +434,14 @@ lf2_status lf2_leapfrog_init(lf2_field phi, lf2_field pi, const lf2_params *p, v
     return LF2_OK;
 }
 
-lf2_status lf2_leapfrog_ex(lf2_field phi, lf2_field pi, const lf2_params *p, int nsteps, const lf2_step_config *cfg,
-                           void *stream) {
-    lf2_status st = check_pair(phi, pi);
-    if (st == LF2_OK) st = check_params(p);
-    if (st != LF2_OK) return st;
-    if (nsteps < 0) return fail(LF2_ERR_INVALID, "nsteps must be >= 0");
-    cudaStream_t s = (cudaStream_t)stream;
-    int kernel = cfg ? cfg->kernel : LF2_KERNEL_AUTO;
-    if (kernel < LF2_KERNEL_AUTO || kernel > LF2_KERNEL_TBLOCK) return fail(LF2_ERR_INVALID, "unknown kernel %d", kernel);
-    if (fault_injected("launch")) return fail(LF2_ERR_CUDA, "launch failure injected by LF2_FAULT=launch");
-    lf2_step_config tuned{};
-    if (kernel == LF2_KERNEL_AUTO && tune_mode() != TuneMode::Off) {
-        bool have = plan_lookup(phi->lat->n, phi->ncomp, phi->prec, &tuned);
-        if (!have && tune_mode() == TuneMode::Force) {
-            st = lf2_tune(phi, pi, p, 0, &tuned, stream);
-            if (st != LF2_OK) return st;
-            have = true;
-        }
-        if (have) {
-            cfg = &tuned;
-            kernel = tuned.kernel;
-        }
-    }
-    const int tile_y = cfg ? cfg->tile_y : 0;
-    const int zchunk = cfg ? cfg->zchunk : 0;
-    st = (kernel == LF2_KERNEL_TBLOCK) ? ensure_tblock(phi, pi, s) : ensure_dynamic(phi, s);
+}  // extern "C"
+
+namespace lf2 {
+
+lf2_status leapfrog_run(lf2_field phi, lf2_field pi, const lf2_params *p, int nsteps, const lf2_step_config *cfg,
+                        cudaStream_t s) {
+    const int kernel = cfg->kernel, tile_y = cfg->tile_y, zchunk = cfg->zchunk;
+    lf2_status st = (kernel == LF2_KERNEL_TBLOCK) ? ensure_tblock(phi, pi, s) : ensure_dynamic(phi, s);
     if (st != LF2_OK) return st;
 
     const StepArgs probe = step_args(phi, pi, p, p->dt, true);
@@ -477,7 +459,7 @@ lf2_status lf2_leapfrog_ex(lf2_field phi, lf2_field pi, const lf2_params *p, int
     };
 
     int done = 0;
-    // small lattices without a tuned plan: all steps in one cooperative launch, when
+    // small lattices without a tuned plan, or tuned to this: all steps in one cooperative launch, when
     // lf2_leapfrog_init (or an energy) has made the scratch its barrier needs
     if (kernel == LF2_KERNEL_AUTO && phi->energy_scratch) {
         const cudaError_t e = launch_steps_plain(probe, nsteps, phi->energy_scratch, fault_injected("timeout"), s);
@@ -524,6 +506,33 @@ lf2_status lf2_leapfrog_ex(lf2_field phi, lf2_field pi, const lf2_params *p, int
         if (st != LF2_OK) return st;
     }
     return LF2_OK;
+}
+
+}  // namespace lf2
+
+extern "C" {
+
+lf2_status lf2_leapfrog_ex(lf2_field phi, lf2_field pi, const lf2_params *p, int nsteps, const lf2_step_config *cfg,
+                           void *stream) {
+    lf2_status st = check_pair(phi, pi);
+    if (st == LF2_OK) st = check_params(p);
+    if (st != LF2_OK) return st;
+    if (nsteps < 0) return fail(LF2_ERR_INVALID, "nsteps must be >= 0");
+    const int kernel = cfg ? cfg->kernel : LF2_KERNEL_AUTO;
+    if (kernel < LF2_KERNEL_AUTO || kernel > LF2_KERNEL_TBLOCK) return fail(LF2_ERR_INVALID, "unknown kernel %d", kernel);
+    if (fault_injected("launch")) return fail(LF2_ERR_CUDA, "launch failure injected by LF2_FAULT=launch");
+    lf2_step_config run = cfg ? *cfg : lf2_step_config{};
+    if (kernel == LF2_KERNEL_AUTO && tune_mode() != TuneMode::Off) {
+        lf2_step_config tuned{};
+        bool have = plan_lookup(phi->lat->n, phi->ncomp, phi->prec, &tuned);
+        if (!have && tune_mode() == TuneMode::Force) {
+            st = lf2_tune(phi, pi, p, 0, &tuned, stream);
+            if (st != LF2_OK) return st;
+            have = true;
+        }
+        if (have) run = tuned;
+    }
+    return leapfrog_run(phi, pi, p, nsteps, &run, (cudaStream_t)stream);
 }
 
 lf2_status lf2_leapfrog(lf2_field phi, lf2_field pi, const lf2_params *p, int nsteps, void *stream) {

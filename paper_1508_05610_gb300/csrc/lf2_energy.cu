@@ -715,7 +715,7 @@ template <bool ENERGY>
 cudaError_t launch_steps(const StepArgs &a, int nsteps, double *scratch, double *records, bool no_wait, cudaStream_t s) {
     if (!a.drift || nsteps < 2) return cudaErrorNotSupported;
     // one site per thread; the launch itself checks that all blocks are resident
-    if (a.g.sites > (ENERGY ? (long long)kStepsMaxBlocks : 8LL * device_sm_count()) * kEnergyThreads)
+    if (a.g.sites > (ENERGY ? (long long)kStepsMaxBlocks * kEnergyThreads : steps_plain_max_sites()))
         return cudaErrorNotSupported;
     const CoefE ke = make_coefE(a.p);
     const unsigned polls = no_wait ? 0u : kBarrierPolls;
@@ -736,6 +736,8 @@ cudaError_t launch_steps_energy(const StepArgs &a, int nsteps, double *scratch, 
                                 cudaStream_t s) {
     return launch_steps<true>(a, nsteps, scratch, records, no_wait, s);
 }
+
+long long steps_plain_max_sites() { return 8LL * device_sm_count() * kEnergyThreads; }
 
 cudaError_t launch_steps_plain(const StepArgs &a, int nsteps, double *scratch, bool no_wait, cudaStream_t s) {
     return launch_steps<false>(a, nsteps, scratch, nullptr, no_wait, s);

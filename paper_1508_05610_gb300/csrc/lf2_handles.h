@@ -64,6 +64,14 @@ lf2_status ensure_tblock(lf2_field phi, lf2_field pi, cudaStream_t s);  // + pi 
 StepArgs step_args(lf2_field phi, lf2_field pi, const lf2_params *p, double dt, bool drift);
 TbArgs tb_args(lf2_field phi, lf2_field pi, const lf2_params *p);
 
+// nsteps of lf2_leapfrog_ex with checked arguments; LF2_KERNEL_AUTO is the untuned choice, whatever plan
+// the shape has.
+lf2_status leapfrog_run(lf2_field phi, lf2_field pi, const lf2_params *p, int nsteps, const lf2_step_config *cfg,
+                        cudaStream_t s);
+
+// Energy scratch of a field, which the multi-step runs use too (lf2_api.cu).
+lf2_status ensure_energy_scratch(lf2_field f);
+
 // Tuned kernel plan for a lattice shape (filled by lf2_tune); false if none.
 bool plan_lookup(const int n[3], int ncomp, lf2_precision prec, lf2_step_config *out);
 

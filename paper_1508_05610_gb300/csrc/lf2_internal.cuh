@@ -84,6 +84,8 @@ cudaError_t launch_steps_energy(const StepArgs &a, int nsteps, double *scratch, 
                                 cudaStream_t s);
 // The same without the records (of `scratch` only the barrier and status words are used).
 cudaError_t launch_steps_plain(const StepArgs &a, int nsteps, double *scratch, bool no_wait, cudaStream_t s);
+// No lattice of more sites runs that way (of those with fewer, the ones whose blocks all fit at once).
+long long steps_plain_max_sites();
 // Whether a multi-step run on this scratch has had a barrier give up since the last report (this one
 // clears it); synchronises `s`.
 cudaError_t steps_energy_timed_out(double *scratch, bool *out, cudaStream_t s);

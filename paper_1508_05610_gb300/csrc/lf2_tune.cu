@@ -2,7 +2,8 @@
 //
 // Every kernel variant computes bitwise the same result, so the tuner only has to find the
 // fastest one.  It times candidate configurations (one-step streaming tiles and temporal
-// blocking of several depths, column widths and tiles) on a proxy lattice with the same x-y
+// blocking of several depths, column widths and tiles; on a small lattice also all steps in one
+// launch, which is what runs there without a plan) on a proxy lattice with the same x-y
 // plane as the real one and at most kProxyPlanes z-planes, filled with a copy of the real
 // fields' first planes: the caller's fields are never modified.  The winner is kept in a
 // process-wide table keyed by (shape, components, precision, SM count) that lf2_leapfrog
@@ -141,7 +142,8 @@ extern "C" lf2_status lf2_tune(lf2_field phi, lf2_field pi, const lf2_params *p,
     // proxy lattice: same x-y plane, first planes of the real fields
     // six buffers (phi, pi, compensation, each with a back buffer) of one plane
     const size_t plane_bytes = (size_t)n[0] * n[1] * phi->ncomp * 4 * sizeof(float) * 2;
-    int pz = n[2] < kProxyPlanes ? n[2] : kProxyPlanes;
+    const bool small = phi->lat->sites <= steps_plain_max_sites();  // timed whole
+    int pz = n[2] < kProxyPlanes || small ? n[2] : kProxyPlanes;
     while (pz > 32 && (size_t)pz * plane_bytes > kProxyBytes) pz /= 2;
     const int psizes[3] = {n[0], n[1], pz};
     lf2_lattice plat = nullptr;
@@ -172,13 +174,17 @@ extern "C" lf2_status lf2_tune(lf2_field phi, lf2_field pi, const lf2_params *p,
     }
     lf2_step_config best{LF2_KERNEL_STREAM, 0, 0, 0, 0, 0};
     float best_ms = -1.0f;
-    for (const lf2_step_config &c : candidates(phi->prec, flags)) {
+    auto time_config = [&](const lf2_step_config &c) {
+        auto run = [&]() {  // without a plan, lest this tunes again or takes an earlier one
+            return c.kernel == LF2_KERNEL_AUTO ? leapfrog_run(pphi, ppi, p, kTuneSteps, &c, s)
+                                               : lf2_leapfrog_ex(pphi, ppi, p, kTuneSteps, &c, stream);
+        };
         // warm-up (also rejects configurations that do not fit this lattice)
-        if (lf2_leapfrog_ex(pphi, ppi, p, kTuneSteps, &c, stream) != LF2_OK) continue;
+        if (run() != LF2_OK) return;
         float ms = -1.0f;
         for (int rep = 0; rep < 2; ++rep) {
             cudaEventRecord(e0, s);
-            if (lf2_leapfrog_ex(pphi, ppi, p, kTuneSteps, &c, stream) != LF2_OK) break;
+            if (run() != LF2_OK) break;
             cudaEventRecord(e1, s);
             if (cudaEventSynchronize(e1) != cudaSuccess) break;
             float t = 0.0f;
@@ -189,7 +195,13 @@ extern "C" lf2_status lf2_tune(lf2_field phi, lf2_field pi, const lf2_params *p,
             best_ms = ms;
             best = c;
         }
-    }
+    };
+    for (const lf2_step_config &c : candidates(phi->prec, flags)) time_config(c);
+    // Without this a plan would shut out the one-launch run that a small lattice takes when it has none
+    // (32^3 real FP64 2.2 us a step, 4.3 in the best streaming tile).  Two steps show whether it fits.
+    if (best_ms > 0.0f && small && ensure_energy_scratch(pphi) == LF2_OK && ensure_energy_scratch(phi) == LF2_OK &&
+        launch_steps_plain(step_args(pphi, ppi, p, p->dt, true), 2, pphi->energy_scratch, false, s) == cudaSuccess)
+        time_config(lf2_step_config{LF2_KERNEL_AUTO, 0, 0, 0, 0, 0});
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
     cleanup();

@@ -320,3 +320,43 @@ def test_32cube_run_with_energy_every_step_in_one_cuda_graph(lf2, ora):
         assert abs(rec[n, 10] - oe["sum_sq"][0]) <= 1e-12 * oe["sum_sq"][0], n
     print(f"32^3 step + energy, one graph: {us_per_step:.1f} us per step")
     assert us_per_step < 1000
+
+
+@pytest.mark.parametrize("prec,ncomp", [("f32k", 1), ("f64", 1), ("f64", 2)])
+def test_tuning_a_small_lattice_keeps_its_one_launch_run(lf2, monkeypatch, prec, ncomp):
+    """A small lattice without a plan takes all steps in one launch, two to four times as fast as a launch
+    per step; a tuned one does too.  That it does shows in a barrier timeout injected into the run,
+    which no other kernel has."""
+    shape = (30, 28, 26)
+    kw = dict(dx=1.0, dt=0.05, lam=1.0, eta=1.0, m2=0.0)
+    p = lf2.params(**kw)
+    phi0 = inputs.gaussian_field(*shape, ncomp, sigma=0.4, seed=64)
+    ref = run_site(lf2, shape, ncomp, prec, phi0, np.zeros_like(phi0), kw, 9)
+    with lf2.System(shape, ncomp, prec) as s:
+        s.upload(phi0, np.zeros_like(phi0))
+        lf2.lf2_tune(s.phi, s.pi, p, flags=lf2.LF2_TUNE_FORCE)
+        lf2.lf2_leapfrog(s.phi, s.pi, p, 9)
+        got = s.download()
+        assert np.array_equal(got[0], ref[0]) and np.array_equal(got[1], ref[1])
+        lf2.lf2_field_check(s.phi)
+        monkeypatch.setenv("LF2_FAULT", "timeout")
+        lf2.lf2_leapfrog(s.phi, s.pi, p, 9)
+        monkeypatch.delenv("LF2_FAULT")
+        with pytest.raises(lf2.LF2Error) as e:
+            lf2.lf2_field_check(s.phi)
+        assert e.value.status == lf2.LF2_ERR_TIMEOUT
+
+
+def test_tuning_still_refuses_what_only_the_default_kernels_run(lf2):
+    with lf2.System((15, 13, 11), 5, "f64") as s:
+        with pytest.raises(lf2.LF2Error) as e:
+            lf2.lf2_tune(s.phi, s.pi, lf2.params(dt=0.05), flags=lf2.LF2_TUNE_FORCE)
+    assert e.value.status == lf2.LF2_ERR_UNSUPPORTED
+
+
+def test_tuning_with_parameters_that_no_step_accepts_is_refused(lf2):
+    with lf2.System((16, 16, 12), 1, "f32k") as s:
+        for bad in (dict(dx=0.0), dict(dt=float("nan"))):
+            with pytest.raises(lf2.LF2Error) as e:
+                lf2.lf2_tune(s.phi, s.pi, lf2.params(**bad), flags=lf2.LF2_TUNE_FORCE)
+            assert e.value.status == lf2.LF2_ERR_UNSUPPORTED
