@@ -59,3 +59,11 @@ def test_streaming_tiles_that_do_not_fit_are_refused(lf2):
         with pytest.raises(lf2.LF2Error) as e:
             lf2.lf2_leapfrog_ex(s.phi, s.pi, lf2.params(**KW), 1, kernel=lf2.LF2_KERNEL_STREAM, tile_y=2)
     assert e.value.status == lf2.LF2_ERR_UNSUPPORTED
+
+
+def test_one_step_plan_of_a_lattice_that_only_tall_tiles_fit(lf2):
+    shape = (4, 262152, 1)
+    with lf2.System(shape, 1, "f32") as s:
+        plan = lf2.lf2_tune(s.phi, s.pi, lf2.params(**KW), flags=lf2.LF2_TUNE_FORCE | lf2.LF2_TUNE_ONE_STEP)
+    assert plan["kernel"] == lf2.LF2_KERNEL_STREAM and plan["tile_y"] == 8
+    same_as_site(lf2, shape, 1, "f32", lambda s, p: lf2.lf2_leapfrog(s.phi, s.pi, p, 2))
