@@ -9,6 +9,7 @@ nb once, each at most u (6 |phi| + |nb|): in all below 6 u (sum|phi_i| + 6 |phi|
 the smallest subnormal for each rounding.  (The range's high end, 2^1017, cannot be seen in a step:
 phi^2 overflows above 2^512 and the step gives NaN whatever the sum.)"""
 from fractions import Fraction
+from functools import reduce
 
 import numpy as np
 import pytest
@@ -121,3 +122,64 @@ def test_gradient_energy_differences_against_exact_rationals(lf2, kind, prec):
             terms += 1
     got = 2 * Fraction(e["gradient"])
     assert abs(got - exact) <= (terms + 3) * Fraction(1, 2 ** 53) * exact, float(abs(got - exact) / exact)
+
+
+@pytest.mark.parametrize("kernel", ["site", "stream", "tblock"])
+def test_sums_of_signed_zeros_have_the_sign_of_ieee_additions(lf2, kernel):
+    """A zero sum is -0 only if all six neighbours are.  It shows at a site of +0 with pi = -0: there
+    pi' = nb + (-g phi + pi) is nb + -0."""
+    rng = np.random.default_rng(9)
+    phi = np.where(rng.random(SHAPE[::-1] + (1,)) < 0.08, 0.0, -0.0)
+    pi = np.full_like(phi, -0.0)
+    f = phi[..., 0]
+    nbrs = [np.roll(f, sh, ax) for ax in range(3) for sh in (1, -1)]
+    nb = reduce(np.add, nbrs)  # sum() would start from +0
+    p = lf2.params(dx=1.0, dt=1.0, lam=0.0, eta=0.0, m2=0.0)
+    with lf2.System(SHAPE, 1, "f64") as s, lf2.System(SHAPE, 1, "f64") as t:
+        for q in (s, t):
+            q.upload(phi, pi)
+        steps, kw = {"site": (1, dict(kernel=1)), "stream": (1, dict(kernel=2)),
+                     "tblock": (2, dict(kernel=3, depth=2, cx=1, tile_x=4, tile_y=4))}[kernel]
+        lf2.lf2_leapfrog_ex(s.phi, s.pi, p, steps, **kw)
+        lf2.lf2_leapfrog_ex(t.phi, t.pi, p, steps, kernel=lf2.LF2_KERNEL_SITE)
+        got, ref = s.download(), t.download()
+    for a, b in zip(got, ref):
+        assert np.array_equal(a, b) and np.array_equal(np.signbit(a), np.signbit(b))
+    if steps == 1:
+        at = ~np.signbit(f)
+        assert at.any() and np.array_equal(np.signbit(got[1][..., 0])[at], np.signbit(nb)[at])
+
+
+@pytest.mark.parametrize("prec", ["f64", "f32k"])
+@pytest.mark.parametrize("what", ["energy", "step"])
+def test_zeros_cost_no_more_than_other_values(lf2, what, prec):
+    """A field of zeros in one component, or in all of them, against one of Gaussian values, on a lattice
+    that fills the GPU.  Nothing is added in FP64 for a zero that other values need not add, but the FP64
+    energy subtracts zeros there: 27 FP64 instructions a site instead of 21.  (With the sums in FP64 too,
+    1.55 and 1.7 times as long.)"""
+    import torch
+    n = (128, 128, 128)
+    p = lf2.params(dx=1.0, dt=0.05, lam=1.0, eta=1.0, m2=0.0)
+    rec = torch.zeros(16, dtype=torch.float64, device="cuda")
+    full = np.random.default_rng(10).standard_normal(n[::-1] + (2,)) * 0.1
+    times = []
+    with lf2.System(n, 2, prec) as s:
+        for zero in ([], [1], [0, 1]):
+            phi = full.copy()
+            phi[..., zero] = 0.0
+            s.upload(phi, np.zeros_like(phi))
+            lf2.lf2_leapfrog_init(s.phi, s.pi, p)
+            best = 1e9
+            for _ in range(8):
+                a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+                a.record()
+                for _ in range(4):
+                    if what == "energy":
+                        lf2.lf2_energy_device(s.phi, s.pi, p, rec.data_ptr())
+                    else:
+                        lf2.lf2_leapfrog_ex(s.phi, s.pi, p, 1, kernel=lf2.LF2_KERNEL_SITE)
+                b.record()
+                torch.cuda.synchronize()
+                best = min(best, a.elapsed_time(b))
+            times.append(best)
+    assert max(times[1:]) <= (1.4 if (what, prec) == ("energy", "f64") else 1.25) * times[0], times
