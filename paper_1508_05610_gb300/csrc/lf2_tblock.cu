@@ -1,5 +1,7 @@
 // lf2_tblock.cu -- temporal blocking: configuration checks and dispatch by precision.
 // The kernels are in lf2_tblock.cuh, instantiated per precision in lf2_tblock_{f64,f32k,f32}.cu.
+#include <cmath>
+
 #include "lf2_internal.cuh"
 
 namespace lf2 {
@@ -58,15 +60,23 @@ bool tblock_supported(const TbArgs &a, TbConfig &c) {
         // chunk of zc planes costs zc + 2 depth iterations, and with one block per SM a launch
         // takes ceil(blocks / SMs) waves.  More chunks shrink the last, partly filled wave
         // but add the 2 depth halo planes per chunk.
+        // Of FP32 passes on pairs (one or two components) a plane costs more in a chunk of more than 32 GB
+        // in all buffers, 1.5 % for each doubling: the next row of tiles returns to memory that was left
+        // that long ago.  1536^3 complex, 24x24 tiles, us a step: chunks of 1536 planes (174 GB, the fewest
+        // waves) 11560, 768 11456, 384 11402, 192 11483, 64 12103; 1792^3 real, 56x24: whole 8353, chunks
+        // of 359 8161; 1280^3 complex: chunks of 427 planes (33 GB) 6669, 256 6701.
+        const bool pairs = esz == 4 && a.ncomp <= 2 && c.cx * a.ncomp >= 4;
+        const double plane_gb = 1e-9 * a.g.nx * a.g.ny * a.ncomp * esz * (a.prec == LF2_F32_KAHAN ? 6 : 4);
         const long long tiles = (long long)((a.g.nx + c.tile_x - 1) / c.tile_x) * ((a.g.ny + c.tile_y - 1) / c.tile_y);
         const long long sms = device_sm_count();
-        long long best = -1;
+        double best = -1.0;
         for (int m = 1; m <= 64; ++m) {
             const int zc = (a.g.nz + m - 1) / m;
             if (m > 1 && zc < 2 * c.depth) break;
             const long long blocks = tiles * c.cluster * ((a.g.nz + zc - 1) / zc);
-            const long long cost = ((blocks + sms - 1) / sms) * (zc + 2 * c.depth);
-            if (best < 0 || cost < best) {
+            double cost = (double)((blocks + sms - 1) / sms) * (zc + 2 * c.depth);
+            if (pairs && plane_gb * zc > 32.0) cost *= 1.0 + 0.015 * std::log2(plane_gb * zc / 32.0);
+            if (best < 0.0 || cost < best) {
                 best = cost;
                 c.zchunk = zc;
             }
