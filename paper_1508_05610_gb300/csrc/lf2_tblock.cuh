@@ -575,10 +575,15 @@ __device__ __forceinline__ void pair_iteration(PairState<T, CX * NC / 2> &st, fl
 
 // Whether a configuration runs on pairs: 16 or 24 bytes per thread and plane (8-byte threads share
 // an SM between two blocks of 64 registers a thread, which pairs exceed; 6 components with the plain
-// drift are 2 % slower on pairs, with the compensated one 5 to 8 % faster).
-template <int NC, int MODE, int CX>
+// drift are 2 % slower on pairs, with the compensated one 5 to 8 % faster).  Of two components not at
+// depth 4, with the plain drift not at depth 6 or in clusters either, unless the region is a compile-time
+// constant (FIXED): 256x256x128 FP32+Kahan, depth 4, a step, tb_iteration and pairs: 56x8 tiles 54.9 and
+// 57.5 us; 64^3 plain, 24x8: 3.7 and 4.1; 256x256x128 plain, clusters of two, depth 3: 51.9 and 53.7;
+// with the constant region, 24x24, 40.5 and 34.4.
+template <int NC, int MODE, int T, int CX, int CL, bool FIXED>
 constexpr bool tb_pairs() {
-    return MODE != 3 && CX * NC >= 4 && (NC == 1 ? CX % 2 == 0 : NC % 2 == 0) && !(NC == 6 && MODE == 0);
+    return MODE != 3 && CX * NC >= 4 && (NC == 1 ? CX % 2 == 0 : NC % 2 == 0) && !(NC == 6 && MODE == 0) &&
+           (FIXED || !(NC == 2 && (T == 4 || (MODE == 0 && (T == 6 || CL > 1)))));
 }
 
 // MODE: 0 = FP32 plain drift, 1 = FP32 Kahan drift, 3 = FP64.
@@ -592,7 +597,7 @@ constexpr int tb_min_blocks() {
 constexpr int kFixedThreadsX = 16, kFixedRows = 32;
 template <int NC, int MODE, int T, int CX>
 constexpr bool tb_fixed_built() {
-    return tb_pairs<NC, MODE, CX>() && NC <= 2 && T <= 4;
+    return tb_pairs<NC, MODE, T, CX, 1, true>() && NC <= 2 && T <= 4;
 }
 
 // One tile x z-chunk of a temporal-blocking pass: (bx, by) is the tile, bz the chunk.  With
@@ -650,7 +655,7 @@ __device__ __forceinline__ void tb_block(const R *__restrict__ phi, R *__restric
     // x-neighbours by warp shuffle when every region row is a whole group of lanes within one
     // warp and the block is whole warps
     const bool shfl_x = FIXED || ((32 % RXT == 0) && ((RXT * RY) % 32 == 0));
-    if constexpr (tb_pairs<NC, MODE, CX>()) {
+    if constexpr (tb_pairs<NC, MODE, T, CX, CL, FIXED>()) {
         PairState<T, W / 2> st;
 #pragma unroll
         for (int e = 0; e < W; ++e) st.in_pi[e] = st.in_cm[e] = 0.0f;
