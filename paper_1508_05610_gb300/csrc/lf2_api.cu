@@ -147,12 +147,10 @@ lf2_status ensure_energy_scratch(lf2_field f) {
     if (!f->energy_scratch) {
         void *d = nullptr;
         LF2_CUDA(cudaMalloc(&d, sizeof(double) * kFieldScratchDoubles), "cudaMalloc(energy scratch)");
-        // the finished-block counter (each reduction leaves it at zero) and the row with the multi-step
-        // runs' status must start at zero
-        const double zero[kEnergySlots] = {};
-        cudaError_t e = cudaMemcpy((double *)d + kEnergyCounterOffset, zero, sizeof zero[0], cudaMemcpyHostToDevice);
-        if (e == cudaSuccess)
-            e = cudaMemcpy((double *)d + kStepsWordsOffset, zero, sizeof zero, cudaMemcpyHostToDevice);
+        // the finished-block counter (each reduction leaves it at zero) and the multi-step runs' status,
+        // in the same row, must start at zero
+        const double zero[kStepsRowsOffset - kEnergyCounterOffset] = {};
+        cudaError_t e = cudaMemcpy((double *)d + kEnergyCounterOffset, zero, sizeof zero, cudaMemcpyHostToDevice);
         if (e != cudaSuccess) {
             cudaFree(d);
             return cuda_fail(e, "energy scratch counter");

@@ -419,7 +419,7 @@ __global__ void __launch_bounds__(kEnergyThreads, NC <= 2 ? 4 : 2)
 // trips through L2 and the loads that follow it.
 
 // The row sets (at most kStepsMaxBlocks rows each) start at kStepsRowsOffset of a field's
-// scratch; the barrier and status words (lf2_barrier.cuh) are in the row after them.
+// scratch; the barrier and status words (lf2_barrier.cuh) are in the counter's row before them.
 constexpr int kRowSets = kEnergyStepsRowSets;
 constexpr int kStepsMaxBlocks = kEnergyStepsBlocks;
 
@@ -444,8 +444,7 @@ __global__ void __launch_bounds__(kEnergyThreads, 2)
     const int nsb = ENERGY ? (int)gridDim.x - 1 : (int)gridDim.x;
     const bool reducer = ENERGY && (int)blockIdx.x == nsb;
     // rows [first, first + count) of the set of `step`, inside the row-set region (checked in
-    // the debug build against that region, so neither the reduction layout before it nor the
-    // barrier row after it can be hit)
+    // the debug build against that region, so that nothing before or after it can be hit)
     auto rows_of = [&](int step, long long first, long long count) {
         const long long rel = checked((long long)(step % kRowSets) * nsb * kEnergySlots + first * kEnergySlots,
                                       count * kEnergySlots, (long long)kRowSets * kStepsMaxBlocks * kEnergySlots);

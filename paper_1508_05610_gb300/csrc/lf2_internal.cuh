@@ -52,21 +52,21 @@ constexpr int kEnergyRecordOffset = kEnergyBlocks * kEnergySlots;
 constexpr int kEnergyCounterOffset = kEnergyRecordOffset + kEnergySlots;
 constexpr int kEnergyScratchDoubles = kEnergyCounterOffset + 1;
 static_assert(3 + 2 * kMaxComp <= kEnergySlots, "energy slots");
-// The multi-step step + energy kernel keeps, after that layout, three rotating sets of up to
-// kEnergyStepsBlocks partial rows and one row of barrier words.  A field's scratch
+// The multi-step kernels keep, after that layout, two words in what is left of the counter's row and
+// three rotating sets of up to kEnergyStepsBlocks partial rows.  A field's scratch
 // (kFieldScratchDoubles doubles) holds both parts; lf2_energy_noalloc's fixed array only the
-// first, since it never runs that kernel.
+// first, since it never runs those kernels.
 // At most 303 site blocks (two 256-thread blocks per SM of a 152-SM GB300, less the reducing
 // block): a size bound of the row sets; the launch itself checks co-residency on the device it
 // runs on and falls back to one launch per step where the grid does not fit.
 constexpr int kEnergyStepsBlocks = 303;
 constexpr int kEnergyStepsRowSets = 3;
 constexpr int kStepsRowsOffset = (kEnergyScratchDoubles + kEnergySlots - 1) / kEnergySlots * kEnergySlots;
-constexpr int kStepsWordsOffset = kStepsRowsOffset + kEnergyStepsRowSets * kEnergyStepsBlocks * kEnergySlots;
-constexpr int kFieldScratchDoubles = kStepsWordsOffset + kEnergySlots;
-// In that last row: the barrier's word, zeroed before each launch, and a word that a run whose barrier
-// gave up sets, which keeps that until it has been reported (zero before the first launch).
-constexpr int kStepsBarrierWord = kStepsWordsOffset, kStepsStatusWord = kStepsWordsOffset + 1;
+constexpr int kFieldScratchDoubles = kStepsRowsOffset + kEnergyStepsRowSets * kEnergyStepsBlocks * kEnergySlots;
+// The words: the barrier's, zeroed before each launch, and one that a run whose barrier gave up sets,
+// which keeps that until it has been reported (zero before the first launch, as the counter is).
+constexpr int kStepsBarrierWord = kEnergyCounterOffset + 8, kStepsStatusWord = kStepsBarrierWord + 1;
+static_assert(kEnergyScratchDoubles <= kStepsBarrierWord && kStepsStatusWord < kStepsRowsOffset, "multi-step scratch layout");
 // Energy of (phi, pi) as an lf2_energy_t record: written to scratch + kEnergyRecordOffset and,
 // when `record` is not NULL, also to `record` (device).  One launch.
 cudaError_t launch_energy(const void *phi, const void *pi, const Geom &g, int ncomp, lf2_precision prec,
