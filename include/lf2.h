@@ -92,7 +92,9 @@ typedef struct {
     double sum_sq[LF2_MAX_COMP]; /* sum_x phi_a(x)^2 per component (unused entries 0) */
 } lf2_energy_t;
 
-/* Kernel selection for lf2_leapfrog_ex.  Every variant computes bitwise the same result. */
+/* Kernel selection for lf2_leapfrog_ex.  Every variant computes bitwise the same result, but that an
+ * exact zero may carry the other sign after FP32 temporal blocking (of fields that hold zeros of both
+ * signs); "bitwise" below is meant so wherever the kernel may differ. */
 typedef enum {
     LF2_KERNEL_AUTO = 0,     /* tuned choice (the one lf2_leapfrog uses); in a plan: what runs without one */
     LF2_KERNEL_SITE = 1,     /* one thread per site, any lattice shape */
@@ -198,7 +200,8 @@ lf2_status lf2_field_derivative(lf2_field src, lf2_field dst, int dim, double dx
  * belongs to shell b = floor(sqrt(m_x^2 + m_y^2 + m_z^2)); shells b < nbins (<= 1024) are
  * returned as host arrays of nbins doubles: mean power, mean |k|, mode count.  The transform is
  * cuFFT (single or double precision after the storage type); buffers are allocated per call, plans
- * (without work areas, at most two idle ones) are kept by the lattice until it is destroyed.  LF2_ERR_UNSUPPORTED for non-cubic lattices.  Synchronises `stream`. */
+ * (without work areas, at most two idle ones) are kept by the lattice until it is destroyed.
+ * LF2_ERR_UNSUPPORTED for non-cubic lattices.  Synchronises `stream`. */
 lf2_status lf2_power_spectrum(lf2_field f, int comp, int nbins, double dx, double *power, double *kmean,
                               double *count, void *stream);
 
@@ -275,8 +278,8 @@ lf2_status lf2_energy_device(lf2_field phi, lf2_field pi, const lf2_params *p, d
  * records from the step before that barrier on (a step's record is finished during the next
  * step); lf2_field_check(phi) then returns LF2_ERR_TIMEOUT.  Enqueues on `stream` without waiting;
  * after the first call on phi (which may allocate its back buffer and energy scratch, so make it
- * outside a stream capture) calls allocate nothing and can be captured into a CUDA graph.  Calls on one phi share its energy
- * scratch with lf2_energy and lf2_energy_device: order them on one stream.
+ * outside a stream capture) calls allocate nothing and can be captured into a CUDA graph.  Calls on
+ * one phi share its energy scratch with lf2_energy and lf2_energy_device: order them on one stream.
  * LF2_ERR_INVALID for nsteps < 0 or dev_records NULL with nsteps > 0. */
 lf2_status lf2_leapfrog_energy(lf2_field phi, lf2_field pi, const lf2_params *p, int nsteps, double *dev_records,
                                void *stream);
@@ -342,9 +345,9 @@ lf2_status lf2_ensemble_create(int n, const lf2_field *phis, const lf2_field *pi
 /* Advances every member by nsteps (each member's phi_n / pi_{n-1/2} convention as in
  * lf2_leapfrog) with ONE CUDA-graph launch on `stream`: nsteps/depth temporal-blocking passes,
  * each a persistent kernel over a work list of (member, tile, z-chunk) items ordered longest
- * first, then passes of depth 3 and 2 and single steps for what is left.  The graph is captured on first use for a given
- * nsteps and buffer state (this first call must not itself be inside a stream capture) and
- * relaunched afterwards.  Results are bitwise those of running each member alone. */
+ * first, then passes of depth 3 and 2 (FP32) and single steps for what is left.  The graph is
+ * captured on first use for a given nsteps and buffer state (this first call must not itself be
+ * inside a stream capture) and relaunched afterwards.  Results are bitwise those of running each member alone. */
 lf2_status lf2_ensemble_run(lf2_ensemble e, int nsteps, void *stream);
 
 /* Chooses the ensemble's pass configuration (depth, cx, tile) by timing candidates on a

@@ -36,8 +36,9 @@ constexpr int kNs = 3 + 2 * NC;
 // two for more (128).  The full grid is four blocks per SM, so four or two resident blocks run it in
 // whole waves, where three leave the fourth block alone on its SM (256^3 real FP32 energy with 72
 // registers: 470 us, with 64: 387 us).  5 and 6 components would take up to 185 registers by
-// themselves, one block per SM (96x80x112 6-component FP32 step with energy 1818 us, now 980 us
-// for 8 steps).  The multi-step launch counts on two.
+// themselves, one block per SM.  At 128 FP64 spills (up to 168 bytes) and gains all the same: energy of
+// 160^3, one block and two: 5 components FP64 586 and 431 us, FP32 536 and 386; 6 components 686 and 551,
+// 636 and 457; FP64 step with energy 715 and 537, 849 and 671.  The multi-step launch counts on two.
 template <int NC>
 constexpr int kEnergyResident = NC == 1 ? 4 : 2;
 constexpr int kKin = 0, kGrad = 1, kPot = 2, kSum = 3;
@@ -383,6 +384,9 @@ __global__ void __launch_bounds__(kEnergyThreads, kEnergyResident<NC>)
     finish_energy<NC>(acc, sh, scratch, ke, record);
 }
 
+// Four blocks for two components too, in spite of 84 bytes of spills and more: 160^3 FP32+Kahan 178.4 us with
+// two, 176.9 with four; 96x80x112 51.1 and 50.1.  (In FP64 four are 5 % slower.)  5 and 6 components with one
+// block: 574 and 702 us, with two 408 and 495.
 template <int NC, bool KAHAN>
 __global__ void __launch_bounds__(kEnergyThreads, NC <= 2 ? 4 : 2)
     k_step_energy_f32(const float *__restrict__ phi, float *__restrict__ phi_out, float *__restrict__ pi,
@@ -415,8 +419,10 @@ __global__ void __launch_bounds__(kEnergyThreads, NC <= 2 ? 4 : 2)
 //
 // 32^3 real FP64, a step: 3.8 us with its energy (4.1 with the energy before the arrival and pi in
 // memory, 5.3 with a two-atomic barrier too), 2.2 without (4.3 at best as launches of the streaming
-// kernel); 48x40x36 real FP32+Kahan without energy 6.1 -> 1.8 us.  What is left is the barrier's
-// trips through L2 and the loads that follow it.
+// kernel); 48x40x36 real FP32+Kahan without energy 6.1 -> 1.8 us.  More components, without energy, as
+// four-row streaming or site launches and here: 32^3 FP64, 2 components 8.3 and 3.0 us, 4: 10.4 and 4.6,
+// 6: 14.5 and 6.4; 48^3 10.4 and 5.1, 16.6 and 10.4, 24.7 and 14.5; FP32+Kahan 48^3 6.3 and 2.6, 8.3 and
+// 4.3, 12.4 and 6.3.  What is left is the barrier's trips through L2 and the loads that follow it.
 
 // The row sets (at most kStepsMaxBlocks rows each) start at kStepsRowsOffset of a field's
 // scratch; the barrier and status words (lf2_barrier.cuh) are in the counter's row before them.
@@ -431,8 +437,8 @@ __device__ __forceinline__ void poison_records(double *records, int from, int ns
         for (int i = 0; i < kEnergySlots; ++i) records[(size_t)j * kEnergySlots + i] = __longlong_as_double(0x7ff8000000000000LL);
 }
 
-// MODE: 0 = FP32 plain drift, 1 = FP32 Kahan drift, 3 = FP64.  Launched with energy_grid(sites)
-// site blocks, and with ENERGY one more.
+// MODE: 0 = FP32 plain drift, 1 = FP32 Kahan drift, 3 = FP64.  Launched with a site block for every 256
+// sites, and with ENERGY, where they are energy_grid(sites) blocks, one more.
 template <typename R, int NC, int MODE, bool ENERGY, typename CoefT>
 __global__ void __launch_bounds__(kEnergyThreads, 2)
     k_steps(R *phi_a, R *phi_b, R *__restrict__ pi, float *__restrict__ comp, Geom g, CoefT k, CoefE ke, int nsteps,

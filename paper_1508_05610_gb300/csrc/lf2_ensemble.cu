@@ -6,7 +6,8 @@
 // single persistent kernel launch whose blocks take (member, tile, z-chunk) items, longest
 // chunks first, from a counter zeroed before the pass, followed by shallower passes for what the
 // depth leaves over (two single steps of 64 lattices were 128 launches, 1.33 ms; a depth-2 pass of
-// them takes 0.8) and at most one single step per member.  Members
+// them takes 0.8) and single steps per member for the rest: at most one in FP32, up to depth - 1 in FP64
+// and where a shallower pass does not fit every member or its list found no memory.  Members
 // are independent, so no block ever waits for another; the graph is captured once per
 // (nsteps, buffer parities) and relaunched.
 #include <cuda_runtime.h>

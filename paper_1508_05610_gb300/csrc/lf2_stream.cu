@@ -317,8 +317,10 @@ bool stream_supported(const StepArgs &a, int tile_y, int zchunk) {
 }
 
 cudaError_t launch_default_step(const StepArgs &a, cudaStream_t s) {
-    // Of the lattices whose rows come in twos but not in fours, 3-component ones take the site kernel:
-    // 40x98x200 FP32 10.5 us a step, streaming 14.7 (100x102x104: 12.6 and 14.6)
+    // Of the lattices whose rows come in twos but not in fours, 3-component ones take the site kernel.  A
+    // step, site and streaming: 40x98x200 FP64 26.9 and 41.2 us, FP32+Kahan 10.9 and 16.7, FP32 10.5 and
+    // 14.6; 100x102x104 34.9 and 44.2, 12.7 and 18.7, 12.5 and 14.6; 512x130x256 FP64 467 and 496.  (In
+    // FP32 it is the other way round from some million sites on: 512x130x256 282 and 195, 204 and 139.)
     const bool fours = a.g.ny % kStreamRows == 0;
     int rows = 0;
     if (a.ncomp != 3 || fours)

@@ -373,8 +373,10 @@ __device__ __forceinline__ void tb_iteration(TbState<R, T, CX * NC> &st, R *__re
 //   - differences are shared: phi(z+1) - phi(z) of one plane is, negated, the phi(z-1) - phi(z) of
 //     the next, so each level keeps its centre plane and that difference in registers instead of
 //     three planes; and in x, phi(x+1) - phi(x) serves both its columns.  Rounding is symmetric,
-//     RN(a - b) = -RN(b - a), so every sum keeps its bits (a zero may keep another sign).  77 instead of 84 FMA cycles and 43
-//     instead of 54 instructions for the arithmetic of a stage of 4 real sites;
+//     RN(a - b) = -RN(b - a), so every sum keeps its bits, but for one sign: a difference of equal
+//     values is +0 taken either way, so a sum of differences that are all zero may be -0 where the
+//     site's own six give +0 (fields of zeros of both signs).  Values never differ.  77 instead of 84
+//     FMA cycles and 43 instead of 54 instructions for the arithmetic of a stage of 4 real sites;
 //   - with the region's size fixed at compile time (16 threads x 32 rows, the best of the tuner's
 //     regions for one and two components) the shared addresses are immediates, which leaves
 //     registers to issue ahead;

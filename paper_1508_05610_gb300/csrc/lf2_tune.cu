@@ -1,6 +1,6 @@
 // lf2_tune.cu -- autotuner for the leapfrog kernel configuration.
 //
-// Every kernel variant computes bitwise the same result, so the tuner only has to find the
+// Every kernel variant computes the same result, so the tuner only has to find the
 // fastest one.  It times candidate configurations (one-step streaming tiles and temporal
 // blocking of several depths, column widths and tiles; on a small lattice also all steps in one
 // launch, which is what runs there without a plan) on a proxy lattice with the same x-y

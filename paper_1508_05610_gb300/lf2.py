@@ -240,7 +240,8 @@ def lf2_energy_device(phi, pi, p: lf2_params, dev_out_ptr, stream=None):
 
 def lf2_leapfrog_energy(phi, pi, p: lf2_params, nsteps, dev_records_ptr, stream=None):
     """nsteps leapfrog steps that also write the energy record of the state at the start of every
-    step, in one launch for a small lattice and one launch per step otherwise (nsteps x 16 doubles of device memory at dev_records_ptr)."""
+    step, in one launch for a small lattice and one launch per step otherwise (nsteps x 16 doubles of
+    device memory at dev_records_ptr)."""
     _call("lf2_leapfrog_energy", phi, pi, ctypes.byref(p), int(nsteps), dev_records_ptr, _stream_ptr(stream))
 
 
