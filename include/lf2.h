@@ -374,7 +374,8 @@ lf2_status lf2_ensemble_destroy(lf2_ensemble e);
  * 256 z-planes (fewer for very large planes, to stay within about 8 GB), filled with a copy
  * of the fields' first planes -- phi and pi are not modified.  On a lattice small enough for it, all
  * steps in one launch (see lf2_leapfrog) are timed as well, on a copy of the whole lattice; where
- * that is the fastest, the plan is LF2_KERNEL_AUTO, and phi's scratch is allocated if missing.
+ * that is the fastest, the plan is LF2_KERNEL_AUTO.  phi's scratch, which such runs need, is allocated
+ * there if missing.
  * The plan is cached per process (and appended to the file named by the environment variable
  * LF2_TUNE_CACHE, which is read on first use) and used by every later lf2_leapfrog on a lattice
  * of that shape.  Results do not depend on the plan: all variants are bitwise identical.

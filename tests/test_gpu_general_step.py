@@ -140,3 +140,29 @@ def test_column_walk_over_chunks_of_several_planes(lf2, monkeypatch, shape, prec
         lf2.lf2_leapfrog_ex(b.phi, b.pi, p, 3, kernel=lf2.LF2_KERNEL_SITE)
         got, ref = a.download(), b.download()
     assert np.array_equal(got[0], ref[0]) and np.array_equal(got[1], ref[1])
+
+
+@pytest.mark.parametrize("shape,ncomp,prec", [((16, 16, 16), 1, "f64"), ((20, 18, 14), 2, "f32k")])
+def test_small_lattice_run_captured_into_a_graph(lf2, monkeypatch, shape, ncomp, prec):
+    """A run of several steps in one launch, captured (an even number of steps, so that the buffers are
+    where they were) and replayed three times, bitwise as many steps of the site kernel."""
+    import torch
+    monkeypatch.setenv("LF2_TUNE", "off")
+    phi0 = inputs.gaussian_field(*shape, ncomp, sigma=0.4, seed=941)
+    pi0 = inputs.gaussian_field(*shape, ncomp, sigma=0.2, seed=942)
+    p = lf2.params(**KW)
+    with lf2.System(shape, ncomp, prec) as a, lf2.System(shape, ncomp, prec) as b:
+        for s in (a, b):
+            s.upload(phi0, pi0)
+            lf2.lf2_leapfrog_init(s.phi, s.pi, p)
+        torch.cuda.synchronize()
+        g = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(g):
+            lf2.lf2_leapfrog(a.phi, a.pi, p, 6, torch.cuda.current_stream())
+        for _ in range(3):
+            g.replay()
+        torch.cuda.synchronize()
+        lf2.lf2_leapfrog_ex(b.phi, b.pi, p, 18, kernel=lf2.LF2_KERNEL_SITE)
+        got, ref = a.download(), b.download()
+        lf2.lf2_field_check(a.phi)
+    assert np.array_equal(got[0], ref[0]) and np.array_equal(got[1], ref[1])
