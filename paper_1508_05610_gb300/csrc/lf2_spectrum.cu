@@ -65,6 +65,7 @@ __global__ void __launch_bounds__(kBinThreads) k_bin(const C *__restrict__ spec,
     __syncthreads();
     const int hx = n / 2 + 1, half = n / 2, lane = threadIdx.x & 31;
     const bool even = n % 2 == 0;
+    const double both = 2.0 * inv_volume;
     auto self = [&](int k) { return k == 0 || (even && k == half); };  // its own mirror image
     const long long pairs = (long long)hx * (hx + 1) / 2;  // 0 <= ky <= kz <= half
     const int segs = (hx + 31) / 32;
@@ -101,7 +102,7 @@ __global__ void __launch_bounds__(kBinThreads) k_bin(const C *__restrict__ spec,
         unsigned count = 0u;
         if (in) {
             const int w = self(x) ? 1 : 2;  // kx and -kx
-            power *= (double)w * inv_volume;  // before the shell's sum, which could overflow where its mean does not
+            power *= w == 1 ? inv_volume : both;  // before the shell's sum, which could overflow where its mean does not
             count = (unsigned)(w * images);
             if (!add_power) ksum = (double)count * sqrt((double)s2);
         }
