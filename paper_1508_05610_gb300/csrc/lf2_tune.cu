@@ -73,13 +73,14 @@ void append_file(const Key &k, const lf2_step_config &c) {
     fclose(f);
 }
 
-std::vector<lf2_step_config> candidates(int ny, lf2_precision prec, int flags) {
+std::vector<lf2_step_config> candidates(const int n[3], lf2_precision prec, int flags) {
     std::vector<lf2_step_config> out;
-    for (int ty : {2, 4})
-        for (int zc : {2, 4, 8}) out.push_back(lf2_step_config{LF2_KERNEL_STREAM, 0, ty, zc, 0, 0});
-    // four rows to a tile are more than 65535 tiles
-    if (ny > 4 * 65535)
-        for (int zc : {4, 8}) out.push_back(lf2_step_config{LF2_KERNEL_STREAM, 0, 8, zc, 0, 0});
+    // taller tiles and longer chunks where these would be more than 65535
+    std::vector<int> rows{2, 4}, planes{2, 4, 8};
+    if (n[1] > 4 * 65535) rows.push_back(8);
+    if (n[2] > 8 * 65535) planes.push_back(16);
+    for (int ty : rows)
+        for (int zc : planes) out.push_back(lf2_step_config{LF2_KERNEL_STREAM, 0, ty, zc, 0, 0});
     if (flags & LF2_TUNE_ONE_STEP) return out;
     const int depths64[] = {2, 4};
     const int depths32[] = {2, 3, 4, 6, 8};
@@ -199,7 +200,10 @@ extern "C" lf2_status lf2_tune(lf2_field phi, lf2_field pi, const lf2_params *p,
             best = c;
         }
     };
-    for (const lf2_step_config &c : candidates(n[1], phi->prec, flags)) time_config(c);
+    const StepArgs whole = step_args(phi, pi, p, p->dt, true);
+    for (const lf2_step_config &c : candidates(n, phi->prec, flags))
+        // a chunk of z-planes that fits the proxy may be too short for all of the lattice's
+        if (c.kernel != LF2_KERNEL_STREAM || stream_supported(whole, c.tile_y, c.zchunk)) time_config(c);
     // Without this a plan would shut out the one-launch run that a small lattice takes when it has none
     // (32^3 real FP64 2.2 us a step, 4.3 in the best streaming tile).  Two steps show whether it fits.
     if (best_ms > 0.0f && small && ensure_energy_scratch(pphi) == LF2_OK && ensure_energy_scratch(phi) == LF2_OK &&

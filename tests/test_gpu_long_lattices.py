@@ -67,3 +67,14 @@ def test_one_step_plan_of_a_lattice_that_only_tall_tiles_fit(lf2):
         plan = lf2.lf2_tune(s.phi, s.pi, lf2.params(**KW), flags=lf2.LF2_TUNE_FORCE | lf2.LF2_TUNE_ONE_STEP)
     assert plan["kernel"] == lf2.LF2_KERNEL_STREAM and plan["tile_y"] == 8
     same_as_site(lf2, shape, 1, "f32", lambda s, p: lf2.lf2_leapfrog(s.phi, s.pi, p, 2))
+
+
+@pytest.mark.parametrize("nz", [131080, 262144, 524288])
+def test_one_step_plan_launches_on_more_planes_than_the_tuner_times(lf2, nz):
+    """The tuner times 256 planes; chunks of two or four planes that win there are more than 65535 chunks
+    here."""
+    shape = (16, 4, nz)
+    with lf2.System(shape, 1, "f32k") as s:
+        plan = lf2.lf2_tune(s.phi, s.pi, lf2.params(**KW), flags=lf2.LF2_TUNE_FORCE | lf2.LF2_TUNE_ONE_STEP)
+    assert plan["kernel"] == lf2.LF2_KERNEL_STREAM and plan["zchunk"] * 65535 >= nz
+    same_as_site(lf2, shape, 1, "f32k", lambda s, p: lf2.lf2_leapfrog(s.phi, s.pi, p, 2))
