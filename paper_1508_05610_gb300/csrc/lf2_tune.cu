@@ -206,9 +206,12 @@ extern "C" lf2_status lf2_tune(lf2_field phi, lf2_field pi, const lf2_params *p,
         if (c.kernel != LF2_KERNEL_STREAM || stream_supported(whole, c.tile_y, c.zchunk)) time_config(c);
     // Without this a plan would shut out the one-launch run that a small lattice takes when it has none
     // (32^3 real FP64 2.2 us a step, 4.3 in the best streaming tile).  Two steps show whether it fits.
-    if (best_ms > 0.0f && small && ensure_energy_scratch(pphi) == LF2_OK && ensure_energy_scratch(phi) == LF2_OK &&
-        launch_steps_plain(step_args(pphi, ppi, p, p->dt, true), 2, pphi->energy_scratch, false, s) == cudaSuccess)
-        time_config(lf2_step_config{LF2_KERNEL_AUTO, 0, 0, 0, 0, 0});
+    if (best_ms > 0.0f && small) {
+        if (ensure_energy_scratch(pphi) != LF2_OK || ensure_energy_scratch(phi) != LF2_OK)
+            (void)cudaGetLastError();  // no memory for it: the plans above remain
+        else if (launch_steps_plain(step_args(pphi, ppi, p, p->dt, true), 2, pphi->energy_scratch, false, s) == cudaSuccess)
+            time_config(lf2_step_config{LF2_KERNEL_AUTO, 0, 0, 0, 0, 0});
+    }
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
     cleanup();
